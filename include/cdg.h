@@ -197,7 +197,8 @@ int cdg_query(const cdg_handle* h, cdg_info* info);
  * the paper; an execution detail of this library).  out[13]: [0] FP64 level-0
  * apply and [1] FP64 level-0 residual (level 0 only), [2] V-cycle residual and
  * [3] V-cycle smoother sweep (V-cycle precision): blocks in flight per step of
- * the vector-load kernel; multi-right-hand-side kernels as (threads across
+ * the vector-load kernel (FP64 operators in integer-digit form, the default,
+ * have one variant and report 2); multi-right-hand-side kernels as (threads across
  * the right-hand sides, block rows per CTA): [4,5] smoother sweep, [6,7]
  * residual, [8,9] FP64 level-0 apply (level 0 only), and their right-hand
  * sides per thread: [10] smoother sweep, [11] residual, [12] FP64 level-0

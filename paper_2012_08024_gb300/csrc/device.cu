@@ -4,7 +4,8 @@
 // (R15).  All device memory is carved from one caller-provided buffer.
 //
 // Layout in HBM (tree order: children of every agglomerate contiguous):
-//   A_l      BSR, int32 rowptr/col, n_p x n_p row-major blocks, FP64 (+FP32 copy)
+//   A_l      BSR, int32 rowptr/col, n_p x n_p row-major blocks, FP64 (+FP32 copy); the FP64
+//            blocks of the operators and transfers in digit form (device_fixed.cu)
 //   Dinv_l   [n_l][n_p][n_p] inverses of the diagonal blocks of A_l
 //   L_l      [n_l][n_p][n_p] prolongation blocks to level l from its parent
 //   vectors  [n_l][n_p] element-major
@@ -16,6 +17,7 @@
 #include <string>
 #include <vector>
 
+#include "device_fixed.h"
 #include "device_kernels.cuh"
 #include "device_state.h"
 
@@ -74,8 +76,26 @@ std::vector<int> agglomerate_chunks(const std::vector<cdg::i32>& cp, int target,
 // fine rows per chunk of the fused restriction: four passes of a 256-thread CTA
 inline int chunk_target(int np) { return 4 * (kThreads / 32) * (32 / np); }
 
+int widest_row(const cdg::BSR& A) {
+  int64_t w = 0;
+  for (int64_t K = 0; K < A.nrows; ++K) w = std::max<int64_t>(w, A.rowptr[K + 1] - A.rowptr[K]);
+  return (int)w;
+}
+
+// columns as [nrows][width], -1 behind a row's last block
+std::vector<int> padded_columns(const cdg::BSR& A, int width) {
+  std::vector<int> o((size_t)A.nrows * width, -1);
+  for (int64_t K = 0; K < A.nrows; ++K)
+    for (int64_t b = A.rowptr[K]; b < A.rowptr[K + 1]; ++b) o[(size_t)K * width + (b - A.rowptr[K])] = A.col[b];
+  return o;
+}
+
+// The FP64 operators are kept in digit form (device_fixed.cu) unless an option asks for
+// kernels that read them as FP64 numbers.
+inline bool digit_form(const cdg_options& o) { return o.fuse_transfers == 0; }
+
 size_t layout(const cdg::Hierarchy& H, int precision, int nrhs, DeviceState* S, char* base, int mr_precision,
-              int gmres_m, int maxit, int tc_fp64) {
+              int gmres_m, int maxit, int tc_fp64, bool fixed) {
   Carver c{base};
   const int np = H.np;
   const int nlev = (int)H.lev.size();
@@ -92,6 +112,7 @@ size_t layout(const cdg::Hierarchy& H, int precision, int nrhs, DeviceState* S, 
   D.ndofs = ne * np;
   D.nbf = (int64_t)H.mesh.bf_K.size();
   D.precision = precision;
+  D.fixed = fixed;
   const size_t vsz = precision ? sizeof(float) : sizeof(double);
   D.nrhs = nrhs;
   for (int l = 0; l < nlev; ++l) {
@@ -107,7 +128,15 @@ size_t layout(const cdg::Hierarchy& H, int precision, int nrhs, DeviceState* S, 
     L.col = c.take<int>(A.nnzb());
     const bool last = l + 1 == nlev;
     // FP64 operator: level 0 always (outer CG); all levels in FP64 mode
-    if (l == 0 || precision == 0) L.A = c.take<double>(A.val.size());
+    if (l == 0 || precision == 0) {
+      L.A = c.take<double>(A.val.size());
+      if (fixed) {
+        L.eA = c.take<int>((size_t)L.n * npl);
+        L.well = widest_row(A);
+        L.ell = c.take<int>((size_t)L.n * L.well + 1);
+      }
+      if (fixed && l == 0 && nrhs > 0) L.Aplain = c.take<double>(A.val.size());
+    }
     if (!last) {
       const cdg::BSR& Sh = H.Ahat_t[l];
       L.hnnzb = Sh.nnzb();
@@ -119,6 +148,18 @@ size_t layout(const cdg::Hierarchy& H, int precision, int nrhs, DeviceState* S, 
         L.Dinv = c.take<double>((size_t)L.n * nb2l);
         if (nL) L.L = c.take<double>(nL);
         L.Ahat = c.take<double>(Sh.val.size() + 1);
+        if (fixed) {
+          L.eD = c.take<int>((size_t)L.n * npl);
+          L.eH = c.take<int>((size_t)L.n * npl);
+          L.whell = widest_row(Sh);
+          L.hell = c.take<int>((size_t)L.n * L.whell + 1);
+          if (nL) {
+            L.Lx = c.take<double>(nL);
+            L.eL = c.take<int>((size_t)L.n * npl);
+            L.Rx = c.take<double>(nL);
+            L.eR = c.take<int>((size_t)H.A_t[l + 1].nrows * npl);
+          }
+        }
       } else {
         L.A32 = c.take<float>(A.val.size());
         L.Dinv32 = c.take<float>((size_t)L.n * nb2l);
@@ -1009,6 +1050,84 @@ const float* opL<float>(const DevLevel& L) { return L.L32; }
 template <typename T>
 int unr_of(const DevLevel& L, int mode) { return L.unr[sizeof(T) == 8 ? 0 : 1][mode]; }
 
+// Block kernels of one level on its operators in their stored form: A (modes 0 and 1) or
+// Ahat (mode 3).  aligned: the vectors start on 16-byte boundaries (the kernels on FP64 and
+// FP32 blocks then take vector loads; the digit form needs no alignment).
+template <typename T>
+bool level_bsr(const DeviceState& D, const DevLevel& L, int mode, const T* x, const T* b, T* y, double omega,
+               double* dot, cudaStream_t s, bool aligned = true, int unr = 0) {
+  const bool hat = mode == 3;
+  const int* rp = hat ? L.hrowptr : L.rowptr;
+  const int* cl = hat ? L.hcol : L.col;
+  if (unr == 0) unr = unr_of<T>(L, mode);
+  if constexpr (sizeof(T) == 8) {
+    if (D.fixed) {
+      FxOp o = operator_op(L, mode);
+      o.x = x;
+      o.b = b;
+      o.y = y;
+      o.omega = omega;
+      o.dot = dot;
+      return fx_run(o, s);
+    }
+  }
+  return launch_bsr<T>(mode, L.np, L.n, rp, cl, hat ? opH<T>(L) : opA<T>(L), x, b, y, omega, dot, s,
+                       aligned ? D.scal + S_FLAG : nullptr, unr);
+}
+
+// bh = D^{-1} b and, with x, x = omega bh (the first smoothing step from a zero guess)
+template <typename T>
+bool level_smooth_first(const DeviceState& D, const DevLevel& L, const T* b, T* bh, T* x, double omega,
+                        cudaStream_t s) {
+  if constexpr (sizeof(T) == 8) {
+    if (D.fixed) {
+      FxOp o = diagonal_op(L, x ? 6 : 7, L.Dinv, L.eD);
+      o.x = b;
+      o.y = bh;
+      o.y2 = x;
+      o.omega = omega;
+      return fx_run(o, s);
+    }
+  }
+  return launch_smooth_first<T>(L.np, L.n, opD<T>(L), b, bh, x, omega, s);
+}
+
+// b_{l+1} = R r_l and x_l (+)= L x_{l+1} inside the V-cycle
+template <typename T>
+bool level_restrict(const DeviceState& D, int l, const T* r, T* bc, cudaStream_t s) {
+  const DevLevel& F = D.lev[l];
+  if constexpr (sizeof(T) == 8) {
+    if (D.fixed && !F.ptrans) {
+      FxOp o;
+      o.mode = 8;
+      o.np = F.np;
+      o.n = D.lev[l + 1].n;
+      o.blocks = F.n;
+          o.rowptr = D.lev[l + 1].childptr;
+      o.A = F.Rx;
+      o.EA = F.eR;
+      o.x = r;
+      o.y = bc;
+      return fx_run(o, s);
+    }
+  }
+  return transfer_restrict<T>(D, l, opL<T>(F), r, bc, s);
+}
+
+template <typename T>
+bool level_prolong(const DeviceState& D, int l, const T* xc, T* x, bool add, cudaStream_t s) {
+  const DevLevel& F = D.lev[l];
+  if constexpr (sizeof(T) == 8) {
+    if (D.fixed && !F.ptrans) {
+      FxOp o = prolong_op(F, add ? 4 : 7);
+      o.x = xc;
+      o.y = x;
+      return fx_run(o, s);
+    }
+  }
+  return transfer_prolong<T>(D, l, opL<T>(F), xc, x, add, s);
+}
+
 // Fused residual + restriction from level l to l+1 (+ the coarse level's first
 // smoothing step, smooth: 0 none, 1 bh only, 2 bh and x = omega bh); false when
 // the level has no chunk table or needs more shared memory than a CTA has by
@@ -1109,8 +1228,7 @@ void coarse_solve(DeviceState& D, const T* b, T* x, cudaStream_t s) {
     if (!C.A || D.precision != 0) return;   // the work vectors of an FP32 V-cycle hold floats
     double* r = (double*)C.r;
     const bool aligned = (((uintptr_t)b | (uintptr_t)x) & 15) == 0;
-    launch_bsr<double>(1, C.np, C.n, C.rowptr, C.col, C.A, x, b, r, 0.0, nullptr, s,
-                       aligned ? D.scal + S_FLAG : nullptr, unr_of<double>(C, 1));
+    level_bsr<double>(D, C, 1, x, b, r, 0.0, nullptr, s, aligned);
     launch(coarse_kernel<double, double, true>, g, 256, s, D.nc, D.crow_seg, D.crow_off, D.cinv_off, D.coarse_inv,
            (const double*)r, x);
   }
@@ -1141,18 +1259,15 @@ bool vcycle(DeviceState& D, const cdg_options& o, const T* b0, T* z0, cudaStream
   // downward sweep
   for (int l = 0; l + 1 < nlev; ++l) {
     DevLevel& L = D.lev[l];
-    const int np = L.np;
     T* x = (T*)L.x;
     T* t = (T*)L.t;
     const T* b = bl[l];
     T* bh = (T*)L.bh;
     const bool coarse_is_last = l + 2 == nlev;
     if (o.nu_pre >= 1) {
-      if (!first_done[l] && !launch_smooth_first<T>(np, L.n, opD<T>(L), b, bh, x, w, s)) return false;
+      if (!first_done[l] && !level_smooth_first<T>(D, L, b, bh, x, w, s)) return false;
       for (int k = 1; k < o.nu_pre; ++k) {
-        if (!launch_bsr<T>(3, np, L.n, L.hrowptr, L.hcol, opH<T>(L), x, bh, t, w, nullptr, s, flag,
-                           unr_of<T>(L, 3)))
-          return false;
+        if (!level_bsr<T>(D, L, 3, x, bh, t, w, nullptr, s)) return false;
         std::swap(x, t);
       }
       const int smooth = coarse_is_last ? 0 : 2;
@@ -1160,21 +1275,19 @@ bool vcycle(DeviceState& D, const cdg_options& o, const T* b0, T* z0, cudaStream
           launch_restrict_fused<T>(D, l, true, smooth, x, b, (T*)D.lev[l + 1].b, w, s, flag)) {
         first_done[l + 1] = smooth != 0;
       } else {
-        if (!launch_bsr<T>(1, np, L.n, L.rowptr, L.col, opA<T>(L), x, b, (T*)L.r, w, nullptr, s, flag,
-                           unr_of<T>(L, 1)))
-          return false;
-        if (!transfer_restrict<T>(D, l, opL<T>(L), (const T*)L.r, (T*)D.lev[l + 1].b, s)) return false;
+        if (!level_bsr<T>(D, L, 1, x, b, (T*)L.r, w, nullptr, s)) return false;
+        if (!level_restrict<T>(D, l, (const T*)L.r, (T*)D.lev[l + 1].b, s)) return false;
       }
       // remember which buffer holds x
       L.x = x;
       L.t = t;
     } else {
-      if (!first_done[l] && !launch_smooth_first<T>(np, L.n, opD<T>(L), b, bh, (T*)nullptr, w, s)) return false;
+      if (!first_done[l] && !level_smooth_first<T>(D, L, b, bh, (T*)nullptr, w, s)) return false;
       const int smooth = coarse_is_last ? 0 : 1;
       if (fuse && !L.ptrans &&
           launch_restrict_fused<T>(D, l, false, smooth, (const T*)nullptr, b, (T*)D.lev[l + 1].b, w, s, flag)) {
         first_done[l + 1] = smooth != 0;
-      } else if (!transfer_restrict<T>(D, l, opL<T>(L), b, (T*)D.lev[l + 1].b, s)) {
+      } else if (!level_restrict<T>(D, l, b, (T*)D.lev[l + 1].b, s)) {
         return false;
       }
     }
@@ -1188,11 +1301,10 @@ bool vcycle(DeviceState& D, const cdg_options& o, const T* b0, T* z0, cudaStream
   std::vector<char> prolonged(nlev, 0);   // the level's correction came with the coarser level's last sweep
   for (int l = nlev - 2; l >= 0; --l) {
     DevLevel& L = D.lev[l];
-    const int np = L.np;
     T* x = (T*)L.x;
     T* t = (T*)L.t;
     if (!prolonged[l] &&
-        !transfer_prolong<T>(D, l, opL<T>(L), (const T*)D.lev[l + 1].x, x, o.nu_pre >= 1, s))
+        !level_prolong<T>(D, l, (const T*)D.lev[l + 1].x, x, o.nu_pre >= 1, s))
       return false;
     // the last sweep of this level also prolongs into level l-1 (agglomeration step)
     const bool carry = fuse_up && l >= 1 && !D.lev[l - 1].ptrans && opL<T>(D.lev[l - 1]) != nullptr;
@@ -1201,15 +1313,14 @@ bool vcycle(DeviceState& D, const cdg_options& o, const T* b0, T* z0, cudaStream
       if (carry && k + 1 == o.nu_post) {
         if (!launch_smooth_prolong<T>(D, l - 1, x, (const T*)L.bh, out, w, o.nu_pre >= 1, s, flag)) return false;
         prolonged[l - 1] = 1;
-      } else if (!launch_bsr<T>(3, np, L.n, L.hrowptr, L.hcol, opH<T>(L), x, (const T*)L.bh, out, w, nullptr, s,
-                                flag, unr_of<T>(L, 3))) {
+      } else if (!level_bsr<T>(D, L, 3, x, (const T*)L.bh, out, w, nullptr, s)) {
         return false;
       }
       if (out == t) std::swap(x, t);
       else x = out;
     }
     if (l == 0 && o.nu_post == 0)
-      cudaMemcpyAsync(z0, x, sizeof(T) * (size_t)L.n * np, cudaMemcpyDeviceToDevice, s);
+      cudaMemcpyAsync(z0, x, sizeof(T) * (size_t)L.n * L.np, cudaMemcpyDeviceToDevice, s);
     if (l > 0) {
       // the coarse solution of this level must sit in L.x for the next prolongation
       if (x != (T*)L.x) {
@@ -1272,6 +1383,16 @@ std::vector<float> to_f32(const std::vector<double>& v) {
   return o;
 }
 
+// every n_p x n_p block transposed
+std::vector<double> transposed_blocks(const std::vector<double>& v, int np) {
+  std::vector<double> o(v.size());
+  const size_t nb2 = (size_t)np * np;
+  for (size_t k = 0; k < v.size() / nb2; ++k)
+    for (int i = 0; i < np; ++i)
+      for (int j = 0; j < np; ++j) o[k * nb2 + (size_t)j * np + i] = v[k * nb2 + (size_t)i * np + j];
+  return o;
+}
+
 std::vector<int> to_i32(const std::vector<int64_t>& v) {
   std::vector<int> o(v.size());
   for (size_t i = 0; i < v.size(); ++i) o[i] = (int)v[i];
@@ -1288,8 +1409,7 @@ int dev_precond(cdg_handle* h, const double* r, double* z, cudaStream_t s) { ret
 int dev_apply0(cdg_handle* h, int mode, const double* x, const double* b, double* y, cudaStream_t s) {
   DeviceState& D = *h->dev;
   const DevLevel& L0 = D.lev[0];
-  if (!launch_bsr<double>(mode, D.np, L0.n, L0.rowptr, L0.col, L0.A, x, b, y, h->opt.omega, nullptr, s,
-                          D.scal + S_FLAG, unr_of<double>(L0, mode))) {
+  if (!level_bsr<double>(D, L0, mode, x, b, y, h->opt.omega, nullptr, s)) {
     h->err = "unsupported number of basis functions per element";
     return CDG_EINVAL;
   }
@@ -1374,11 +1494,9 @@ int dev_smooth_static(cdg_handle* h, int level, const double* x, const double* b
     scratch = g_static_ptr[dev];
   }
   cudaStream_t s = (cudaStream_t)stream;
-  const bool ok = launch_smooth_first<double>(L.np, L.n, L.Dinv, b, scratch, (double*)nullptr, h->opt.omega, s) &&
-                  launch_bsr<double>(3, L.np, L.n, L.hrowptr, L.hcol, L.Ahat, x, (const double*)scratch, y,
-                                     h->opt.omega, nullptr, s,
-                                     (((uintptr_t)x | (uintptr_t)y) & 15) == 0 ? D.scal + S_FLAG : nullptr,
-                                     unr_of<double>(L, 3));
+  const bool ok = level_smooth_first<double>(D, L, b, scratch, (double*)nullptr, h->opt.omega, s) &&
+                  level_bsr<double>(D, L, 3, x, (const double*)scratch, y, h->opt.omega, nullptr, s,
+                                    (((uintptr_t)x | (uintptr_t)y) & 15) == 0);
   if (!ok) {
     h->err = "unsupported n_p";
     return CDG_EINVAL;
@@ -1391,7 +1509,7 @@ static int gmres_len(const cdg_options& o) { return o.krylov == 1 ? o.restart : 
 
 int dev_bytes(const cdg_handle* h, int64_t* bytes) {
   *bytes = (int64_t)layout(h->H, h->opt.precision == 2 ? 1 : h->opt.precision, h->opt.nrhs, nullptr, nullptr,
-                          h->opt.precision, gmres_len(h->opt), h->opt.maxit, h->opt.tc_fp64_apply);
+                          h->opt.precision, gmres_len(h->opt), h->opt.maxit, h->opt.tc_fp64_apply, digit_form(h->opt));
   return CDG_OK;
 }
 
@@ -1415,8 +1533,8 @@ void dev_release(cdg_handle* h) {
 
 // Autotuner of the block-row tiling: times the vector-load block-sparse kernel
 // with 1, 2 and 4 blocks in flight per step for every (level, operator
-// precision, mode) that a solve launches, on the handle's own operators and
-// zero-filled work vectors, and keeps the fastest.  Every variant sums in the
+// precision, mode) that a solve launches (operators in digit form have no
+// variants), on the handle's own operators and zero-filled work vectors, and keeps the fastest.  Every variant sums in the
 // same order, so the choice changes the timing only, never a result.
 static int autotune_bsr(cdg_handle* h, cudaStream_t s) {
   DeviceState& D = *h->dev;
@@ -1425,7 +1543,6 @@ static int autotune_bsr(cdg_handle* h, cudaStream_t s) {
   if (e == cudaSuccess) e = cudaEventCreate(&e1);
   if (e != cudaSuccess) return cuda_fail(h, e, "autotune");
   const double w = h->opt.omega;
-  double* flag = D.scal + S_FLAG;
   auto pick = [&](auto&& launch_one) -> int {
     int best = 2;
     float tbest = 3.0e38f;
@@ -1438,27 +1555,24 @@ static int autotune_bsr(cdg_handle* h, cudaStream_t s) {
     }
     return best;
   };
-  // odd n_p: the scalar-load kernel has no variants (levels keep the default)
+  // odd n_p and operators in digit form: those kernels have no variants (levels keep the default)
   // level 0, FP64: the outer apply and residual
-  if (D.lev[0].np % 2 == 0) {
+  if (D.lev[0].np % 2 == 0 && !D.fixed) {
     DevLevel& L = D.lev[0];
-    const int np = L.np;
     const size_t nb = sizeof(double) * (size_t)D.ndofs;
     cudaMemsetAsync(D.p, 0, nb, s);
     cudaMemsetAsync(D.q, 0, nb, s);
     cudaMemsetAsync(D.r, 0, nb, s);
     L.unr[0][0] = pick([&](int u) {
-      launch_bsr<double>(0, np, L.n, L.rowptr, L.col, L.A, D.p, (const double*)nullptr, D.q, w, nullptr, s, flag, u);
+      level_bsr<double>(D, L, 0, D.p, (const double*)nullptr, D.q, w, nullptr, s, true, u);
     });
-    L.unr[0][1] = pick([&](int u) {
-      launch_bsr<double>(1, np, L.n, L.rowptr, L.col, L.A, D.p, D.r, D.q, w, nullptr, s, flag, u);
-    });
+    L.unr[0][1] = pick([&](int u) { level_bsr<double>(D, L, 1, D.p, D.r, D.q, w, nullptr, s, true, u); });
   }
   // V-cycle levels in the V-cycle precision: residual and smoother sweep
   auto tune_level = [&](auto zero, DevLevel& L, int l) {
     using T = decltype(zero);
     const int np = L.np;
-    if (np % 2 != 0) return;
+    if (np % 2 != 0 || (sizeof(T) == 8 && D.fixed)) return;
     const int ti = sizeof(T) == 8 ? 0 : 1;
     const size_t nb = sizeof(T) * (size_t)L.n * np;
     T *x = (T*)L.x, *b = (T*)L.b, *bh = (T*)L.bh, *y = (T*)L.t;
@@ -1467,16 +1581,10 @@ static int autotune_bsr(cdg_handle* h, cudaStream_t s) {
     cudaMemsetAsync(bh, 0, nb, s);
     cudaMemsetAsync(y, 0, nb, s);
     if (l > 0 || ti == 1)
-      L.unr[ti][1] = pick([&](int u) {
-        launch_bsr<T>(1, np, L.n, L.rowptr, L.col, opA<T>(L), x, b, y, w, nullptr, s, flag, u);
-      });
-    L.unr[ti][3] = pick([&](int u) {
-      launch_bsr<T>(3, np, L.n, L.hrowptr, L.hcol, opH<T>(L), x, bh, y, w, nullptr, s, flag, u);
-    });
+      L.unr[ti][1] = pick([&](int u) { level_bsr<T>(D, L, 1, x, b, y, w, nullptr, s, true, u); });
+    L.unr[ti][3] = pick([&](int u) { level_bsr<T>(D, L, 3, x, bh, y, w, nullptr, s, true, u); });
     if (ti == 1)   // the FP32 apply (cdg_apply_f32)
-      L.unr[1][0] = pick([&](int u) {
-        launch_bsr<T>(0, np, L.n, L.rowptr, L.col, opA<T>(L), x, (const T*)nullptr, y, w, nullptr, s, flag, u);
-      });
+      L.unr[1][0] = pick([&](int u) { level_bsr<T>(D, L, 0, x, (const T*)nullptr, y, w, nullptr, s, true, u); });
   };
   for (int l = 0; l + 1 < D.nlev; ++l) {
     if (D.precision == 0) tune_level(0.0, D.lev[l], l);
@@ -1513,7 +1621,7 @@ int dev_bind(cdg_handle* h, void* buf, int64_t bytes, void* stream) {
   const int prec = h->opt.precision == 2 ? 1 : h->opt.precision;
   const int64_t need =
       (int64_t)layout(H, prec, h->opt.nrhs, nullptr, nullptr, h->opt.precision, gmres_len(h->opt), h->opt.maxit,
-                      h->opt.tc_fp64_apply);
+                      h->opt.tc_fp64_apply, digit_form(h->opt));
   if (bytes < need) {
     h->err = "device buffer too small: need " + std::to_string(need) + " bytes";
     return CDG_ENOMEM;
@@ -1528,7 +1636,7 @@ int dev_bind(cdg_handle* h, void* buf, int64_t bytes, void* stream) {
   D.base = (char*)buf;
   D.bytes = bytes;
   layout(H, prec, h->opt.nrhs, &D, (char*)buf, h->opt.precision, gmres_len(h->opt), h->opt.maxit,
-         h->opt.tc_fp64_apply);
+         h->opt.tc_fp64_apply, digit_form(h->opt));
   D.precision = h->opt.precision == 2 ? 1 : h->opt.precision;
   cudaStream_t s = (cudaStream_t)stream;
   const int nlev = D.nlev;
@@ -1538,6 +1646,7 @@ int dev_bind(cdg_handle* h, void* buf, int64_t bytes, void* stream) {
     upload(L.rowptr, to_i32(A.rowptr), s);
     upload(L.col, A.col, s);
     if (L.A) upload(L.A, A.val, s);
+    if (L.ell) upload(L.ell, padded_columns(A, L.well), s);
     if (L.A32) upload(L.A32, to_f32(A.val), s);
     if (l + 1 < nlev) {
       if (L.Dinv) upload(L.Dinv, H.Dinv_t[l], s);
@@ -1549,15 +1658,36 @@ int dev_bind(cdg_handle* h, void* buf, int64_t bytes, void* stream) {
       upload(L.hrowptr, to_i32(Sh.rowptr), s);
       upload(L.hcol, Sh.col, s);
       if (L.Ahat) upload(L.Ahat, Sh.val, s);
+      if (L.hell) upload(L.hell, padded_columns(Sh, L.whell), s);
       if (L.Ahat32) upload(L.Ahat32, to_f32(Sh.val), s);
+      if (L.Lx) {
+        upload(L.Lx, H.L_t[l], s);
+        upload(L.Rx, transposed_blocks(H.L_t[l], L.np), s);
+      }
     }
     if (l > 0) upload(L.childptr, H.childptr_t[l], s);
+    if (L.Aplain) upload(L.Aplain, A.val, s);
     if (L.chunk) {
       int rows = 0, parents = 0;
       upload(L.chunk, agglomerate_chunks(H.childptr_t[l + 1], chunk_target(L.np), &rows, &parents), s);
     }
     // every synchronous upload above finishes before the host vectors die
     cudaStreamSynchronize(s);
+  }
+  if (D.fixed) {   // FP64 blocks to digits (the restriction reads the next level's children ranges)
+    bool ok = true;
+    for (int l = 0; l < nlev; ++l) {
+      const DevLevel& L = D.lev[l];
+      if (L.A) ok = ok && fx_encode(L.np, L.n, L.rowptr, L.A, L.eA, s);
+      if (L.Ahat) ok = ok && fx_encode(L.np, L.n, L.hrowptr, L.Ahat, L.eH, s);
+      if (L.Dinv) ok = ok && fx_encode(L.np, L.n, nullptr, L.Dinv, L.eD, s);
+      if (L.Lx) ok = ok && fx_encode(L.np, L.n, nullptr, L.Lx, L.eL, s);
+      if (L.Rx) ok = ok && fx_encode(L.np, D.lev[l + 1].n, D.lev[l + 1].childptr, L.Rx, L.eR, s);
+    }
+    if (!ok) {
+      h->err = "unsupported number of basis functions per element";
+      return CDG_EINVAL;
+    }
   }
   upload(D.coarse_inv, H.coarse_inv, s);
   {
@@ -1660,14 +1790,11 @@ int dev_level_op(cdg_handle* h, int op, int level, const double* x, const double
   bool ok = true;
   // caller vectors that are not 16-byte aligned take the kernel without vector loads
   const bool aligned = (((uintptr_t)x | (uintptr_t)y | (uintptr_t)b) & 15) == 0;
-  double* flag = aligned ? D.scal + S_FLAG : nullptr;
   if (op <= 1) {
-    ok = launch_bsr<double>(op, L.np, L.n, L.rowptr, L.col, L.A, x, b, y, h->opt.omega, nullptr, s, flag,
-                            unr_of<double>(L, op));
+    ok = level_bsr<double>(D, L, op, x, b, y, h->opt.omega, nullptr, s, aligned);
   } else if (op == 2) {
-    ok = launch_smooth_first<double>(L.np, L.n, L.Dinv, b, (double*)L.bh, (double*)nullptr, h->opt.omega, s) &&
-         launch_bsr<double>(3, L.np, L.n, L.hrowptr, L.hcol, L.Ahat, x, (const double*)L.bh, y, h->opt.omega,
-                            nullptr, s, flag, unr_of<double>(L, 3));
+    ok = level_smooth_first<double>(D, L, b, (double*)L.bh, (double*)nullptr, h->opt.omega, s) &&
+         level_bsr<double>(D, L, 3, x, (const double*)L.bh, y, h->opt.omega, nullptr, s, aligned);
   }
   else if (op == 3) ok = transfer_restrict<double>(D, level, L.L, x, y, s);
   else ok = transfer_prolong<double>(D, level, L.L, x, y, true, s);
@@ -1758,14 +1885,12 @@ static int cg_part1(cdg_handle* h, cudaStream_t s) {
   const DevLevel& L0 = D.lev[0];
   const unsigned gseg = (unsigned)(D.nseg * D.bps);
   if (D.nseg == 1) {
-    const unsigned g = rows_grid(L0.n, D.np);
-    launch_bsr<double>(0, D.np, L0.n, L0.rowptr, L0.col, L0.A, D.p, (const double*)nullptr, D.q, h->opt.omega,
-                       D.partial, s, D.scal + S_FLAG, unr_of<double>(L0, 0));
+    const unsigned g = D.fixed ? fx_grid(operator_op(L0, 0)) : rows_grid(L0.n, D.np);
+    level_bsr<double>(D, L0, 0, D.p, (const double*)nullptr, D.q, h->opt.omega, D.partial, s);
     launch(finalize_kernel, 1u, kThreads, s, (const double*)D.partial, (int)g, D.npartial, 0, 0, h->opt.tol,
            D.scal);
   } else {
-    launch_bsr<double>(0, D.np, L0.n, L0.rowptr, L0.col, L0.A, D.p, (const double*)nullptr, D.q, h->opt.omega,
-                       (double*)nullptr, s, D.scal + S_FLAG, unr_of<double>(L0, 0));
+    level_bsr<double>(D, L0, 0, D.p, (const double*)nullptr, D.q, h->opt.omega, nullptr, s);
     int rc = dot_to(h, D.p, D.q, nullptr, 0, s);
     if (rc != CDG_OK) return rc;
   }
@@ -1907,8 +2032,7 @@ int dev_solve(cdg_handle* h, const double* f_q, const double* gD, const double* 
   const DevLevel& L0 = D.lev[0];
   if (use_u0) {
     launch(permute_kernel, vec_grid(n), kThreads, s, (int)D.ne, D.np, D.perm0, u_dev, D.x, 1);
-    launch_bsr<double>(1, D.np, L0.n, L0.rowptr, L0.col, L0.A, D.x, D.bt, D.r, o.omega, nullptr, s, D.scal + S_FLAG,
-                       unr_of<double>(L0, 1));
+    level_bsr<double>(D, L0, 1, D.x, D.bt, D.r, o.omega, nullptr, s);
   } else {
     cudaMemsetAsync(D.x, 0, sizeof(double) * n, s);
     cudaMemcpyAsync(D.r, D.bt, sizeof(double) * n, cudaMemcpyDeviceToDevice, s);

@@ -1,0 +1,311 @@
+// Device side of the FP64 block products in integer digits (device_fixed.cu says why and how): the
+// digits, their products and the work of one warp on one pack of rows, shared by the kernels of
+// device_fixed.cu and the persistent V-cycle (device_persist.cu), whose results are therefore the same.
+#pragma once
+
+#include <cuda_runtime.h>
+
+#include "device_fixed.h"
+
+namespace fx {
+
+
+constexpr int kFxThreads = 128;
+constexpr int kFxWarps = kFxThreads / 32;
+constexpr int kMaxTerms = 127;
+constexpr int kNotFinite = 1 << 20;   // row exponent of a matrix row that holds an infinity or NaN
+
+// blocks of a row per step of a group: the level-0 rows of tetrahedra hold five; where
+// all groups of a warp share a row their terms together stay within kMaxTerms
+constexpr int fx_chunk(int np, bool wpr) {
+  const int c = np == 4 || np == 10 || np == 20 ? 5 : 4;
+  const int most = kMaxTerms / (np * (wpr ? 32 / np : 1));
+  return c < most ? c : most;
+}
+constexpr bool fx_one(int mode) { return mode == 4 || mode == 6 || mode == 7; }   // one block per row
+// resident CTAs of 128 threads per SM that the registers are held to
+constexpr int fx_ctas_per_sm(int np) { return np > 10 ? 4 : 8; }
+
+// position of entry (i, j) of a block in the digit layout
+__host__ __device__ constexpr int fx_pos(int np, int i, int j) {
+  return np % 2 == 0 ? ((j >> 1) * np + i) * 2 + (j & 1) : j * np + i;
+}
+
+__device__ __forceinline__ int biased_exponent(double v) {
+  return (__double2hiint(v) >> 20) & 0x7FF;
+}
+
+// v 2^(58 - E) rounded to an integer, |v| < 2^E, as digits (E = em - 1022, em the biased
+// exponent field of the largest value); subnormal values keep their own scale
+// (exponent field 1, no implicit bit)
+__device__ __forceinline__ int2 split_digits(double v, int em) {
+  const long long bits = __double_as_longlong(v);
+  const int e = (int)(bits >> 52) & 0x7FF;
+  unsigned long long m = (unsigned long long)bits & 0xFFFFFFFFFFFFFull;
+  if (e) m |= 1ull << 52;
+  const int s = min(em - max(e, 1), 63);
+  long long q = (long long)((((m << 6) >> s) + 1) >> 1);
+  const long long sg = bits >> 63;
+  q = (q ^ sg) - sg;
+  const int lo = ((int)((unsigned int)q << 2)) >> 2;   // the low 30 bits, signed
+  return make_int2((int)((q - lo) >> 30), lo);
+}
+
+// d 2^e: on the exponent field where the result is a normal number
+__device__ __forceinline__ double scale2(double d, int e) {
+  const int f = biased_exponent(d) + e;
+  if (d == 0.0) return d;
+  if (f >= 1 && f <= 2046 && biased_exponent(d) != 0)
+    return __longlong_as_double(__double_as_longlong(d) + ((long long)e << 52));
+  return scalbn(d, e);
+}
+
+// A sum of digit products, hi 2^60 + lo with 0 <= lo < 2^60 after carrying
+struct Acc {
+  long long hh = 0, mm = 0, ll = 0;
+  // carries of one block's products into the higher sums
+  __device__ __forceinline__ void carry() {
+    mm += ll >> 30;
+    ll &= 0x3FFFFFFF;
+    hh += mm >> 30;
+    mm &= 0x3FFFFFFF;
+  }
+  __device__ __forceinline__ unsigned long long low() const { return ((unsigned long long)mm << 30) | ll; }
+};
+
+// (hi 2^60 + lo) 2^(e - 116), rounded once; e = EA + EX of the digits' scales
+__device__ __forceinline__ double fx_value(long long hi, unsigned long long lo, int e) {
+  const int k = min(60, __clzll(hi ^ (hi >> 63)) - 1);   // low bits that fit beside hi in 63 bits
+  const long long v = (long long)((unsigned long long)hi << k) | (long long)(lo >> (60 - k));
+  return scale2(__ll2double_rn(v), e - 56 - k);
+}
+
+template <int NP>
+struct DigitRow {
+  int h[NP], l[NP];
+  // row i of the block at a (digit layout)
+  __device__ __forceinline__ void load(const int2* __restrict__ a, int i) {
+    if constexpr (NP % 2 == 0) {
+      const int4* p = reinterpret_cast<const int4*>(a) + i;
+#pragma unroll
+      for (int j = 0; j < NP / 2; ++j) {
+        const int4 t = __ldg(p + j * NP);
+        h[2 * j] = t.x;
+        l[2 * j] = t.y;
+        h[2 * j + 1] = t.z;
+        l[2 * j + 1] = t.w;
+      }
+    } else {
+#pragma unroll
+      for (int j = 0; j < NP; ++j) {
+        const int2 t = __ldg(a + j * NP + i);
+        h[j] = t.x;
+        l[j] = t.y;
+      }
+    }
+  }
+};
+
+__device__ __forceinline__ void mac(Acc& s, int ah, int al, int xh, int xl) {
+  s.hh += (long long)ah * xh;
+  s.mm += (long long)ah * xl;
+  s.mm += (long long)al * xh;
+  s.ll += (long long)al * xl;
+}
+
+template <int NP>
+__device__ __forceinline__ void fx_mac(const DigitRow<NP>& r, const int2* __restrict__ xs, Acc& s) {
+  if constexpr (NP % 2 == 0) {
+    const int4* x4 = reinterpret_cast<const int4*>(xs);
+#pragma unroll
+    for (int j = 0; j < NP / 2; ++j) {
+      const int4 t = x4[j];
+      mac(s, r.h[2 * j], r.l[2 * j], t.x, t.y);
+      mac(s, r.h[2 * j + 1], r.l[2 * j + 1], t.z, t.w);
+    }
+  } else {
+#pragma unroll
+    for (int j = 0; j < NP; ++j) {
+      const int2 t = xs[j];
+      mac(s, r.h[j], r.l[j], t.x, t.y);
+    }
+  }
+  s.carry();
+}
+
+// what becomes of a row's sum (modes below); returns the dot partial of mode 0
+template <int MODE>
+__device__ __forceinline__ double finish(double acc, size_t o, double xo, double bo, double* y, double* y2,
+                                         double omega, double dsum) {
+  if constexpr (MODE == 1) y[o] = bo - acc;
+  else if constexpr (MODE == 3) y[o] = fma(omega, bo - xo - acc, xo);
+  else if constexpr (MODE == 4) y[o] = xo + acc;
+  else y[o] = acc;
+  if constexpr (MODE == 6) y2[o] = omega * acc;
+  return MODE == 0 ? fma(xo, acc, dsum) : dsum;
+}
+
+template <bool COHERENT>
+__device__ __forceinline__ double vload(const double* p) { return COHERENT ? __ldcg(p) : *p; }
+
+// digits of one warp's gathered values in shared memory
+template <int NP, int MODE, bool WPR>
+struct Pack {
+  static constexpr int RPW = 32 / NP;
+  static constexpr bool ONE = fx_one(MODE);
+  static constexpr int CH = ONE ? 1 : fx_chunk(NP, WPR);
+  static constexpr int SPL = WPR ? RPW : 1;                       // groups that share a block row
+  static constexpr int GS = CH * NP + 2 + (CH * NP) % 2;          // digits of one group's chunk (padded against bank conflicts)
+  static constexpr int DIGITS = RPW * GS;
+};
+
+// One warp on one pack of rows: acc = (A x)_(K, i), then by MODE: 0 y = acc; 1 y = b - acc;
+// 3 y = x + omega (b - x - acc); 8 y = acc, block t meeting element t; with one block per row (no
+// rowptr): 4 y += acc; 6 y = acc, y2 = omega acc; 7 y = acc.  Returns the dot partial of mode 0.
+// q.cols: the rows' columns, q.width of them per row (missing: -1), so that the gathers of x need not
+// wait for the row pointer; one-block modes meet element cols[K] (nullptr: K).
+// COHERENT: vectors are read through L2 only (written earlier in the same kernel).
+template <int NP, int MODE, bool WPR, bool COHERENT>
+__device__ __forceinline__ double fx_pack(const FxOp& q, int pack, int2* __restrict__ digits, double dsum) {
+  using P = Pack<NP, MODE, WPR>;
+  constexpr int RPW = P::RPW, CH = P::CH, SPL = P::SPL;
+  constexpr bool ONE = P::ONE;
+  const int2* A = reinterpret_cast<const int2*>(q.A);
+  const int lane = threadIdx.x & 31;
+  const int sub = lane / NP;
+  const int i = lane - sub * NP;
+  const bool grp = sub < RPW;
+  int2* xs = digits + (grp ? sub : 0) * P::GS;
+  const int K = WPR ? pack : pack * RPW + sub;
+  const bool active = grp && K < q.n;
+  int b0 = K, nb = active ? 1 : 0;
+  if constexpr (!ONE) {
+    b0 = active ? __ldg(q.rowptr + K) : 0;
+    nb = active ? __ldg(q.rowptr + K + 1) - b0 : 0;
+  }
+  // blocks of this group: b0 + sub, b0 + sub + SPL, ... (WPR) or all of the row
+  const int cnt = !active ? 0 : WPR ? (nb - sub + SPL - 1) / SPL : nb;
+  const int first = WPR ? b0 + sub : b0;
+  const int maxc = __reduce_max_sync(0xffffffffu, cnt);
+  Acc sum;
+  int ex = 0, terms = 0;                           // running exponent field of the x digits, terms summed
+  double flushed = 0.0;
+  bool any_flush = false, special = false;
+  const bool writes = active && (!WPR || sub == 0);
+  const size_t o = (size_t)K * NP + i;
+  const int ea = active ? __ldg(q.EA + o) : 0;
+  double xo = 0.0, bo = 0.0;                       // the epilogue's operands, on their way early
+  if (writes) {
+    if constexpr (MODE == 4) xo = vload<COHERENT>(q.y + o);
+    if constexpr (MODE == 1 || MODE == 3) bo = vload<COHERENT>(q.b + o);
+  }
+  for (int base = 0; base < maxc; base += CH) {
+    double xv[CH];
+    int em = 0;
+    DigitRow<NP> row;
+#pragma unroll
+    for (int c = 0; c < CH; ++c) {
+      const int t = base + c;
+      int J = -1;
+      if constexpr (ONE) {
+        if (active) J = q.cols ? __ldg(q.cols + K) : K;
+      } else if (q.cols) {
+        const int tt = WPR ? sub + t * SPL : t;
+        if (active && tt < q.width) J = __ldg(q.cols + (size_t)K * q.width + tt);
+      } else if (t < cnt) {
+        J = first + t * SPL;
+      }
+      xv[c] = J >= 0 ? vload<COHERENT>(q.x + (size_t)J * NP + i) : 0.0;
+    }
+    if (base < cnt) row.load(A + (size_t)(first + base * SPL) * NP * NP, i);
+#pragma unroll
+    for (int c = 0; c < CH; ++c) em = max(em, biased_exponent(xv[c]));
+    em = max(1, __reduce_max_sync(0xffffffffu, em));
+    if (em == 0x7FF) {
+      special = true;
+      break;
+    }
+    if (em > ex || terms + CH * NP * SPL > kMaxTerms) {   // the same in every lane
+      if (terms > 0) {
+        flushed += fx_value(sum.hh, sum.low(), ea + ex - 1022);
+        any_flush = true;
+        sum = Acc();
+        terms = 0;
+      }
+      ex = max(em, ex);
+    }
+    terms += CH * NP * SPL;
+    __syncwarp();
+#pragma unroll
+    for (int c = 0; c < CH; ++c)
+      if (base + c < maxc) {   // the same in every lane
+        const int2 d = split_digits(xv[c], ex);
+        if (grp) xs[c * NP + i] = d;
+      }
+    __syncwarp();
+#pragma unroll
+    for (int c = 0; c < CH; ++c) {
+      if (base + c < cnt) {
+        fx_mac<NP>(row, xs + c * NP, sum);
+        if (c + 1 < CH && base + c + 1 < cnt) row.load(A + (size_t)(first + (base + c + 1) * SPL) * NP * NP, i);
+      }
+    }
+  }
+  double acc;
+  if (special) {
+    // an infinity or NaN among the values: FP64 products, so that it spreads as IEEE arithmetic says
+    acc = 0.0;
+    for (int t = 0; t < cnt; ++t) {
+      const int blk = first + t * SPL;
+      const int J = ONE ? (q.cols ? q.cols[K] : K) : q.cols ? q.cols[(size_t)K * q.width + (WPR ? sub + t * SPL : t)] : blk;
+      const double* xj = q.x + (size_t)J * NP;
+      for (int j = 0; j < NP; ++j) {
+        const int2 d = A[(size_t)blk * NP * NP + fx_pos(NP, i, j)];
+        acc = fma(scale2(__ll2double_rn(((long long)d.x << 30) + d.y), ea - 58), vload<COHERENT>(xj + j), acc);
+      }
+    }
+    any_flush = true;
+  } else if (any_flush) {
+    acc = flushed + fx_value(sum.hh, sum.low(), ea + ex - 1022);
+  }
+  long long hi = sum.hh;
+  unsigned long long lo = sum.low();
+  if constexpr (WPR && RPW > 1) {
+    // sum over the groups of the row: the integer sums exactly
+    if (any_flush) {
+#pragma unroll
+      for (int m = RPW; m > 1; m = (m + 1) / 2) {
+        const int h = (m + 1) / 2;
+        const double t = __shfl_down_sync(0xffffffffu, acc, h * NP);
+        if (sub + h < m) acc += t;
+      }
+    } else {
+#pragma unroll
+      for (int m = RPW; m > 1; m = (m + 1) / 2) {
+        const int h = (m + 1) / 2;
+        const long long th = __shfl_down_sync(0xffffffffu, hi, h * NP);
+        const unsigned long long tl = __shfl_down_sync(0xffffffffu, lo, h * NP);
+        if (sub + h < m) {   // at most ten groups: the low parts stay below 2^64
+          hi += th;
+          lo += tl;
+        }
+      }
+      hi += (long long)(lo >> 60);
+      lo &= (1ull << 60) - 1;
+    }
+  }
+  if (!any_flush) acc = fx_value(hi, lo, ea + ex - 1022);
+  if (ea == kNotFinite) acc = nan("");
+  if (writes && (MODE == 3 || (MODE == 0 && q.dot))) xo = vload<COHERENT>(q.x + o);
+  return writes ? finish<MODE>(acc, o, xo, bo, q.y, q.y2, q.omega, dsum) : dsum;
+}
+
+// one block row per warp (see device_fixed.cu)
+constexpr int kFxSms = 152;
+inline bool warp_per_row(int mode, int np, int n, int64_t blocks) {
+  const int rpw = 32 / np, resident = kFxSms * kFxWarps * fx_ctas_per_sm(np);
+  if (fx_one(mode) || rpw < 2) return false;
+  return n <= resident || (blocks >= (int64_t)n * 3 * rpw && n <= 4 * resident);
+}
+
+}  // namespace fx

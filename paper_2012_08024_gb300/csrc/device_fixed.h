@@ -1,0 +1,40 @@
+// FP64 block-sparse products by exact integer arithmetic (device_fixed.cu).
+#pragma once
+
+#include <cuda_runtime.h>
+
+#include <cstdint>
+
+// One product with a block-sparse matrix in digit form and what is done with it:
+// mode 0 y = A x (dot: per-CTA partials of x . y, fx_grid of them), 1 y = b - A x,
+// 3 y = x + omega (b - x - A x), 8 y = A x with block t meeting element t; with one block per row
+// (no rowptr): 4 y += A x, 6 y = A x and y2 = omega A x, 7 y = A x.
+// x and y do not overlap.
+struct FxOp {
+  int mode = 0, np = 0, n = 0;
+  int64_t blocks = 0;         // blocks of the matrix
+  const int* rowptr = nullptr;
+  const int* cols = nullptr;  // [n][width], -1 behind a row's last block; one-block modes: [n] or nullptr (K)
+  int width = 0;
+  const void* A = nullptr;    // digits
+  const int* EA = nullptr;    // [n][np] row exponents
+  const double* x = nullptr;
+  const double* b = nullptr;
+  double* y = nullptr;
+  double* y2 = nullptr;
+  double omega = 0.0;
+  double* dot = nullptr;
+};
+
+struct DevLevel;
+// products with a level's operators: A (modes 0, 1) or Ahat (3); a diagonal of blocks (6, 7); the
+// prolongation to level F from its parents (4, 7); the restriction from F to the next level C (8)
+FxOp operator_op(const DevLevel& L, int mode);
+FxOp diagonal_op(const DevLevel& L, int mode, const double* blocks, const int* exps);
+FxOp prolong_op(const DevLevel& F, int mode = 4);
+FxOp restrict_op(const DevLevel& F, const DevLevel& C);
+
+unsigned fx_grid(const FxOp& o);                  // CTAs of fx_run
+bool fx_run(const FxOp& o, cudaStream_t s);       // false: no instance for this np
+// FP64 blocks [blocks][np][np] of n block rows to digits, in place, with the row exponents EA [n][np]
+bool fx_encode(int np, int n, const int* rowptr, double* A, int* EA, cudaStream_t s);

@@ -778,6 +778,9 @@ bool mr_vcycle(DeviceState& D, MR& M, const cdg_options& o, const float* b0, flo
   return true;
 }
 
+// A_0 as FP64 numbers
+inline const double* plain_A0(const DeviceState& D) { return D.fixed ? D.lev[0].Aplain : D.lev[0].A; }
+
 // maxb_ready: the column exponents of x are already in M.oz_maxb (mr_p_kernel
 // stores them for p); pq_groups (split apply only): the apply also leaves the
 // partial sums of x . y in M.partial, *pq_groups of them per column
@@ -789,7 +792,7 @@ bool mr_apply64(DeviceState& D, MR& M, const double* x, double* y, cudaStream_t 
                     pq_groups ? M.partial : nullptr, pq_groups, M.tc_err, D.wait_limit, s);
   const int tx = tile_of(M, 0, 0), br = rows_of(M, 0, 0), rc = cols_of(M, 0, 0);
   MR_NP_DISPATCH(D.np, (mr_bsr_launch<double, double, double, NP, 0>(tx, br, rc, false, L0.n, M.R, L0.rowptr, L0.col,
-                                                                     L0.A,
+                                                                     plain_A0(D),
                                                                      x, (const double*)nullptr, y, 0.0, s)));
   return true;
 }
@@ -836,7 +839,7 @@ bool mr_autotune(DeviceState& D, MR& M, double omega, cudaStream_t s) {
     cudaMemsetAsync(M.p, 0, nv * sizeof(double), s);
     pick(0, 0, [&](int tx, int br, int rc, bool) {
       MR_NP_DISPATCH_V(np, (mr_bsr_launch<double, double, double, NP, 0>(tx, br, rc, false, L0.n, R, L0.rowptr, L0.col,
-                                                                         L0.A,
+                                                                         plain_A0(D),
                                                                          (const double*)M.p, (const double*)nullptr,
                                                                          M.q, 0.0, s)));
     });

@@ -19,6 +19,7 @@
 #include <algorithm>
 #include <cstdint>
 
+#include "device_fixed.cuh"
 #include "device_kernels.cuh"
 #include "device_state.h"
 
@@ -36,6 +37,10 @@ struct PLevel {
   const int *rowptr, *col, *hrowptr, *hcol, *parent, *childptr;
   const void *A, *Ahat, *Dinv, *L;
   void *x, *t, *r, *b, *bh;
+  // FP64 (digit form, device_fixed.cu): products with A, Ahat, D^-1, L^T (to the next level) and L;
+  // the vectors are filled in by the phases
+  FxOp oA, oH, oD, oR, oL;
+  int wprA, wprH, wprR;   // one block row per warp, as in the per-phase kernels
 };
 
 struct PParams {
@@ -174,9 +179,88 @@ __device__ void ph_coarse(const PParams& P, const T* b, T* x, bool add) {
   }
 }
 
+// FP64: a product in digit form, by the same packs as the per-phase kernels.  Three CTAs per SM:
+// V-cycle of the 181^2 (p = 2) mesh 324 -> 278 us against FP64 blocks, 32^2 137 -> 121 us, but the
+// 64-mesh batch 63.5 -> 76.6 ms per solve (its phases wait for memory, and 24 warps per SM hide less
+// than the 40 of the FP64-block kernel); two CTAs 265 us, 102 us, 80.3 ms.
+template <int NP>
+constexpr int most_digits() {
+  constexpr int packed = fx::Pack<NP, 8, false>::DIGITS, shared = fx::Pack<NP, 8, true>::DIGITS;
+  return packed > shared ? packed : shared;
+}
+
+template <int NP, int MODE, bool WPR>
+__device__ __forceinline__ void fx_phase(const FxOp* op) {
+  extern __shared__ __align__(16) int2 warp_digits[];   // [warps][most_digits]
+  int2* digits = warp_digits + (threadIdx.x >> 5) * most_digits<NP>();
+  const FxOp q = *op;   // into registers
+  constexpr int RPW = fx::Pack<NP, MODE, WPR>::RPW;
+  const int packs = WPR ? q.n : (q.n + RPW - 1) / RPW;
+  const int warps = (int)(gridDim.x * (blockDim.x >> 5));
+  for (int p = (int)(blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5)); p < packs; p += warps)
+    fx::fx_pack<NP, MODE, WPR, true>(q, p, digits, 0.0);
+}
+
+template <int NP, int MODE>
+__device__ __forceinline__ void fx_product(FxOp q, bool wpr, const double* x, const double* b, double* y, double* y2,
+                                           double omega) {
+  q.x = x;
+  q.b = b;
+  q.y = y;
+  q.y2 = y2;
+  q.omega = omega;
+  if (wpr) {
+    if constexpr (!fx::fx_one(MODE) && 32 / NP > 1) fx_phase<NP, MODE, true>(&q);
+  } else {
+    fx_phase<NP, MODE, false>(&q);
+  }
+}
+
+// the phases in the precision of the cycle
 template <typename T, int NP>
-__global__ void __launch_bounds__(kPThreads) vcycle_persistent_kernel(PParams P) {
-  constexpr bool VEC = NP % 2 == 0;
+struct Phase {
+  static constexpr bool VEC = NP % 2 == 0;
+  static __device__ void first(const PLevel& L, const T* b, T* bh, T* x, T w, bool write_x) {
+    ph_first<T, NP>(L.n, (const T*)L.Dinv, b, bh, x, w, write_x);
+  }
+  static __device__ void sweep(const PLevel& L, const T* x, const T* bh, T* y, T w) {
+    ph_bsr<T, NP, VEC, 3>(L.n, L.hrowptr, L.hcol, (const T*)L.Ahat, x, bh, y, w);
+  }
+  static __device__ void residual(const PLevel& L, const T* x, const T* b, T* r, T w) {
+    ph_bsr<T, NP, VEC, 1>(L.n, L.rowptr, L.col, (const T*)L.A, x, b, r, w);
+  }
+  static __device__ void restrict_to(const PLevel& L, const PLevel& C, const T* r, T* bc) {
+    ph_restrict<T, NP>(C.n, C.childptr, (const T*)L.L, r, bc);
+  }
+  static __device__ void prolong(const PLevel& L, const T* xc, T* x, bool add) {
+    ph_prolong<T, NP>(L.n, L.parent, (const T*)L.L, xc, x, add);
+  }
+};
+
+template <int NP>
+struct Phase<double, NP> {
+  static __device__ void first(const PLevel& L, const double* b, double* bh, double* x, double w, bool write_x) {
+    if (write_x) fx_product<NP, 6>(L.oD, false, b, nullptr, bh, x, w);
+    else fx_product<NP, 7>(L.oD, false, b, nullptr, bh, nullptr, w);
+  }
+  static __device__ void sweep(const PLevel& L, const double* x, const double* bh, double* y, double w) {
+    fx_product<NP, 3>(L.oH, L.wprH, x, bh, y, nullptr, w);
+  }
+  static __device__ void residual(const PLevel& L, const double* x, const double* b, double* r, double w) {
+    fx_product<NP, 1>(L.oA, L.wprA, x, b, r, nullptr, w);
+  }
+  static __device__ void restrict_to(const PLevel& L, const PLevel&, const double* r, double* bc) {
+    fx_product<NP, 8>(L.oR, L.wprR, r, nullptr, bc, nullptr, 0.0);
+  }
+  static __device__ void prolong(const PLevel& L, const double* xc, double* x, bool add) {
+    if (add) fx_product<NP, 4>(L.oL, false, xc, nullptr, x, nullptr, 0.0);
+    else fx_product<NP, 7>(L.oL, false, xc, nullptr, x, nullptr, 0.0);
+  }
+};
+
+template <typename T, int NP>
+__global__ void __launch_bounds__(kPThreads, 3) vcycle_persistent_kernel(const __grid_constant__ PParams P) {
+  using Ph = Phase<T, NP>;
   const T w = (T)P.omega;
   const int nlev = P.nlev;
   // where each level's iterate is at the end of its downward (x_down) and upward (x_fin) visit
@@ -191,21 +275,21 @@ __global__ void __launch_bounds__(kPThreads) vcycle_persistent_kernel(PParams P)
     T* xa = (T*)L.x;
     T* xb = (T*)L.t;
     if (P.nu_pre >= 1) {
-      ph_first<T, NP>(L.n, (const T*)L.Dinv, b, (T*)L.bh, xa, w, true);
+      Ph::first(L, b, (T*)L.bh, xa, w, true);
       CDG_SYNC;
       for (int k = 1; k < P.nu_pre; ++k) {
-        ph_bsr<T, NP, VEC, 3>(L.n, L.hrowptr, L.hcol, (const T*)L.Ahat, xa, (const T*)L.bh, xb, w);
+        Ph::sweep(L, xa, (const T*)L.bh, xb, w);
         CDG_SYNC;
         T* tmp = xa;
         xa = xb;
         xb = tmp;
       }
-      ph_bsr<T, NP, VEC, 1>(L.n, L.rowptr, L.col, (const T*)L.A, xa, b, (T*)L.r, w);
+      Ph::residual(L, xa, b, (T*)L.r, w);
       CDG_SYNC;
-      ph_restrict<T, NP>(P.lev[l + 1].n, P.lev[l + 1].childptr, (const T*)L.L, (const T*)L.r, (T*)P.lev[l + 1].b);
+      Ph::restrict_to(L, P.lev[l + 1], (const T*)L.r, (T*)P.lev[l + 1].b);
     } else {
-      ph_first<T, NP>(L.n, (const T*)L.Dinv, b, (T*)L.bh, xa, w, false);
-      ph_restrict<T, NP>(P.lev[l + 1].n, P.lev[l + 1].childptr, (const T*)L.L, b, (T*)P.lev[l + 1].b);
+      Ph::first(L, b, (T*)L.bh, xa, w, false);
+      Ph::restrict_to(L, P.lev[l + 1], b, (T*)P.lev[l + 1].b);
     }
     x_down[l] = xa;
     CDG_SYNC;
@@ -218,7 +302,7 @@ __global__ void __launch_bounds__(kPThreads) vcycle_persistent_kernel(PParams P)
     ph_coarse<T>(P, bc, xc, false);
     if (P.refine) {
       CDG_SYNC;
-      ph_bsr<T, NP, VEC, 1>(C.n, C.rowptr, C.col, (const T*)C.A, xc, bc, (T*)C.r, w);
+      Ph::residual(C, xc, bc, (T*)C.r, w);
       CDG_SYNC;
       ph_coarse<T>(P, (const T*)C.r, xc, true);
     }
@@ -231,11 +315,11 @@ __global__ void __launch_bounds__(kPThreads) vcycle_persistent_kernel(PParams P)
     const PLevel& L = P.lev[l];
     T* xa = x_down[l];
     T* xb = xa == (T*)L.x ? (T*)L.t : (T*)L.x;
-    ph_prolong<T, NP>(L.n, L.parent, (const T*)L.L, x_fin[l + 1], xa, P.nu_pre >= 1);
+    Ph::prolong(L, x_fin[l + 1], xa, P.nu_pre >= 1);
     for (int k = 0; k < P.nu_post; ++k) {
       CDG_SYNC;
       T* out = (l == 0 && k + 1 == P.nu_post) ? (T*)P.z0 : xb;
-      ph_bsr<T, NP, VEC, 3>(L.n, L.hrowptr, L.hcol, (const T*)L.Ahat, xa, (const T*)L.bh, out, w);
+      Ph::sweep(L, xa, (const T*)L.bh, out, w);
       xb = xa;
       xa = out;
     }
@@ -253,7 +337,8 @@ template <typename T, int NP>
 int launch_one(const PParams& P, cudaStream_t s, int* grid_out) {
   auto kern = vcycle_persistent_kernel<T, NP>;
   int per_sm = 0;
-  if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, kPThreads, 0) != cudaSuccess || per_sm < 1)
+  const size_t smem = sizeof(T) == 8 ? (kPThreads / 32) * most_digits<NP>() * sizeof(int2) : 0;
+  if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, kPThreads, smem) != cudaSuccess || per_sm < 1)
     return -1;
   int dev = 0, sms = 0;
   cudaGetDevice(&dev);
@@ -262,7 +347,7 @@ int launch_one(const PParams& P, cudaStream_t s, int* grid_out) {
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3((unsigned)grid);
   cfg.blockDim = dim3(kPThreads);
-  cfg.dynamicSmemBytes = 0;
+  cfg.dynamicSmemBytes = smem;
   cfg.stream = s;
   cudaLaunchAttribute attr[1];
   attr[0].id = cudaLaunchAttributeCooperative;
@@ -281,6 +366,7 @@ int launch_one(const PParams& P, cudaStream_t s, int* grid_out) {
 // count: two device words, cleared here; err: the device error flag.
 bool vcycle_persistent(DeviceState& D, const cdg_options& o, bool fp32, const void* b0, void* z0, unsigned* count,
                        int* err, cudaStream_t s) {
+  if (!fp32 && !D.fixed) return false;
   PParams P = {};
   P.nlev = D.nlev;
   P.nu_pre = o.nu_pre;
@@ -308,6 +394,19 @@ bool vcycle_persistent(DeviceState& D, const cdg_options& o, bool fp32, const vo
     Q.r = L.r;
     Q.b = L.b;
     Q.bh = L.bh;
+    if (!fp32) {
+      const bool last = l + 1 == D.nlev;
+      Q.oA = operator_op(L, 1);
+      Q.wprA = fx::warp_per_row(1, L.np, L.n, L.nnzb);
+      if (!last) {
+        Q.oH = operator_op(L, 3);
+        Q.wprH = fx::warp_per_row(3, L.np, L.n, L.hnnzb);
+        Q.oD = diagonal_op(L, 7, L.Dinv, L.eD);
+        Q.oL = prolong_op(L);
+        Q.oR = restrict_op(L, D.lev[l + 1]);
+        Q.wprR = fx::warp_per_row(8, L.np, Q.oR.n, Q.oR.blocks);
+      }
+    }
   }
   if (P.refine) P.lev[D.nlev - 1].A = D.lev[D.nlev - 1].A;
   P.crow_seg = D.crow_seg;

@@ -27,6 +27,14 @@ struct DevLevel {
   double* A = nullptr;
   double* Dinv = nullptr;
   double* L = nullptr;
+  // digit form (DeviceState::fixed): A, Ahat and Dinv then hold digits with the row
+  // exponents eA, eH, eD; Lx / Rx are L_K and L_K^T (one block row per agglomerate) in
+  // digits for the V-cycle's prolongation and restriction (L itself stays FP64)
+  int *eA = nullptr, *eH = nullptr, *eD = nullptr, *eL = nullptr, *eR = nullptr;
+  double *Lx = nullptr, *Rx = nullptr;
+  int *ell = nullptr, *hell = nullptr;   // columns of A and Ahat as [n][width], -1 behind a row's last
+  int well = 0, whell = 0;
+  double* Aplain = nullptr;  // level 0: A in FP64 for the many-right-hand-side apply
   int* parent = nullptr;
   int* childptr = nullptr;   // children range of each element of this level (l >= 1)
   // chunks of whole agglomerates of level l+1 for the fused residual + restriction
@@ -56,6 +64,7 @@ struct DeviceState {
   int64_t bytes = 0;
   int nlev = 0, np = 0, d = 0, nq = 0, nfq = 0, precision = 0;
   int64_t ne = 0, ndofs = 0, nbf = 0;
+  bool fixed = false;   // FP64 operators in digit form (device_fixed.cu)
   DevLevel lev[kMaxLev];
   double* coarse_inv = nullptr;
   int nc = 0;
