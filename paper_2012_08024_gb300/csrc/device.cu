@@ -411,6 +411,38 @@ __global__ void __launch_bounds__(kThreads, 8 / (UNR < 2 ? 2 : UNR)) smooth_prol
   }
 }
 
+// FP32 levels with few rows: a warp per block row (cdgk::split_row_acc), 128-thread CTAs.  bsr_kernel
+// gives such a level one CTA per 24 (n_p = 10) to 64 (n_p = 4) rows, and a thread its row's blocks
+// one after the other: 59 rows of 43 blocks at n_p = 4 took 18.2 us on 4 CTAs.
+constexpr int kRowThreads = 128;
+
+template <typename T, int NP, int MODE>
+__global__ void __launch_bounds__(kRowThreads) bsr_row_kernel(int n, const int* __restrict__ rowptr,
+                                                              const int* __restrict__ col, const T* __restrict__ A,
+                                                              const T* __restrict__ x, const T* __restrict__ b,
+                                                              T* __restrict__ y, T omega) {
+  const int K = blockIdx.x * (kRowThreads / 32) + (threadIdx.x >> 5);
+  if (K >= n) return;
+  const T acc = cdgk::split_row_acc<T, NP>(K, rowptr, col, A, x);
+  const int i = threadIdx.x & 31;
+  if (i >= NP) return;
+  const size_t row = (size_t)K * NP + i;
+  if (MODE == 0) y[row] = acc;
+  else if (MODE == 1) y[row] = b[row] - acc;
+  else y[row] = x[row] + omega * (b[row] - x[row] - acc);
+}
+
+template <typename T, int NP>
+__global__ void __launch_bounds__(kRowThreads) restrict_row_kernel(int nc, const int* __restrict__ childptr,
+                                                                   const T* __restrict__ L, const T* __restrict__ r,
+                                                                   T* __restrict__ bc) {
+  const int Ag = blockIdx.x * (kRowThreads / 32) + (threadIdx.x >> 5);
+  if (Ag >= nc) return;
+  const T acc = cdgk::split_restrict<T, NP>(Ag, childptr, L, r);
+  const int i = threadIdx.x & 31;
+  if (i < NP) bc[(size_t)Ag * NP + i] = acc;
+}
+
 // bh = Dinv b; with WRITE_X also x = omega bh (first smoothing step from a zero guess)
 template <typename T, int NP, bool WRITE_X>
 __global__ void __launch_bounds__(kThreads) smooth_first_kernel(int n, const T* __restrict__ Dinv,
@@ -1071,6 +1103,23 @@ bool level_bsr(const DeviceState& D, const DevLevel& L, int mode, const T* x, co
       return fx_run(o, s);
     }
   }
+  if constexpr (sizeof(T) == 4) {
+    if (aligned && L.np <= 15 && warp_per_row(L.np, L.n, hat ? L.hnnzb : L.nnzb)) {
+      const unsigned g = (unsigned)((L.n + kRowThreads / 32 - 1) / (kRowThreads / 32));
+      const T* M = hat ? opH<T>(L) : opA<T>(L);
+      switch (L.np) {
+#define CDG_ROW(NPV)                                                                                             \
+  case NPV:                                                                                                      \
+    if (mode == 0) launch(bsr_row_kernel<T, NPV, 0>, g, kRowThreads, s, L.n, rp, cl, M, x, b, y, (T)omega);      \
+    else if (mode == 1) launch(bsr_row_kernel<T, NPV, 1>, g, kRowThreads, s, L.n, rp, cl, M, x, b, y, (T)omega); \
+    else launch(bsr_row_kernel<T, NPV, 3>, g, kRowThreads, s, L.n, rp, cl, M, x, b, y, (T)omega);                \
+    return true;
+        CDG_ROW(3) CDG_ROW(4) CDG_ROW(6) CDG_ROW(10) CDG_ROW(15)
+#undef CDG_ROW
+        default: break;
+      }
+    }
+  }
   return launch_bsr<T>(mode, L.np, L.n, rp, cl, hat ? opH<T>(L) : opA<T>(L), x, b, y, omega, dot, s,
                        aligned ? D.scal + S_FLAG : nullptr, unr);
 }
@@ -1109,6 +1158,18 @@ bool level_restrict(const DeviceState& D, int l, const T* r, T* bc, cudaStream_t
       o.x = r;
       o.y = bc;
       return fx_run(o, s);
+    }
+  } else if (!F.ptrans && F.np <= 15 && warp_per_row(F.np, D.lev[l + 1].n, F.n)) {
+    const int nc = D.lev[l + 1].n;
+    const unsigned g = (unsigned)((nc + kRowThreads / 32 - 1) / (kRowThreads / 32));
+    const int* cp = D.lev[l + 1].childptr;
+    switch (F.np) {
+      case 3: launch(restrict_row_kernel<T, 3>, g, kRowThreads, s, nc, cp, opL<T>(F), r, bc); return true;
+      case 4: launch(restrict_row_kernel<T, 4>, g, kRowThreads, s, nc, cp, opL<T>(F), r, bc); return true;
+      case 6: launch(restrict_row_kernel<T, 6>, g, kRowThreads, s, nc, cp, opL<T>(F), r, bc); return true;
+      case 10: launch(restrict_row_kernel<T, 10>, g, kRowThreads, s, nc, cp, opL<T>(F), r, bc); return true;
+      case 15: launch(restrict_row_kernel<T, 15>, g, kRowThreads, s, nc, cp, opL<T>(F), r, bc); return true;
+      default: break;
     }
   }
   return transfer_restrict<T>(D, l, opL<T>(F), r, bc, s);
@@ -1858,8 +1919,7 @@ int dev_apply_f32(cdg_handle* h, int level, const float* x, float* y, void* stre
   }
   const DevLevel& L = D.lev[level];
   const bool aligned = (((uintptr_t)x | (uintptr_t)y) & 15) == 0;
-  if (!launch_bsr<float>(0, L.np, L.n, L.rowptr, L.col, L.A32, x, (const float*)nullptr, y, h->opt.omega, nullptr,
-                         (cudaStream_t)stream, aligned ? D.scal + S_FLAG : nullptr, unr_of<float>(L, 0))) {
+  if (!level_bsr<float>(D, L, 0, x, (const float*)nullptr, y, h->opt.omega, nullptr, (cudaStream_t)stream, aligned)) {
     h->err = "unsupported n_p";
     return CDG_EINVAL;
   }

@@ -129,14 +129,9 @@ __global__ void __launch_bounds__(kFxThreads) fx_encode_kernel(int n, const int*
     default: return false;                                  \
   }
 
-// One block row per warp while the rows then fit on the GPU at once, or are long (three and more
-// blocks per group): a row's blocks, not the number of rows, are what there is to spread.  256^2,
-// p = 3: 4,135 rows of 7 blocks 8.2 -> 6.9 us; 24^3 tetrahedra, p = 2: 4,875 rows of 10 blocks
-// 12.8 -> 9.4 us; but 8,102 rows of 7 blocks at p = 2 (five groups share a row) 6.3 -> 8.5 us
-// (warp_per_row).
 template <int NP, int MODE>
 unsigned go(const FxOp& o, cudaStream_t s, bool launch) {
-  const bool wpr = warp_per_row(MODE, NP, o.n, o.blocks);
+  const bool wpr = !fx_one(MODE) && warp_per_row(NP, o.n, o.blocks);
   const int packs = wpr ? o.n : (o.n + 32 / NP - 1) / (32 / NP);
   const unsigned g =
       (unsigned)std::max(1, std::min((packs + kFxWarps - 1) / kFxWarps, kFxSms * fx_ctas_per_sm(NP)));

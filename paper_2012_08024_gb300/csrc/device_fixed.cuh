@@ -300,12 +300,4 @@ __device__ __forceinline__ double fx_pack(const FxOp& q, int pack, int2* __restr
   return writes ? finish<MODE>(acc, o, xo, bo, q.y, q.y2, q.omega, dsum) : dsum;
 }
 
-// one block row per warp (see device_fixed.cu)
-constexpr int kFxSms = 152;
-inline bool warp_per_row(int mode, int np, int n, int64_t blocks) {
-  const int rpw = 32 / np, resident = kFxSms * kFxWarps * fx_ctas_per_sm(np);
-  if (fx_one(mode) || rpw < 2) return false;
-  return n <= resident || (blocks >= (int64_t)n * 3 * rpw && n <= 4 * resident);
-}
-
 }  // namespace fx

@@ -142,4 +142,73 @@ __device__ __forceinline__ T row_acc(int K, int i, const int* __restrict__ rowpt
   return acc;
 }
 
+// The same for a whole warp on one block row: floor(32 / n_p) groups of n_p lanes share its blocks
+// (group g takes blocks g, g + G, ...; two at a time in flight), lane i of a group row i; the sums
+// of the groups are added in a fixed order.  Valid in the lanes of group 0.  x aligned for VecLoad.
+template <typename T, int NP, bool COHERENT = false>
+__device__ __forceinline__ T split_row_acc(int K, const int* __restrict__ rowptr, const int* __restrict__ col,
+                                           const T* __restrict__ A, const T* __restrict__ x) {
+  constexpr int G = 32 / NP;
+  const int lane = threadIdx.x & 31;
+  const int sub = lane / NP, i = lane - sub * NP;
+  T acc = T(0);
+  if (sub < G) {
+    const int b1 = ldg(rowptr + K + 1);
+    int bb = ldg(rowptr + K) + sub;
+    for (; bb + G < b1; bb += 2 * G) {
+      T av[2][NP], xv[2][NP];
+#pragma unroll
+      for (int u = 0; u < 2; ++u) {
+        VecLoad<T, NP>::load(A + (size_t)(bb + u * G) * NP * NP + i * NP, av[u]);
+        VecLoad<T, NP, COHERENT>::load(x + (size_t)ldg(col + bb + u * G) * NP, xv[u]);
+      }
+#pragma unroll
+      for (int u = 0; u < 2; ++u)
+#pragma unroll
+        for (int j = 0; j < NP; ++j) acc = fma(av[u][j], xv[u][j], acc);
+    }
+    if (bb < b1) {
+      T av[NP], xv[NP];
+      VecLoad<T, NP>::load(A + (size_t)bb * NP * NP + i * NP, av);
+      VecLoad<T, NP, COHERENT>::load(x + (size_t)ldg(col + bb) * NP, xv);
+#pragma unroll
+      for (int j = 0; j < NP; ++j) acc = fma(av[j], xv[j], acc);
+    }
+  }
+#pragma unroll
+  for (int m = G; m > 1; m = (m + 1) / 2) {
+    const int h = (m + 1) / 2;
+    const T t = __shfl_down_sync(0xffffffffu, acc, h * NP);
+    if (sub + h < m) acc += t;
+  }
+  return acc;
+}
+
+// The sum over the children K of agglomerate Ag of (L_K^T r_K)_i, its children shared by the groups
+// of the warp in the same way; valid in the lanes of group 0.
+template <typename T, int NP, bool COHERENT = false>
+__device__ __forceinline__ T split_restrict(int Ag, const int* __restrict__ childptr, const T* __restrict__ L,
+                                            const T* __restrict__ r) {
+  constexpr int G = 32 / NP;
+  const int lane = threadIdx.x & 31;
+  const int sub = lane / NP, i = lane - sub * NP;
+  T acc = T(0);
+  if (sub < G) {
+    const int k1 = ldg(childptr + Ag + 1);
+    for (int K = ldg(childptr + Ag) + sub; K < k1; K += G) {
+      const T* LK = L + (size_t)K * NP * NP + i;
+      const T* rk = r + (size_t)K * NP;
+#pragma unroll
+      for (int j = 0; j < NP; ++j) acc = fma(ldg(LK + j * NP), COHERENT ? __ldcg(rk + j) : ldg(rk + j), acc);
+    }
+  }
+#pragma unroll
+  for (int m = G; m > 1; m = (m + 1) / 2) {
+    const int h = (m + 1) / 2;
+    const T t = __shfl_down_sync(0xffffffffu, acc, h * NP);
+    if (sub + h < m) acc += t;
+  }
+  return acc;
+}
+
 }  // namespace cdgk

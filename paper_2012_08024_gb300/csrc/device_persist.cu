@@ -216,6 +216,13 @@ __device__ __forceinline__ void fx_product(FxOp q, bool wpr, const double* x, co
   }
 }
 
+// one warp per row of level n
+template <typename F>
+__device__ __forceinline__ void for_rows(int n, F&& f) {
+  const int warps = (int)(gridDim.x * (blockDim.x >> 5));
+  for (int K = (int)(blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5)); K < n; K += warps) f(K);
+}
+
 // the phases in the precision of the cycle
 template <typename T, int NP>
 struct Phase {
@@ -224,13 +231,37 @@ struct Phase {
     ph_first<T, NP>(L.n, (const T*)L.Dinv, b, bh, x, w, write_x);
   }
   static __device__ void sweep(const PLevel& L, const T* x, const T* bh, T* y, T w) {
-    ph_bsr<T, NP, VEC, 3>(L.n, L.hrowptr, L.hcol, (const T*)L.Ahat, x, bh, y, w);
+    if (L.wprH)
+      for_rows(L.n, [&](int K) {
+        const T acc = cdgk::split_row_acc<T, NP, true>(K, L.hrowptr, L.hcol, (const T*)L.Ahat, x);
+        const int i = threadIdx.x & 31;
+        if (i >= NP) return;
+        const size_t row = (size_t)K * NP + i;
+        const T xv = __ldcg(x + row);
+        y[row] = xv + w * (__ldcg(bh + row) - xv - acc);
+      });
+    else
+      ph_bsr<T, NP, VEC, 3>(L.n, L.hrowptr, L.hcol, (const T*)L.Ahat, x, bh, y, w);
   }
   static __device__ void residual(const PLevel& L, const T* x, const T* b, T* r, T w) {
-    ph_bsr<T, NP, VEC, 1>(L.n, L.rowptr, L.col, (const T*)L.A, x, b, r, w);
+    if (L.wprA)
+      for_rows(L.n, [&](int K) {
+        const T acc = cdgk::split_row_acc<T, NP, true>(K, L.rowptr, L.col, (const T*)L.A, x);
+        const int i = threadIdx.x & 31;
+        if (i < NP) r[(size_t)K * NP + i] = __ldcg(b + (size_t)K * NP + i) - acc;
+      });
+    else
+      ph_bsr<T, NP, VEC, 1>(L.n, L.rowptr, L.col, (const T*)L.A, x, b, r, w);
   }
   static __device__ void restrict_to(const PLevel& L, const PLevel& C, const T* r, T* bc) {
-    ph_restrict<T, NP>(C.n, C.childptr, (const T*)L.L, r, bc);
+    if (L.wprR)
+      for_rows(C.n, [&](int Ag) {
+        const T acc = cdgk::split_restrict<T, NP, true>(Ag, C.childptr, (const T*)L.L, r);
+        const int i = threadIdx.x & 31;
+        if (i < NP) bc[(size_t)Ag * NP + i] = acc;
+      });
+    else
+      ph_restrict<T, NP>(C.n, C.childptr, (const T*)L.L, r, bc);
   }
   static __device__ void prolong(const PLevel& L, const T* xc, T* x, bool add) {
     ph_prolong<T, NP>(L.n, L.parent, (const T*)L.L, xc, x, add);
@@ -394,17 +425,17 @@ bool vcycle_persistent(DeviceState& D, const cdg_options& o, bool fp32, const vo
     Q.r = L.r;
     Q.b = L.b;
     Q.bh = L.bh;
+    Q.wprA = warp_per_row(L.np, L.n, L.nnzb);
+    Q.wprH = warp_per_row(L.np, L.n, L.hnnzb);
+    Q.wprR = l + 1 < D.nlev && warp_per_row(L.np, D.lev[l + 1].n, L.n);
     if (!fp32) {
       const bool last = l + 1 == D.nlev;
       Q.oA = operator_op(L, 1);
-      Q.wprA = fx::warp_per_row(1, L.np, L.n, L.nnzb);
       if (!last) {
         Q.oH = operator_op(L, 3);
-        Q.wprH = fx::warp_per_row(3, L.np, L.n, L.hnnzb);
         Q.oD = diagonal_op(L, 7, L.Dinv, L.eD);
         Q.oL = prolong_op(L);
         Q.oR = restrict_op(L, D.lev[l + 1]);
-        Q.wprR = fx::warp_per_row(8, L.np, Q.oR.n, Q.oR.blocks);
       }
     }
   }
