@@ -130,12 +130,13 @@ size_t layout(const cdg::Hierarchy& H, int precision, int nrhs, DeviceState* S, 
     // FP64 operator: level 0 always (outer CG); all levels in FP64 mode
     if (l == 0 || precision == 0) {
       L.A = c.take<double>(A.val.size());
+      // digits of A_0 of their own for the many-right-hand-side apply where A itself stays in FP64
+      if (!fixed && l == 0 && nrhs > 0) L.Adig = c.take<double>(A.val.size());
+      if (fixed || (l == 0 && nrhs > 0)) L.eA = c.take<int>((size_t)L.n * npl);
       if (fixed) {
-        L.eA = c.take<int>((size_t)L.n * npl);
         L.well = widest_row(A);
         L.ell = c.take<int>((size_t)L.n * L.well + 1);
       }
-      if (fixed && l == 0 && nrhs > 0) L.Aplain = c.take<double>(A.val.size());
     }
     if (!last) {
       const cdg::BSR& Sh = H.Ahat_t[l];
@@ -1727,13 +1728,16 @@ int dev_bind(cdg_handle* h, void* buf, int64_t bytes, void* stream) {
       }
     }
     if (l > 0) upload(L.childptr, H.childptr_t[l], s);
-    if (L.Aplain) upload(L.Aplain, A.val, s);
     if (L.chunk) {
       int rows = 0, parents = 0;
       upload(L.chunk, agglomerate_chunks(H.childptr_t[l + 1], chunk_target(L.np), &rows, &parents), s);
     }
     // every synchronous upload above finishes before the host vectors die
     cudaStreamSynchronize(s);
+  }
+  if (D.lev[0].Adig) {
+    upload(D.lev[0].Adig, H.A_t[0].val, s);
+    fx_encode(D.lev[0].np, D.lev[0].n, D.lev[0].rowptr, D.lev[0].Adig, D.lev[0].eA, s);
   }
   if (D.fixed) {   // FP64 blocks to digits (the restriction reads the next level's children ranges)
     bool ok = true;

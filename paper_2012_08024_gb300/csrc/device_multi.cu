@@ -20,6 +20,7 @@
 #include <string>
 #include <vector>
 
+#include "device_fixed.cuh"
 #include "device_kernels.cuh"
 #include "device_state.h"
 
@@ -50,199 +51,269 @@ __device__ __forceinline__ void stage_block(TC* s, const TA* a, int ne) {
   for (int t = threadIdx.x; t < ne; t += blockDim.x) s[t] = (TC)Conv<TA>::f(a[t]);
 }
 
-// y = A x (MODE 0), y = b - A x (1), y = x + omega (b - x - A x) (3; A = Ahat, b = D^-1 b).
-// A CTA of blockDim (TX, BR) owns BR consecutive block rows and one tile of
-// TX C right-hand sides: row group threadIdx.y stages its blocks in shared
-// memory and thread x applies them to columns x + c TX (c < C) of the tile.
-// Each block value read from shared memory feeds C fused multiply-adds, so
-// with C = 1 the shared-memory reads, not the FMA pipe, set the pace.  TX, BR
-// and C are the autotuned right-hand-side tile; every choice sums each column
-// in the same order, so they change the timing only.
-constexpr int kMrMaxBR = 4;
-
-template <typename TA, typename TV, typename TC, int NP, int MODE, int C>
-__device__ __forceinline__ void mr_bsr_body(int n, int R, const int* __restrict__ rowptr, const int* __restrict__ col,
-                                            const TA* __restrict__ A, const TV* __restrict__ x,
-                                            const TV* __restrict__ b, TV* __restrict__ y, TC omega) {
-  __shared__ __align__(16) TC as[kMrMaxBR][NP * NP];
-  const int BR = (int)blockDim.y, TX = (int)blockDim.x;
-  const int K0 = blockIdx.x * BR;
-  const int K = K0 + threadIdx.y;
-  const int r0 = blockIdx.y * TX * C + threadIdx.x;
-  int b0 = 0, nb = 0, nbmax = 0;
-  for (int q = 0; q < BR; ++q) {
-    if (K0 + q < n) {
-      const int a0 = rowptr[K0 + q], cnt = rowptr[K0 + q + 1] - a0;
-      nbmax = max(nbmax, cnt);
-      if (q == (int)threadIdx.y) {
-        b0 = a0;
-        nb = cnt;
-      }
-    }
+// V consecutive right-hand sides of one coefficient, aligned for one load
+template <int V>
+struct Cols;
+template <>
+struct Cols<1> {
+  static __device__ __forceinline__ void load(const float* p, float* v) { v[0] = *p; }
+  static __device__ __forceinline__ void store(float* p, const float* v) { *p = v[0]; }
+};
+template <>
+struct Cols<2> {
+  static __device__ __forceinline__ void load(const float* p, float* v) {
+    const float2 t = *reinterpret_cast<const float2*>(p);
+    v[0] = t.x, v[1] = t.y;
   }
-  TC acc[C][NP];
+  static __device__ __forceinline__ void store(float* p, const float* v) {
+    *reinterpret_cast<float2*>(p) = make_float2(v[0], v[1]);
+  }
+};
+template <>
+struct Cols<4> {
+  static __device__ __forceinline__ void load(const float* p, float* v) {
+    const float4 t = *reinterpret_cast<const float4*>(p);
+    v[0] = t.x, v[1] = t.y, v[2] = t.z, v[3] = t.w;
+  }
+  static __device__ __forceinline__ void store(float* p, const float* v) {
+    *reinterpret_cast<float4*>(p) = make_float4(v[0], v[1], v[2], v[3]);
+  }
+};
+
+// y = b - A x (MODE 1), y = x + omega (b - x - A x) (3; A = Ahat, b = D^-1 b), FP32; the restriction
+// y_A = sum_K L_K^T x_K over A's children (8: block t meets element t); and with one block per row (no
+// rowptr), x from element col[K] (nullptr: K): y += A x (4), y = A x and y2 = omega A x (6), y = A x (7).
+// A warp owns one block row and a tile of 32 V right-hand sides, V consecutive ones per lane (R is a
+// multiple of V: the vectors start on 256-byte boundaries and a coefficient's columns on multiples of
+// 4 R bytes); warps share nothing, so nothing waits on another warp.  It copies up to four of the row's
+// blocks at once into shared memory; PF starts the gather of the next block's x before the products of
+// this one.  What bounds the kernel is the latency of the x gathers: the CTA-wide form before it, two
+// barriers per block with the gathers behind them, moved its 638 MB (20,000 rows, n_p = 10, R = 256) in
+// 179 us, 0.52 of the copy rate.  V, PF and the warps per CTA are autotuned; every choice sums a
+// column in the same order.
+constexpr int kMrMaxBR = 4;
+constexpr int kMrStage = 4;
+
+template <int V, bool PF>
+constexpr int mr_min_ctas() { return V == 4 ? 3 : V == 2 ? (PF ? 5 : 6) : 8; }
+
+template <typename TA, int NP, int MODE, int V, bool PF>
+__global__ void __launch_bounds__(128, mr_min_ctas<V, PF>()) mr_row_kernel(int n, int R, const int* __restrict__ rowptr,
+                                                                        const int* __restrict__ col,
+                                                                        const TA* __restrict__ A,
+                                                                        const float* __restrict__ x,
+                                                                        const float* __restrict__ b,
+                                                                        float* y, float* __restrict__ y2,
+                                                                        float omega) {
+  constexpr bool ONE = MODE == 4 || MODE == 6 || MODE == 7;
+  constexpr int STAGE = ONE ? 1 : kMrStage;
+  constexpr int NN = NP * NP, SZ = (NN + 3) / 4 * 4;
+  __shared__ __align__(16) float as_s[kMrMaxBR][STAGE * SZ];
+  float* as = as_s[threadIdx.y];
+  const int K = blockIdx.x * blockDim.y + threadIdx.y;
+  const int lane = threadIdx.x;
+  const int r = (blockIdx.y * 32 + lane) * V;
+  if (K >= n) return;   // a whole warp
+  const bool on = r < R;
+  const int b0 = ONE ? K : rowptr[K], b1 = ONE ? K + 1 : rowptr[K + 1];
+  float acc[NP][V];
 #pragma unroll
-  for (int c = 0; c < C; ++c)
+  for (int i = 0; i < NP; ++i)
 #pragma unroll
-    for (int i = 0; i < NP; ++i) acc[c][i] = TC(0);
-  for (int t = 0; t < nbmax; ++t) {
-    __syncthreads();
-    if (t < nb) stage_block<TA, TC>(as[threadIdx.y], A + (size_t)(b0 + t) * NP * NP, NP * NP);
-    __syncthreads();
-    if (t < nb) {
-      const TV* xj = x + (size_t)col[b0 + t] * NP * R;
-      TC xv[C][NP];
+    for (int c = 0; c < V; ++c) acc[i][c] = 0.f;
+  auto gather = [&](int t, float (&v)[NP][V]) {
+    const int J = MODE == 8 || (ONE && !col) ? t : col[t];
+    const float* xj = x + (size_t)J * NP * R + r;
 #pragma unroll
-      for (int c = 0; c < C; ++c) {
-        const int r = r0 + c * TX;
+    for (int j = 0; j < NP; ++j) Cols<V>::load(xj + (size_t)j * R, v[j]);
+  };
+  auto products = [&](const float* a, const float (&v)[NP][V]) {
 #pragma unroll
-        for (int j = 0; j < NP; ++j) xv[c][j] = r < R ? (TC)xj[(size_t)j * R + r] : TC(0);
-      }
+    for (int q = 0; q < SZ / 4; ++q) {
+      const float4 a4 = reinterpret_cast<const float4*>(a)[q];
+      const float e[4] = {a4.x, a4.y, a4.z, a4.w};
 #pragma unroll
-      for (int i = 0; i < NP; ++i)
+      for (int k = 0; k < 4; ++k)
+        if (4 * q + k < NN) {
+          const int row = (4 * q + k) / NP, cl = (4 * q + k) % NP;   // entry of the stored block
+          const int i = MODE == 8 ? cl : row, j = MODE == 8 ? row : cl;
 #pragma unroll
-        for (int j = 0; j < NP; ++j) {
-          const TC a = as[threadIdx.y][i * NP + j];
-#pragma unroll
-          for (int c = 0; c < C; ++c) acc[c][i] = fma(a, xv[c][j], acc[c][i]);
+          for (int c = 0; c < V; ++c) acc[i][c] = fmaf(e[k], v[j][c], acc[i][c]);
         }
     }
+  };
+  for (int t0 = b0; t0 < b1; t0 += STAGE) {
+    const int cnt = min(STAGE, b1 - t0);
+    float xa[NP][V], xb[NP][V];
+    if (on) gather(t0, xa);
+    __syncwarp();
+    for (int u = lane; u < cnt * NN; u += 32) {
+      const int blk = SZ == NN ? 0 : u / NN;
+      as[blk * (SZ - NN) + u] = Conv<TA>::f(A[(size_t)t0 * NN + u]);
+    }
+    __syncwarp();
+    if (on) {
+#pragma unroll
+      for (int t = 0; t < STAGE; t += 2) {
+        if (t < cnt) {
+          if (PF && t + 1 < cnt) gather(t0 + t + 1, xb);
+          products(as + t * SZ, xa);
+        }
+        if (t + 1 < cnt) {
+          if (!PF) gather(t0 + t + 1, xb);
+          if (PF && t + 2 < cnt) gather(t0 + t + 2, xa);
+          products(as + (t + 1) * SZ, xb);
+          if (!PF && t + 2 < cnt) gather(t0 + t + 2, xa);
+        }
+      }
+    }
   }
-  if (K >= n) return;
+  if (!on) return;
+  const size_t base = (size_t)K * NP * R + r;
 #pragma unroll
-  for (int c = 0; c < C; ++c) {
-    const int r = r0 + c * TX;
-    if (r >= R) continue;
-    const size_t base = (size_t)K * NP * R + r;
+  for (int i = 0; i < NP; ++i) {
+    const size_t o = base + (size_t)i * R;
+    float v[V], xv[V];
+    if constexpr (MODE == 1 || MODE == 3) Cols<V>::load(b + o, v);
+    if constexpr (MODE == 3) Cols<V>::load(x + o, xv);
+    if constexpr (MODE == 4) Cols<V>::load(y + o, v);
 #pragma unroll
-    for (int i = 0; i < NP; ++i) {
-      const size_t o = base + (size_t)i * R;
-      if (MODE == 0) y[o] = (TV)acc[c][i];
-      else if (MODE == 1) y[o] = (TV)((TC)b[o] - acc[c][i]);
-      else y[o] = (TV)((TC)x[o] + omega * ((TC)b[o] - (TC)x[o] - acc[c][i]));
+    for (int c = 0; c < V; ++c) {
+      if constexpr (MODE == 1) v[c] -= acc[i][c];
+      else if constexpr (MODE == 3) v[c] = xv[c] + omega * (v[c] - xv[c] - acc[i][c]);
+      else if constexpr (MODE == 4) v[c] += acc[i][c];
+      else v[c] = acc[i][c];
+    }
+    Cols<V>::store(y + o, v);
+    if constexpr (MODE == 6) {
+#pragma unroll
+      for (int c = 0; c < V; ++c) v[c] *= omega;
+      Cols<V>::store(y2 + o, v);
     }
   }
 }
 
-template <typename TA, typename TV, typename TC, int NP, int MODE, int C>
-__global__ void mr_bsr_kernel(int n, int R, const int* __restrict__ rowptr, const int* __restrict__ col,
-                              const TA* __restrict__ A, const TV* __restrict__ x, const TV* __restrict__ b,
-                              TV* __restrict__ y, TC omega) {
-  mr_bsr_body<TA, TV, TC, NP, MODE, C>(n, R, rowptr, col, A, x, b, y, omega);
-}
-
-// The same for CTAs of at most 128 threads, with the registers held so that
-// eight such CTAs fit on an SM: the V-cycle sweeps wait on their x gathers,
-// and more resident warps hide more of that latency (an autotuner choice).
-template <typename TA, typename TV, typename TC, int NP, int MODE, int C>
-__global__ void __launch_bounds__(128, 8) mr_bsr_kernel_lb(int n, int R, const int* __restrict__ rowptr,
-                                                         const int* __restrict__ col, const TA* __restrict__ A,
-                                                         const TV* __restrict__ x, const TV* __restrict__ b,
-                                                         TV* __restrict__ y, TC omega) {
-  mr_bsr_body<TA, TV, TC, NP, MODE, C>(n, R, rowptr, col, A, x, b, y, omega);
-}
-
-// per element K: out = B_K in (block-diagonal apply); with WRITE_X also x = omega out
-template <typename TA, typename TV, int NP, bool WRITE_X>
-__global__ void mr_diag_kernel(int R, const TA* __restrict__ B, const TV* __restrict__ in, TV* __restrict__ out,
-                               TV* __restrict__ x, float omega) {
-  __shared__ float as[NP * NP];
-  const int K = blockIdx.x;
-  const int r = threadIdx.x;
-  stage_block<TA, float>(as, B + (size_t)K * NP * NP, NP * NP);
-  __syncthreads();
-  if (r >= R) return;
-  const size_t base = (size_t)K * NP * R + r;
-  float v[NP];
+// y = A_0 x in FP64 by integer digits (device_fixed.cu says why and how): a warp owns one block row and
+// 32 right-hand sides, one per lane.  A lane takes the largest exponent of its column over the row's
+// neighbours (a first pass, which also brings x into the caches), splits its values and keeps the n_p
+// sums in registers; the digits of a block are read from shared memory, each 16 bytes feeding eight
+// integer multiply-adds.  A_0 has at most dim + 2 blocks per row (compact stencil), so its rows need no
+// flush.  5,000 rows, n_p = 6, 40 columns: 82 us with FP64 multiply-adds (46 us at the FP64 rate).
+template <int NP>
+__global__ void __launch_bounds__(128, 4) mr_fx_kernel(int n, int R, const int* __restrict__ rowptr,
+                                                       const int* __restrict__ col, const int2* __restrict__ A,
+                                                       const int* __restrict__ EA, const double* __restrict__ x,
+                                                       double* __restrict__ y) {
+  constexpr int NN = NP * NP;
+  constexpr int CARRY = 31 / NP;   // blocks between carries
+  __shared__ __align__(16) int2 as_s[kMrMaxBR][(NN + 1) / 2 * 2];
+  int2* as = as_s[threadIdx.y];
+  const int K = blockIdx.x * blockDim.y + threadIdx.y;
+  const int lane = threadIdx.x;
+  const int r = blockIdx.y * 32 + lane;
+  if (K >= n) return;   // a whole warp
+  const bool on = r < R;
+  const int b0 = rowptr[K], b1 = rowptr[K + 1];
+  int em = 1;
+  if (on)
+    for (int t = b0; t < b1; ++t) {
+      const double* xj = x + (size_t)col[t] * NP * R + r;
 #pragma unroll
-  for (int j = 0; j < NP; ++j) v[j] = (float)in[base + (size_t)j * R];
+      for (int j = 0; j < NP; ++j) em = max(em, fx::biased_exponent(xj[(size_t)j * R]));
+    }
+  const bool special = em == 0x7FF;
+  fx::Acc acc[NP];
+  for (int t = b0, since = 0; t < b1; ++t) {
+    __syncwarp();
+    for (int u = lane; u < NN; u += 32) as[u] = A[(size_t)t * NN + u];
+    int2 xd[NP];
+    if (on && !special) {
+      const double* xj = x + (size_t)col[t] * NP * R + r;
 #pragma unroll
-  for (int i = 0; i < NP; ++i) {
-    float s = 0.f;
+      for (int j = 0; j < NP; ++j) xd[j] = fx::split_digits(xj[(size_t)j * R], em);
+    }
+    __syncwarp();
+    if (on && !special) {
+      if constexpr (NP % 2 == 0) {
+        const int4* a4 = reinterpret_cast<const int4*>(as);
 #pragma unroll
-    for (int j = 0; j < NP; ++j) s = fmaf(as[i * NP + j], v[j], s);
-    out[base + (size_t)i * R] = (TV)s;
-    if (WRITE_X) x[base + (size_t)i * R] = (TV)(omega * s);
-  }
-}
-
-// bc[A] = sum over children K of L_K^T r[K]
-template <typename TA, typename TV, int NP>
-__global__ void mr_restrict_kernel(int R, const int* __restrict__ childptr, const TA* __restrict__ L,
-                                   const TV* __restrict__ rf, TV* __restrict__ bc) {
-  __shared__ float ls[NP * NP];
-  const int Ag = blockIdx.x;
-  const int r = threadIdx.x;
-  float acc[NP];
+        for (int j = 0; j < NP; j += 2)
 #pragma unroll
-  for (int i = 0; i < NP; ++i) acc[i] = 0.f;
-  for (int K = childptr[Ag]; K < childptr[Ag + 1]; ++K) {
-    __syncthreads();
-    stage_block<TA, float>(ls, L + (size_t)K * NP * NP, NP * NP);
-    __syncthreads();
-    if (r < R) {
-      float v[NP];
+          for (int i = 0; i < NP; ++i) {
+            const int4 d = a4[(j >> 1) * NP + i];
+            fx::mac(acc[i], d.x, d.y, xd[j].x, xd[j].y);
+            fx::mac(acc[i], d.z, d.w, xd[j + 1].x, xd[j + 1].y);
+          }
+      } else {
 #pragma unroll
-      for (int j = 0; j < NP; ++j) v[j] = (float)rf[(size_t)K * NP * R + (size_t)j * R + r];
+        for (int j = 0; j < NP; ++j)
 #pragma unroll
-      for (int i = 0; i < NP; ++i)
+          for (int i = 0; i < NP; ++i) {
+            const int2 d = as[j * NP + i];
+            fx::mac(acc[i], d.x, d.y, xd[j].x, xd[j].y);
+          }
+      }
+      if (++since == CARRY || t + 1 == b1) {
+        since = 0;
 #pragma unroll
-        for (int j = 0; j < NP; ++j) acc[i] = fmaf(ls[j * NP + i], v[j], acc[i]);
+        for (int i = 0; i < NP; ++i) acc[i].carry();
+      }
     }
   }
-  if (r >= R) return;
-#pragma unroll
-  for (int i = 0; i < NP; ++i) bc[(size_t)Ag * NP * R + (size_t)i * R + r] = (TV)acc[i];
-}
-
-// x[K] (+)= L_K xc[parent K]
-template <typename TA, typename TV, int NP, bool ADD>
-__global__ void mr_prolong_kernel(int R, const int* __restrict__ parent, const TA* __restrict__ L,
-                                  const TV* __restrict__ xc, TV* __restrict__ x) {
-  __shared__ float ls[NP * NP];
-  const int K = blockIdx.x;
-  const int r = threadIdx.x;
-  stage_block<TA, float>(ls, L + (size_t)K * NP * NP, NP * NP);
-  __syncthreads();
-  if (r >= R) return;
-  const TV* xa = xc + (size_t)parent[K] * NP * R + r;
-  float v[NP];
-#pragma unroll
-  for (int j = 0; j < NP; ++j) v[j] = (float)xa[(size_t)j * R];
-  const size_t base = (size_t)K * NP * R + r;
+  if (!on) return;
 #pragma unroll
   for (int i = 0; i < NP; ++i) {
-    float s = 0.f;
-#pragma unroll
-    for (int j = 0; j < NP; ++j) s = fmaf(ls[i * NP + j], v[j], s);
-    x[base + (size_t)i * R] = ADD ? (TV)((float)x[base + (size_t)i * R] + s) : (TV)s;
+    const int ea = EA[(size_t)K * NP + i];
+    double v = fx::fx_value(acc[i].hh, acc[i].low(), ea + em - 1022);
+    if (special) {   // an infinity or NaN in the column: FP64 products
+      v = 0.0;
+      for (int t = b0; t < b1; ++t)
+        for (int j = 0; j < NP; ++j) {
+          const int2 d = A[(size_t)t * NN + fx::fx_pos(NP, i, j)];
+          v = fma(fx::scale2(__ll2double_rn(((long long)d.x << 30) + d.y), ea - 58),
+                  x[((size_t)col[t] * NP + j) * R + r], v);
+        }
+    }
+    if (ea == fx::kNotFinite) v = nan("");
+    y[((size_t)K * NP + i) * R + r] = v;
   }
 }
 
-// coarsest (one mesh): x[row][r] = sum_j Ainv[row][j] b[j][r], FP64 accumulation
-// in ascending j; a CTA owns CR consecutive rows and thread r one column, so
-// each b value is widened once per CR rows
+// coarsest (one mesh): x[row][r] = sum_j Ainv[row][j] b[j][r], FP64 accumulation.  A CTA owns
+// kCoarseRows rows and 32 columns; its eight warps share the j (each b value is widened once per
+// kCoarseRows rows) and their sums are added in order.  With one warp per 32 columns walking all j,
+// 228 unknowns x 40 columns kept 114 warps busy for 84 us (5 us at the FP64 rate).
 constexpr int kCoarseRows = 4;
+constexpr int kCoarseWarps = 8;
 
-template <typename TV, int CR>
-__global__ void mr_coarse_kernel(int nc, int R, const double* __restrict__ Ainv, const TV* __restrict__ b,
-                                 TV* __restrict__ x) {
-  const int row0 = blockIdx.x * CR;
-  const int r = threadIdx.x;
-  if (r >= R) return;
-  const int nr = min(CR, nc - row0);
-  double s[CR];
+template <typename TV>
+__global__ void __launch_bounds__(32 * kCoarseWarps) mr_coarse_kernel(int nc, int R, const double* __restrict__ Ainv,
+                                                                      const TV* __restrict__ b, TV* __restrict__ x) {
+  __shared__ double part[kCoarseWarps][kCoarseRows][32];
+  const int row0 = blockIdx.x * kCoarseRows;
+  const int lane = threadIdx.x, w = threadIdx.y;
+  const int r = blockIdx.y * 32 + lane;
+  const int j0 = nc * w / kCoarseWarps, j1 = nc * (w + 1) / kCoarseWarps;
+  double s[kCoarseRows];
 #pragma unroll
-  for (int q = 0; q < CR; ++q) s[q] = 0.0;
-  for (int j = 0; j < nc; ++j) {
-    const double bv = cvt<double>(b[(size_t)j * R + r]);
+  for (int q = 0; q < kCoarseRows; ++q) s[q] = 0.0;
+  if (r < R) {
+#pragma unroll 4
+    for (int j = j0; j < j1; ++j) {
+      const double bv = cvt<double>(b[(size_t)j * R + r]);
 #pragma unroll
-    for (int q = 0; q < CR; ++q)
-      if (q < nr) s[q] = fma(Ainv[(size_t)(row0 + q) * nc + j], bv, s[q]);
+      for (int q = 0; q < kCoarseRows; ++q)
+        s[q] = fma(Ainv[(size_t)min(row0 + q, nc - 1) * nc + j], bv, s[q]);
+    }
   }
 #pragma unroll
-  for (int q = 0; q < CR; ++q)
-    if (q < nr) x[(size_t)(row0 + q) * R + r] = cvt<TV>(s[q]);
+  for (int q = 0; q < kCoarseRows; ++q) part[w][q][lane] = s[q];
+  __syncthreads();
+  if (w < kCoarseRows && row0 + w < nc && r < R) {
+    double t = 0.0;
+    for (int k = 0; k < kCoarseWarps; ++k) t += part[k][w][lane];
+    x[(size_t)(row0 + w) * R + r] = cvt<TV>(t);
+  }
 }
 
 template <typename TI, typename TO>
@@ -251,11 +322,14 @@ __global__ void mr_convert_kernel(size_t n, const TI* __restrict__ a, TO* __rest
     b[i] = cvt<TO>(a[i]);
 }
 
-// The per-column vector kernels of the outer CG share one partition: CTA g of
-// G owns rows [nrows g / G, nrows (g + 1) / G) and thread r one column, so a
-// column's partial sums run over its rows in ascending order whichever kernel
-// forms them.  Rows go four at a time, all loads of a group before its
-// arithmetic, to keep enough loads in flight per thread.
+// The per-column vector kernels of the outer CG share one partition: row group g
+// of G = gridDim.x blockDim.y (threadIdx.y of its CTA) owns rows
+// [nrows g / G, nrows (g + 1) / G) and thread x one column, so a column's partial
+// sums run over its rows in ascending order whichever kernel forms them.  Rows go
+// four at a time, all loads of a group before its arithmetic, to keep enough
+// loads in flight per thread; with few columns a CTA holds several row groups
+// (40 columns, 30,000 rows, one group of 64 threads per CTA: update 42.6 us for
+// 62 MB).
 __device__ __forceinline__ void mr_rows(int nrows, int G, int g, int& lo, int& hi) {
   lo = (int)((long long)nrows * g / G);
   hi = (int)((long long)nrows * (g + 1) / G);
@@ -266,7 +340,7 @@ __device__ __forceinline__ void mr_rows(int nrows, int G, int g, int& lo, int& h
 template <typename TY>
 __global__ void mr_dot_kernel(int nrows, int R, int G, const double* __restrict__ x, const TY* __restrict__ y,
                               const TY* __restrict__ w, double* __restrict__ partial) {
-  const int g = blockIdx.x, r = threadIdx.x;
+  const int g = blockIdx.x * blockDim.y + threadIdx.y, r = threadIdx.x;
   if (r >= R) return;
   int lo, hi;
   mr_rows(nrows, G, g, lo, hi);
@@ -299,16 +373,42 @@ __global__ void mr_dot_kernel(int nrows, int R, int G, const double* __restrict_
   if (w) partial[(size_t)(G + g) * R + r] = s2;
 }
 
-// per column: sum the G partials in order and update that column's CG scalars
-// (same rules as the single-column finalize: which 0 PQ, 1 RR, 2 RZ, 3 BB, 4 initial RR)
-__global__ void mr_finalize_kernel(int R, int G, const double* __restrict__ partial, int which, int flexible,
-                                   double tol, double* __restrict__ scal) {
-  const int r = blockIdx.x * blockDim.x + threadIdx.x;
-  if (r >= R) return;
+// per column: the sum of the G partials, and that column's CG scalars (same rules as the
+// single-column finalize: which 0 PQ, 1 RR, 2 RZ, 3 BB, 4 initial RR).  A CTA owns four columns, 64
+// threads each share a column's partials, and their sums are added in a fixed order.  Few columns per
+// CTA, since an SM's FP64 pipe adds only two numbers per clock (32 columns per CTA: 11.8 us); one
+// thread per column walking its 304 partials took 54 us.
+constexpr int kFinCols = 4;
+constexpr int kFinThreads = 256;
+
+__global__ void __launch_bounds__(kFinThreads) mr_finalize_kernel(int R, int G, const double* __restrict__ partial,
+                                                                    int which, int flexible, double tol,
+                                                                    double* __restrict__ scal) {
+  __shared__ double part[2][kFinThreads / 32][kFinCols];
+  const int c = threadIdx.x % kFinCols, seg = threadIdx.x / kFinCols;
+  const int r = blockIdx.x * kFinCols + c;
+  const bool two = which == 2 && flexible;
+  double s = 0.0, s2 = 0.0;
+  if (r < R)
+    for (int g = seg; g < G; g += kFinThreads / kFinCols) {
+      s += partial[(size_t)g * R + r];
+      if (two) s2 += partial[(size_t)(G + g) * R + r];
+    }
+  for (int o = kFinCols; o < 32; o *= 2) {
+    s += __shfl_xor_sync(0xffffffffu, s, o);
+    if (two) s2 += __shfl_xor_sync(0xffffffffu, s2, o);
+  }
+  if ((threadIdx.x & 31) < kFinCols) {
+    part[0][threadIdx.x >> 5][c] = s;
+    part[1][threadIdx.x >> 5][c] = s2;
+  }
+  __syncthreads();
+  if (threadIdx.x >= kFinCols || r >= R) return;
   double tot = 0.0, tot2 = 0.0;
-  for (int g = 0; g < G; ++g) tot += partial[(size_t)g * R + r];
-  if (which == 2 && flexible)
-    for (int g = 0; g < G; ++g) tot2 += partial[(size_t)(G + g) * R + r];
+  for (int w = 0; w < kFinThreads / 32; ++w) {
+    tot += part[0][w][c];
+    tot2 += part[1][w][c];
+  }
   double* sc = scal + (size_t)r * S_COUNT;
   const bool done = sc[S_DONE] != 0.0;
   if (which == 0) {
@@ -344,7 +444,7 @@ __global__ void mr_finalize_kernel(int R, int G, const double* __restrict__ part
 __global__ void mr_update_kernel(int nrows, int R, int G, const double* __restrict__ scal,
                                  const double* __restrict__ p, const double* __restrict__ q, double* __restrict__ x,
                                  double* __restrict__ res, float* __restrict__ r32, double* __restrict__ partial) {
-  const int g = blockIdx.x, r = threadIdx.x;
+  const int g = blockIdx.x * blockDim.y + threadIdx.y, r = threadIdx.x;
   if (r >= R) return;
   int lo, hi;
   mr_rows(nrows, G, g, lo, hi);
@@ -391,7 +491,7 @@ __device__ __forceinline__ int biased_exp(double v) {
 
 __global__ void mr_p_kernel(int nrows, int R, int G, const double* __restrict__ scal, int first,
                             const float* __restrict__ z, double* __restrict__ p, int* __restrict__ maxb) {
-  const int g = blockIdx.x, r = threadIdx.x;
+  const int g = blockIdx.x * blockDim.y + threadIdx.y, r = threadIdx.x;
   if (r >= R) return;
   int lo, hi;
   mr_rows(nrows, G, g, lo, hi);
@@ -466,7 +566,8 @@ struct MRLevel {
 };
 
 struct MR {
-  int R = 0, G = 0;
+  int R = 0, G = 0;             // columns; row groups of the vector kernels
+  int rows_per_cta = 1;         // row groups per CTA
   bool bf16 = false;
   MRLevel lev[kMaxLev];
   double *x = nullptr, *r = nullptr, *p = nullptr, *q = nullptr, *bt = nullptr;
@@ -475,12 +576,12 @@ struct MR {
   float *r32 = nullptr, *z32 = nullptr, *z32old = nullptr;
   double* scal = nullptr;      // [R][S_COUNT]
   double* partial = nullptr;   // [2G][R]
-  // autotuned (right-hand-side tile width, block rows per CTA) of mr_bsr_kernel per
-  // level and mode (0 FP64 level-0 apply, 1 residual, 3 smoother sweep); 0 = not tuned
-  int tile[kMaxLev][4] = {};
+  // autotuned block rows (warps) per CTA, right-hand sides per lane and gather ahead (1) or not of
+  // mr_row_kernel and mr_fx_kernel per level and mode (0 FP64 level-0 apply, 1 residual, 3 smoother
+  // sweep); 0 = not tuned
   int rows[kMaxLev][4] = {};
-  int cols[kMaxLev][4] = {};   // right-hand sides per thread
-  int lb[kMaxLev][4] = {};     // 1: the register-capped instance (CTAs of at most 128 threads)
+  int cols[kMaxLev][4] = {};
+  int ahead[kMaxLev][4] = {};
   bool tuned = false;
   bool tc = false;             // smoother sweeps on tcgen05 (BF16 blocks)
   int* tc_err = nullptr;       // set by a tensor-core kernel whose wait timed out
@@ -496,15 +597,15 @@ struct MR {
 void mr_tuning(const MR& M, int level, int nlev, int32_t* out) {
   if (!M.tuned) return;
   if (level + 1 < nlev) {
-    out[4] = M.tile[level][3];
+    out[4] = 32;
     out[5] = M.rows[level][3];
-    out[6] = M.tile[level][1];
+    out[6] = 32;
     out[7] = M.rows[level][1];
     out[10] = M.cols[level][3];
     out[11] = M.cols[level][1];
   }
   if (level == 0) {
-    out[8] = M.tile[0][0];
+    out[8] = M.rows[0][0] ? 32 : 0;
     out[9] = M.rows[0][0];
     out[12] = M.cols[0][0];
   }
@@ -544,7 +645,8 @@ size_t mr_layout(const cdg::Hierarchy& H, int R, int precision, int tc_fp64, MR*
   MR tmp;
   MR& M = mr ? *mr : tmp;
   M.R = R;
-  M.G = 2 * 152;
+  M.rows_per_cta = std::max(1, 256 / (((R + 31) / 32) * 32));
+  M.G = (M.rows_per_cta > 2 ? 2 : 4) * 152 * M.rows_per_cta;
   M.bf16 = precision == 2;
   const size_t ts = M.bf16 ? sizeof(__nv_bfloat16) : sizeof(float);
   const int np = H.np;
@@ -643,76 +745,73 @@ namespace {
 
 inline unsigned threads_for(int R) { return (unsigned)(((R + 31) / 32) * 32); }
 
-// threads per CTA that a kernel's register use allows (cached per instance)
-template <typename Kern>
-int max_threads_of(Kern k) {
-  cudaFuncAttributes a{};
-  return cudaFuncGetAttributes(&a, (const void*)k) == cudaSuccess ? a.maxThreadsPerBlock : 256;
-}
-
-template <typename TA, typename TV, typename TC, int NP, int MODE, int C>
-void mr_bsr_launch_c(int tx, int br, bool lb, int n, int R, const int* rp, const int* cl, const TA* A, const TV* x,
-                     const TV* b, TV* y, TC omega, cudaStream_t s) {
-  if constexpr (C <= 2 && sizeof(TC) == 4) {   // the register-capped instance: FP32 arithmetic, <= 2 columns
-    if (lb && tx * std::min(std::max(br, 1), kMrMaxBR) <= 128) {
-      br = std::min(std::max(br, 1), kMrMaxBR);
-      const dim3 grid((unsigned)((n + br - 1) / br), (unsigned)((R + tx * C - 1) / (tx * C))),
-          block((unsigned)tx, (unsigned)br);
-      mr_bsr_kernel_lb<TA, TV, TC, NP, MODE, C><<<grid, block, 0, s>>>(n, R, rp, cl, A, x, b, y, omega);
-      count_launch();
-      return;
-    }
-  }
-  static const int mt = max_threads_of(mr_bsr_kernel<TA, TV, TC, NP, MODE, C>);
+// mr_row_kernel with v columns per lane (brought down to what divides R), br warps (block rows) per
+// CTA, pf: the next gather ahead
+template <typename TA, int NP, int MODE>
+void mr_row_launch(int br, int v, bool pf, int n, int R, const int* rp, const int* cl, const TA* A, const float* x,
+                   const float* b, float* y, float* y2, float omega, cudaStream_t s) {
   br = std::min(std::max(br, 1), kMrMaxBR);
-  // a CTA larger than the register file allows runs as fewer block rows, then
-  // narrower tiles: the same columns in the same order, so the same results
-  while (tx * br > mt && br > 1) br /= 2;
-  while (tx * br > mt && tx > 32) tx /= 2;
-  const dim3 grid((unsigned)((n + br - 1) / br), (unsigned)((R + tx * C - 1) / (tx * C))),
-      block((unsigned)tx, (unsigned)br);
-  mr_bsr_kernel<TA, TV, TC, NP, MODE, C><<<grid, block, 0, s>>>(n, R, rp, cl, A, x, b, y, omega);
+  while (R % v != 0) v /= 2;
+  const dim3 grid((unsigned)((n + br - 1) / br), (unsigned)((R + 32 * v - 1) / (32 * v))), block(32, (unsigned)br);
+  auto go = [&](auto kern) { kern<<<grid, block, 0, s>>>(n, R, rp, cl, A, x, b, y, y2, omega); };
+  if (v == 4) pf ? go(mr_row_kernel<TA, NP, MODE, 4, true>) : go(mr_row_kernel<TA, NP, MODE, 4, false>);
+  else if (v == 2) pf ? go(mr_row_kernel<TA, NP, MODE, 2, true>) : go(mr_row_kernel<TA, NP, MODE, 2, false>);
+  else pf ? go(mr_row_kernel<TA, NP, MODE, 1, true>) : go(mr_row_kernel<TA, NP, MODE, 1, false>);
   count_launch();
 }
 
-// mr_bsr_kernel with tx threads across the right-hand sides, rc columns per
-// thread (a tile of tx rc columns) and br block rows per CTA
-template <typename TA, typename TV, typename TC, int NP, int MODE>
-void mr_bsr_launch(int tx, int br, int rc, bool lb, int n, int R, const int* rp, const int* cl, const TA* A,
-                   const TV* x, const TV* b, TV* y, TC omega, cudaStream_t s) {
-  if (rc >= 4) mr_bsr_launch_c<TA, TV, TC, NP, MODE, 4>(tx, br, lb, n, R, rp, cl, A, x, b, y, omega, s);
-  else if (rc == 2) mr_bsr_launch_c<TA, TV, TC, NP, MODE, 2>(tx, br, lb, n, R, rp, cl, A, x, b, y, omega, s);
-  else mr_bsr_launch_c<TA, TV, TC, NP, MODE, 1>(tx, br, lb, n, R, rp, cl, A, x, b, y, omega, s);
-}
-
-inline int tile_of(const MR& M, int l, int mode) { return M.tile[l][mode] ? M.tile[l][mode] : (int)threads_for(M.R); }
-inline int rows_of(const MR& M, int l, int mode) { return M.rows[l][mode] ? M.rows[l][mode] : 1; }
-inline int cols_of(const MR& M, int l, int mode) { return M.cols[l][mode] ? M.cols[l][mode] : 1; }
-inline bool lb_of(const MR& M, int l, int mode) { return M.lb[l][mode] != 0; }
+// untuned: two columns per lane where R has them to give, the next gather ahead, four rows per CTA
+inline int rows_of(const MR& M, int l, int mode) { return M.rows[l][mode] ? M.rows[l][mode] : kMrMaxBR; }
+inline int cols_of(const MR& M, int l, int mode) { return M.cols[l][mode] ? M.cols[l][mode] : M.R >= 64 ? 2 : 1; }
+inline bool ahead_of(const MR& M, int l, int mode) { return M.cols[l][mode] ? M.ahead[l][mode] != 0 : true; }
 
 template <typename TA>
 bool mr_vcycle(DeviceState& D, MR& M, const cdg_options& o, const float* b0, float* z0, cudaStream_t s) {
   const int np = D.np, nlev = D.nlev, R = M.R;
-  const unsigned T = threads_for(R);
   const float w = (float)o.omega;
   auto bsr = [&](int mode, int l, const int* rp, const int* cl, const void* A, const float* x, const float* b,
                  float* y) -> bool {
     const int n = D.lev[l].n;
     if (mode == 3 && M.tc)
       return mr_tc_smooth(np, n, R, rp, cl, A, x, b, y, w, M.tc_err, D.wait_limit, s);
-    const int tx = tile_of(M, l, mode), br = rows_of(M, l, mode), rc = cols_of(M, l, mode);
-    const bool lb = lb_of(M, l, mode);
+    const int br = rows_of(M, l, mode), v = cols_of(M, l, mode);
+    const bool pf = ahead_of(M, l, mode);
     MR_NP_DISPATCH(np, {
-      if (mode == 1)
-        mr_bsr_launch<float, float, float, NP, 1>(tx, br, rc, lb, n, R, rp, cl, (const float*)A, x, b, y, w, s);
-      else
-        mr_bsr_launch<TA, float, float, NP, 3>(tx, br, rc, lb, n, R, rp, cl, (const TA*)A, x, b, y, w, s);
+      if (mode == 1) mr_row_launch<float, NP, 1>(br, v, pf, n, R, rp, cl, (const float*)A, x, b, y, nullptr, w, s);
+      else mr_row_launch<TA, NP, 3>(br, v, pf, n, R, rp, cl, (const TA*)A, x, b, y, nullptr, w, s);
     });
     return true;
   };
+  // the transfers and D^-1 b: untuned shapes
+  const int v1 = R >= 128 ? 4 : R >= 64 ? 2 : 1;
+  auto first = [&](int l, const float* b, float* bh, float* x) -> bool {
+    const float* Dinv = (const float*)M.lev[l].Dinv;
+    const int n = D.lev[l].n;
+    MR_NP_DISPATCH(np, {
+      if (x) mr_row_launch<float, NP, 6>(kMrMaxBR, v1, false, n, R, nullptr, nullptr, Dinv, b, nullptr, bh, x, w, s);
+      else mr_row_launch<float, NP, 7>(kMrMaxBR, v1, false, n, R, nullptr, nullptr, Dinv, b, nullptr, bh, nullptr, w, s);
+    });
+    return true;
+  };
+  auto restrict_to = [&](int l, const float* r, float* bc) -> bool {
+    const DevLevel& C = D.lev[l + 1];
+    MR_NP_DISPATCH(np, (mr_row_launch<TA, NP, 8>(kMrMaxBR, v1, true, C.n, R, C.childptr, nullptr,
+                                                 (const TA*)M.lev[l].L, r, nullptr, bc, nullptr, w, s)));
+    return true;
+  };
+  auto prolong = [&](int l, const float* xc, float* x, bool add) -> bool {
+    const DevLevel& F = D.lev[l];
+    const TA* L = (const TA*)M.lev[l].L;
+    MR_NP_DISPATCH(np, {
+      if (add) mr_row_launch<TA, NP, 4>(kMrMaxBR, v1, false, F.n, R, nullptr, F.parent, L, xc, nullptr, x, nullptr, w, s);
+      else mr_row_launch<TA, NP, 7>(kMrMaxBR, v1, false, F.n, R, nullptr, F.parent, L, xc, nullptr, x, nullptr, w, s);
+    });
+    return true;
+  };
+  const dim3 coarse_grid((unsigned)((D.nc + kCoarseRows - 1) / kCoarseRows), (unsigned)((R + 31) / 32));
+  const dim3 coarse_block(32, kCoarseWarps);
   if (nlev == 1) {
-    mr_coarse_kernel<float, kCoarseRows><<<(D.nc + kCoarseRows - 1) / kCoarseRows, T, 0, s>>>(D.nc, R, D.coarse_inv,
-                                                                                            b0, z0);
+    mr_coarse_kernel<float><<<coarse_grid, coarse_block, 0, s>>>(D.nc, R, D.coarse_inv, b0, z0);
     count_launch();
     return true;
   }
@@ -726,42 +825,28 @@ bool mr_vcycle(DeviceState& D, MR& M, const cdg_options& o, const float* b0, flo
     float* t = L.t;
     const float* b = bl[l];
     if (o.nu_pre >= 1) {
-      MR_NP_DISPATCH(np, mr_diag_kernel<float, float, NP, true><<<DL.n, T, 0, s>>>(R, (const float*)L.Dinv, b, L.bh, x, w));
-      count_launch();
+      if (!first(l, b, L.bh, x)) return false;
       for (int k = 1; k < o.nu_pre; ++k) {
         if (!bsr(3, l, DL.hrowptr, DL.hcol, L.Ahat, x, L.bh, t)) return false;
         std::swap(x, t);
       }
       if (!bsr(1, l, DL.rowptr, DL.col, L.A, x, b, L.r)) return false;
-      MR_NP_DISPATCH(np, mr_restrict_kernel<TA, float, NP><<<D.lev[l + 1].n, T, 0, s>>>(
-                             R, D.lev[l + 1].childptr, (const TA*)L.L, L.r, M.lev[l + 1].b));
-      count_launch();
+      if (!restrict_to(l, L.r, M.lev[l + 1].b)) return false;
       L.x = x;
       L.t = t;
     } else {
-      MR_NP_DISPATCH(np, mr_diag_kernel<float, float, NP, false><<<DL.n, T, 0, s>>>(R, (const float*)L.Dinv, b,
-                                                                                    L.bh, (float*)nullptr, w));
-      MR_NP_DISPATCH(np, mr_restrict_kernel<TA, float, NP><<<D.lev[l + 1].n, T, 0, s>>>(
-                             R, D.lev[l + 1].childptr, (const TA*)L.L, b, M.lev[l + 1].b));
-      count_launch(2);
+      if (!first(l, b, L.bh, nullptr) || !restrict_to(l, b, M.lev[l + 1].b)) return false;
     }
   }
-  mr_coarse_kernel<float, kCoarseRows><<<(D.nc + kCoarseRows - 1) / kCoarseRows, T, 0, s>>>(
-      D.nc, R, D.coarse_inv, M.lev[nlev - 1].b, M.lev[nlev - 1].x);
+  mr_coarse_kernel<float><<<coarse_grid, coarse_block, 0, s>>>(D.nc, R, D.coarse_inv, M.lev[nlev - 1].b,
+                                                               M.lev[nlev - 1].x);
   count_launch();
   for (int l = nlev - 2; l >= 0; --l) {
     MRLevel& L = M.lev[l];
     const DevLevel& DL = D.lev[l];
     float* x = L.x;
     float* t = L.t;
-    if (o.nu_pre >= 1) {
-      MR_NP_DISPATCH(np, mr_prolong_kernel<TA, float, NP, true><<<DL.n, T, 0, s>>>(R, DL.parent, (const TA*)L.L,
-                                                                                   M.lev[l + 1].x, x));
-    } else {
-      MR_NP_DISPATCH(np, mr_prolong_kernel<TA, float, NP, false><<<DL.n, T, 0, s>>>(R, DL.parent, (const TA*)L.L,
-                                                                                    M.lev[l + 1].x, x));
-    }
-    count_launch();
+    if (!prolong(l, M.lev[l + 1].x, x, o.nu_pre >= 1)) return false;
     for (int k = 0; k < o.nu_post; ++k) {
       float* out = (l == 0 && k + 1 == o.nu_post) ? z0 : t;
       if (!bsr(3, l, DL.hrowptr, DL.hcol, L.Ahat, x, L.bh, out)) return false;
@@ -778,71 +863,57 @@ bool mr_vcycle(DeviceState& D, MR& M, const cdg_options& o, const float* b0, flo
   return true;
 }
 
-// A_0 as FP64 numbers
-inline const double* plain_A0(const DeviceState& D) { return D.fixed ? D.lev[0].Aplain : D.lev[0].A; }
-
 // maxb_ready: the column exponents of x are already in M.oz_maxb (mr_p_kernel
 // stores them for p); pq_groups (split apply only): the apply also leaves the
 // partial sums of x . y in M.partial, *pq_groups of them per column
 bool mr_apply64(DeviceState& D, MR& M, const double* x, double* y, cudaStream_t s, bool maxb_ready = false,
-                int* pq_groups = nullptr) {
+                int* pq_groups = nullptr, int rows = 0) {
   const DevLevel& L0 = D.lev[0];
   if (M.oz)
     return oz_apply(D.np, L0.n, M.R, L0.rowptr, L0.col, M.oz_img, M.oz_eA, M.oz_xs, M.oz_maxb, maxb_ready, x, y,
                     pq_groups ? M.partial : nullptr, pq_groups, M.tc_err, D.wait_limit, s);
-  const int tx = tile_of(M, 0, 0), br = rows_of(M, 0, 0), rc = cols_of(M, 0, 0);
-  MR_NP_DISPATCH(D.np, (mr_bsr_launch<double, double, double, NP, 0>(tx, br, rc, false, L0.n, M.R, L0.rowptr, L0.col,
-                                                                     plain_A0(D),
-                                                                     x, (const double*)nullptr, y, 0.0, s)));
+  const int br = rows ? rows : rows_of(M, 0, 0);
+  const dim3 grid((unsigned)((L0.n + br - 1) / br), (unsigned)((M.R + 31) / 32)), block(32, (unsigned)br);
+  const int2* A = reinterpret_cast<const int2*>(D.fixed ? L0.A : L0.Adig);
+  if (L0.n > 0 && (int64_t)(D.d + 2) * D.np > fx::kMaxTerms) return false;   // the sums of a row (compact stencil)
+  MR_NP_DISPATCH(D.np, mr_fx_kernel<NP><<<grid, block, 0, s>>>(L0.n, M.R, L0.rowptr, L0.col, A, L0.eA, x, y));
+  count_launch();
   return true;
 }
 
-// Autotuner of the multi-right-hand-side block-sparse kernel: for every level
-// and mode the solve launches, times the (tile width, block rows per CTA)
-// pairs with tile width in {32, ..., 1024} up to the padded R and at most 1024
-// threads per CTA, on the handle's operators and zero-filled work vectors, and
-// keeps the fastest.
+// Autotuner of the many-right-hand-side block kernels: for every level and mode the solve launches,
+// times the columns per lane (1, 2, 4 where they divide R and leave a lane work) x warps per CTA x
+// gather ahead or not, on the handle's operators and zero-filled work vectors, and keeps the fastest.
 template <typename TA>
 bool mr_autotune(DeviceState& D, MR& M, double omega, cudaStream_t s) {
   const int np = D.np, nlev = D.nlev, R = M.R;
-  const int tmax = (int)threads_for(R);
   cudaEvent_t e0 = nullptr, e1 = nullptr;
   if (cudaEventCreate(&e0) != cudaSuccess || cudaEventCreate(&e1) != cudaSuccess) return false;
+  const int padded = (R + 31) / 32 * 32;
   auto pick = [&](int l, int mode, auto&& launch_one) {
     float tbest = 3.0e38f;
-    for (int rc : {1, 2, 4}) {
-      for (int tx = 32; tx <= 1024; tx *= 2) {
-        if (tx * rc > tmax && tx != 32) break;
-        if (rc > 1 && tx * rc > tmax) break;   // a thread's extra columns would all be padding
-        for (int br : {1, 2, 4}) {
-          if (tx * br > 1024) continue;
-          // the register-capped instance exists for FP32 arithmetic, CTAs of <= 128 threads, rc <= 2
-          const bool lb_ok = mode != 0 && rc <= 2 && tx * br <= 128;
-          for (int lb = 0; lb <= (lb_ok ? 1 : 0); ++lb) {
-            const float t = time_calls(s, e0, e1, 2, [&] { launch_one(tx, br, rc, lb != 0); });
-            if (t < tbest) {
-              tbest = t;
-              M.tile[l][mode] = tx;
-              M.rows[l][mode] = br;
-              M.cols[l][mode] = rc;
-              M.lb[l][mode] = lb;
-            }
+    for (int v : {1, 2, 4}) {
+      if (mode == 0 && v > 1) break;
+      if (R % v != 0 || (v > 1 && 32 * v > padded)) continue;
+      for (int br : {1, 2, 4}) {
+        for (int pf = 0; pf <= (mode == 0 ? 0 : 1); ++pf) {
+          const float t = time_calls(s, e0, e1, 2, [&] { launch_one(br, v, pf != 0); });
+          if (t < tbest) {
+            tbest = t;
+            M.rows[l][mode] = br;
+            M.cols[l][mode] = v;
+            M.ahead[l][mode] = pf;
           }
         }
       }
     }
   };
   bool ok = true;
-  if (!M.oz) {   // the FP64 CUDA-core apply (the split apply has no variants)
+  if (!M.oz) {   // the FP64 apply on CUDA cores (the split apply has no variants)
     const DevLevel& L0 = D.lev[0];
     const size_t nv = (size_t)L0.n * np * R;
     cudaMemsetAsync(M.p, 0, nv * sizeof(double), s);
-    pick(0, 0, [&](int tx, int br, int rc, bool) {
-      MR_NP_DISPATCH_V(np, (mr_bsr_launch<double, double, double, NP, 0>(tx, br, rc, false, L0.n, R, L0.rowptr, L0.col,
-                                                                         plain_A0(D),
-                                                                         (const double*)M.p, (const double*)nullptr,
-                                                                         M.q, 0.0, s)));
-    });
+    pick(0, 0, [&](int br, int, bool) { mr_apply64(D, M, M.p, M.q, s, false, nullptr, br); });
   }
   const float w = (float)omega;
   for (int l = 0; l + 1 < nlev; ++l) {
@@ -850,15 +921,13 @@ bool mr_autotune(DeviceState& D, MR& M, double omega, cudaStream_t s) {
     MRLevel& L = M.lev[l];
     const size_t nv = (size_t)DL.n * np * R;
     for (float* v : {L.x, L.b, L.bh, L.t}) cudaMemsetAsync(v, 0, nv * sizeof(float), s);
-    pick(l, 1, [&](int tx, int br, int rc, bool lb) {
-      MR_NP_DISPATCH_V(np, (mr_bsr_launch<float, float, float, NP, 1>(tx, br, rc, lb, DL.n, R, DL.rowptr, DL.col,
-                                                                      (const float*)L.A, (const float*)L.x,
-                                                                      (const float*)L.b, L.t, w, s)));
+    pick(l, 1, [&](int br, int v, bool pf) {
+      MR_NP_DISPATCH_V(np, (mr_row_launch<float, NP, 1>(br, v, pf, DL.n, R, DL.rowptr, DL.col, (const float*)L.A,
+                                                        (const float*)L.x, (const float*)L.b, L.t, nullptr, w, s)));
     });
-    pick(l, 3, [&](int tx, int br, int rc, bool lb) {
-      MR_NP_DISPATCH_V(np, (mr_bsr_launch<TA, float, float, NP, 3>(tx, br, rc, lb, DL.n, R, DL.hrowptr, DL.hcol,
-                                                                   (const TA*)L.Ahat, (const float*)L.x,
-                                                                   (const float*)L.bh, L.t, w, s)));
+    pick(l, 3, [&](int br, int v, bool pf) {
+      MR_NP_DISPATCH_V(np, (mr_row_launch<TA, NP, 3>(br, v, pf, DL.n, R, DL.hrowptr, DL.hcol, (const TA*)L.Ahat,
+                                                     (const float*)L.x, (const float*)L.bh, L.t, nullptr, w, s)));
     });
   }
   ok = cudaStreamSynchronize(s) == cudaSuccess && cudaGetLastError() == cudaSuccess;
@@ -870,16 +939,16 @@ bool mr_autotune(DeviceState& D, MR& M, double omega, cudaStream_t s) {
 
 // sums G partials per column (G = M.G unless given) into the CG scalars
 void mr_finalize(MR& M, int which, bool flexible, double tol, cudaStream_t s, int G = 0) {
-  mr_finalize_kernel<<<(M.R + 127) / 128, 128, 0, s>>>(M.R, G > 0 ? G : M.G, M.partial, which, flexible ? 1 : 0, tol,
-                                                         M.scal);
+  mr_finalize_kernel<<<(M.R + kFinCols - 1) / kFinCols, kFinThreads, 0, s>>>(M.R, G > 0 ? G : M.G, M.partial, which,
+                                                                           flexible ? 1 : 0, tol, M.scal);
   count_launch();
 }
 
 template <typename TY>
 void mr_dot(DeviceState& D, MR& M, const double* x, const TY* y, const TY* w, int which, double tol, cudaStream_t s) {
   const int nrows = (int)(D.ne * D.np);
-  const unsigned T = threads_for(M.R);
-  mr_dot_kernel<TY><<<M.G, T, 0, s>>>(nrows, M.R, M.G, x, y, w, M.partial);
+  const dim3 T(threads_for(M.R), (unsigned)M.rows_per_cta);
+  mr_dot_kernel<TY><<<M.G / M.rows_per_cta, T, 0, s>>>(nrows, M.R, M.G, x, y, w, M.partial);
   mr_finalize(M, which, w != nullptr, tol, s);
 }
 
@@ -907,6 +976,11 @@ int dev_solve_multi(cdg_handle* h, const double* f_q, double* u, double* res_his
   const size_t nv = (size_t)D.ne * D.np * R;
   const size_t nrows = (size_t)D.ne * D.np;
   const unsigned T = threads_for(R);
+  const dim3 Tv(T, (unsigned)M.rows_per_cta);   // vector kernels
+  const unsigned Gv = (unsigned)(M.G / M.rows_per_cta);
+  // the update (four reads, three writes) runs two CTAs per SM: 256 columns of 200,000 rows 456 us, with
+  // the four of the dots 496 us (the dots 162 against 202 us, the p update 147 against 198 us)
+  const int Gu = 2 * 152 * M.rows_per_cta;
   const unsigned gv = 4 * 152;
   bool ok = true;
   if (o.autotune && !M.tuned) {
@@ -958,7 +1032,7 @@ int dev_solve_multi(cdg_handle* h, const double* f_q, double* u, double* res_his
     ok = precond();
     mr_dot<float>(D, M, M.r, M.z32, nullptr, 2, o.tol, s);
     if (M.oz) cudaMemsetAsync(M.oz_maxb, 0, sizeof(int) * R, s);
-    mr_p_kernel<<<M.G, T, 0, s>>>((int)nrows, R, M.G, M.scal, 1, M.z32, M.p, M.oz ? M.oz_maxb : nullptr);
+    mr_p_kernel<<<Gv, Tv, 0, s>>>((int)nrows, R, M.G, M.scal, 1, M.z32, M.p, M.oz ? M.oz_maxb : nullptr);
     count_launch();
     while (ok) {
       if (it >= o.maxit) {
@@ -973,9 +1047,9 @@ int dev_solve_multi(cdg_handle* h, const double* f_q, double* u, double* res_his
         ok = mr_apply64(D, M, M.p, M.q, s);
         mr_dot<double>(D, M, M.p, M.q, nullptr, 0, o.tol, s);
       }
-      mr_update_kernel<<<M.G, T, 0, s>>>((int)nrows, R, M.G, M.scal, M.p, M.q, M.x, M.r, M.r32, M.partial);
+      mr_update_kernel<<<2 * 152, Tv, 0, s>>>((int)nrows, R, Gu, M.scal, M.p, M.q, M.x, M.r, M.r32, M.partial);
       count_launch();
-      mr_finalize(M, 1, false, o.tol, s);
+      mr_finalize(M, 1, false, o.tol, s, Gu);
       cudaMemcpyAsync(hs.data(), M.scal, sizeof(double) * hs.size(), cudaMemcpyDeviceToHost, s);
       int tc_err_it = 0;
       if (M.tc || M.oz) cudaMemcpyAsync(&tc_err_it, M.tc_err, sizeof(int), cudaMemcpyDeviceToHost, s);
@@ -1005,7 +1079,7 @@ int dev_solve_multi(cdg_handle* h, const double* f_q, double* u, double* res_his
       ok = precond();
       mr_dot<float>(D, M, M.r, M.z32, M.z32old, 2, o.tol, s);
       if (M.oz) cudaMemsetAsync(M.oz_maxb, 0, sizeof(int) * R, s);
-      mr_p_kernel<<<M.G, T, 0, s>>>((int)nrows, R, M.G, M.scal, 0, M.z32, M.p, M.oz ? M.oz_maxb : nullptr);
+      mr_p_kernel<<<Gv, Tv, 0, s>>>((int)nrows, R, M.G, M.scal, 0, M.z32, M.p, M.oz ? M.oz_maxb : nullptr);
       count_launch();
     }
   }

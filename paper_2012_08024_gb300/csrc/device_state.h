@@ -34,7 +34,7 @@ struct DevLevel {
   double *Lx = nullptr, *Rx = nullptr;
   int *ell = nullptr, *hell = nullptr;   // columns of A and Ahat as [n][width], -1 behind a row's last
   int well = 0, whell = 0;
-  double* Aplain = nullptr;  // level 0: A in FP64 for the many-right-hand-side apply
+  double* Adig = nullptr;    // level 0: A in digits beside an FP64 A (nrhs handles)
   int* parent = nullptr;
   int* childptr = nullptr;   // children range of each element of this level (l >= 1)
   // chunks of whole agglomerates of level l+1 for the fused residual + restriction
