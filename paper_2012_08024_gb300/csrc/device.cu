@@ -239,7 +239,7 @@ size_t layout(const cdg::Hierarchy& H, int precision, int nrhs, DeviceState* S, 
   }
   if (nrhs > 0) {
     if (S && !S->mr) S->mr = mr_new();
-    c.off = mr_layout(H, nrhs, mr_precision, tc_fp64, S ? S->mr : nullptr, base, c.off);
+    c.off = mr_layout(H, nrhs, mr_precision, tc_fp64, maxit, S ? S->mr : nullptr, base, c.off);
   }
   return (c.off + 255) & ~size_t(255);
 }
@@ -1886,6 +1886,7 @@ int dev_set_wait_limit(cdg_handle* h, int limit) {
     if (D.gsolve) cudaGraphExecDestroy(D.gsolve);
     D.g1 = D.g2 = D.gsolve = nullptr;
     gmres_release(D);
+    mr_drop_graph(D.mr);
   }
   D.wait_limit = v;
   return CDG_OK;

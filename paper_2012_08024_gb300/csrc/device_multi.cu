@@ -335,42 +335,36 @@ __device__ __forceinline__ void mr_rows(int nrows, int G, int g, int& lo, int& h
   hi = (int)((long long)nrows * (g + 1) / G);
 }
 
-// per-column partial dots over a chunk of rows: partial[g][r] = sum x y (and
-// partial[G + g][r] = sum x w); Y is FP64 or FP32 (a V-cycle output, widened exactly)
+// per-column partial dots over a chunk of rows: partial[g][r] = sum x y; Y is FP64 or FP32 (a
+// V-cycle output, widened exactly)
 template <typename TY>
 __global__ void mr_dot_kernel(int nrows, int R, int G, const double* __restrict__ x, const TY* __restrict__ y,
-                              const TY* __restrict__ w, double* __restrict__ partial) {
+                              double* __restrict__ partial) {
   const int g = blockIdx.x * blockDim.y + threadIdx.y, r = threadIdx.x;
   if (r >= R) return;
   int lo, hi;
   mr_rows(nrows, G, g, lo, hi);
-  double s = 0.0, s2 = 0.0;
+  double s = 0.0;
   int row = lo;
   for (; row + 4 <= hi; row += 4) {
     // all loads of the group first (raw words), conversions after: a
     // conversion's branch between two loads would keep them from overlapping
     double xv[4];
-    TY yv[4], wv[4];
+    TY yv[4];
 #pragma unroll
     for (int u = 0; u < 4; ++u) {
       const size_t o = (size_t)(row + u) * R + r;
       xv[u] = x[o];
       yv[u] = y[o];
-      wv[u] = w ? w[o] : TY(0);
     }
 #pragma unroll
-    for (int u = 0; u < 4; ++u) {
-      s = fma(xv[u], cvt<double>(yv[u]), s);
-      if (w) s2 = fma(xv[u], cvt<double>(wv[u]), s2);
-    }
+    for (int u = 0; u < 4; ++u) s = fma(xv[u], cvt<double>(yv[u]), s);
   }
   for (; row < hi; ++row) {
     const size_t o = (size_t)row * R + r;
     s = fma(x[o], cvt<double>(y[o]), s);
-    if (w) s2 = fma(x[o], cvt<double>(w[o]), s2);
   }
   partial[(size_t)g * R + r] = s;
-  if (w) partial[(size_t)(G + g) * R + r] = s2;
 }
 
 // per column: the sum of the G partials, and that column's CG scalars (same rules as the
@@ -382,12 +376,12 @@ constexpr int kFinCols = 4;
 constexpr int kFinThreads = 256;
 
 __global__ void __launch_bounds__(kFinThreads) mr_finalize_kernel(int R, int G, const double* __restrict__ partial,
-                                                                    int which, int flexible, double tol,
+                                                                    int which, double tol,
                                                                     double* __restrict__ scal) {
   __shared__ double part[2][kFinThreads / 32][kFinCols];
   const int c = threadIdx.x % kFinCols, seg = threadIdx.x / kFinCols;
   const int r = blockIdx.x * kFinCols + c;
-  const bool two = which == 2 && flexible;
+  const bool two = which == 1;   // r.r and the new r times the previous z
   double s = 0.0, s2 = 0.0;
   if (r < R)
     for (int g = seg; g < G; g += kFinThreads / kFinCols) {
@@ -421,6 +415,7 @@ __global__ void __launch_bounds__(kFinThreads) mr_finalize_kernel(int R, int G, 
   } else if (which == 1 || which == 4) {
     if (!done) {
       sc[S_RR] = tot;
+      sc[S_RZO] = tot2;
       if (which == 1) sc[S_IT] += 1.0;
       if (!isfinite(tot)) {
         sc[S_BREAK] = 1.0;
@@ -429,9 +424,8 @@ __global__ void __launch_bounds__(kFinThreads) mr_finalize_kernel(int R, int G, 
         sc[S_DONE] = 1.0;
       }
     }
-  } else if (which == 2) {
-    const double rz_old = sc[S_RZ];
-    sc[S_BETA] = done ? 0.0 : (flexible ? (tot - tot2) / rz_old : tot / rz_old);
+  } else if (which == 2) {   // flexible CG; unused by the first p
+    sc[S_BETA] = done ? 0.0 : (tot - sc[S_RZO]) / sc[S_RZ];
     sc[S_RZ] = tot;
   } else {
     sc[S_BB] = tot;
@@ -439,20 +433,23 @@ __global__ void __launch_bounds__(kFinThreads) mr_finalize_kernel(int R, int G, 
   }
 }
 
-// x += alpha_r p; r -= alpha_r q per column, with the FP32 copy of r that the
-// V-cycle reads and the partial r.r of the chunk (the sum mr_dot_kernel forms)
+// x += alpha_r p; r -= alpha_r q per column, with the FP32 copy of r that the V-cycle reads and the
+// chunk's partial sums of r.r and (G rows further) of r times z, the V-cycle's last output: the flexible
+// beta needs that product, and taken here the V-cycle may overwrite z
 __global__ void mr_update_kernel(int nrows, int R, int G, const double* __restrict__ scal,
                                  const double* __restrict__ p, const double* __restrict__ q, double* __restrict__ x,
-                                 double* __restrict__ res, float* __restrict__ r32, double* __restrict__ partial) {
+                                 double* __restrict__ res, float* __restrict__ r32, const float* __restrict__ z,
+                                 double* __restrict__ partial) {
   const int g = blockIdx.x * blockDim.y + threadIdx.y, r = threadIdx.x;
   if (r >= R) return;
   int lo, hi;
   mr_rows(nrows, G, g, lo, hi);
   const double a = scal[(size_t)r * S_COUNT + S_ALPHA];
-  double s = 0.0;
+  double s = 0.0, s2 = 0.0;
   int row = lo;
   for (; row + 4 <= hi; row += 4) {
     double pv[4], qv[4], xv[4], rv[4];
+    float zv[4];
 #pragma unroll
     for (int u = 0; u < 4; ++u) {
       const size_t o = (size_t)(row + u) * R + r;
@@ -460,6 +457,7 @@ __global__ void mr_update_kernel(int nrows, int R, int G, const double* __restri
       qv[u] = q[o];
       xv[u] = x[o];
       rv[u] = res[o];
+      zv[u] = z[o];
     }
 #pragma unroll
     for (int u = 0; u < 4; ++u) {
@@ -469,6 +467,7 @@ __global__ void mr_update_kernel(int nrows, int R, int G, const double* __restri
       res[o] = v;
       r32[o] = f64_to_f32(v);
       s = fma(v, v, s);
+      s2 = fma(v, f32_to_f64(zv[u]), s2);
     }
   }
   for (; row < hi; ++row) {
@@ -478,8 +477,10 @@ __global__ void mr_update_kernel(int nrows, int R, int G, const double* __restri
     res[o] = v;
     r32[o] = f64_to_f32(v);
     s = fma(v, v, s);
+    s2 = fma(v, f32_to_f64(z[o]), s2);
   }
   partial[(size_t)g * R + r] = s;
+  partial[(size_t)(G + g) * R + r] = s2;
 }
 
 // p = z + beta_r p per column (p = z on the first step); z is the V-cycle's FP32 output.
@@ -523,6 +524,38 @@ __global__ void mr_p_kernel(int nrows, int R, int G, const double* __restrict__ 
     em = max(em, biased_exp(v));
   }
   if (maxb) atomicMax(maxb + r, em);
+}
+
+// Single-graph solve: columns converged before the loop are closed, the counters start at zero
+__global__ void mr_open_kernel(int R, double* __restrict__ scal, int* __restrict__ it_dev, int* __restrict__ iters) {
+  for (int r = threadIdx.x; r < R; r += blockDim.x) {
+    scal[(size_t)r * S_COUNT + S_HDONE] = scal[(size_t)r * S_COUNT + S_DONE];
+    iters[r] = 0;
+  }
+  if (threadIdx.x == 0) *it_dev = 0;
+}
+
+// Single-graph solve, after the residual norms of an iteration: its entry in the history and the
+// iteration count of every open column (one closes in the iteration it converges or breaks down), and
+// whether to go on: a column is open, there are iterations left and no device wait has expired.
+__global__ void mr_check_kernel(cudaGraphConditionalHandle cond, int R, int maxit, double* __restrict__ scal,
+                                int* __restrict__ it_dev, double* __restrict__ hist, int* __restrict__ iters,
+                                const int* __restrict__ wait_err) {
+  const int it = *it_dev + 1;
+  int open = 0;
+  for (int r = threadIdx.x; r < R; r += blockDim.x) {
+    double* sc = scal + (size_t)r * S_COUNT;
+    if (sc[S_HDONE] != 0.0) continue;
+    hist[(size_t)r * (maxit + 1) + it] = sc[S_BB] > 0.0 ? sqrt(sc[S_RR] / sc[S_BB]) : 0.0;
+    iters[r] = it;
+    if (sc[S_DONE] != 0.0) sc[S_HDONE] = 1.0;
+    else open = 1;
+  }
+  open = __syncthreads_or(open);
+  if (threadIdx.x == 0) {
+    *it_dev = it;
+    cudaGraphSetConditional(cond, (open && it < maxit && *wait_err == 0) ? 1u : 0u);
+  }
 }
 
 // b[k][i][r] = sum_q w_q phi_i(x_q) f[r][K][q], K = perm0[k]  (f only; zero boundary data)
@@ -571,9 +604,7 @@ struct MR {
   bool bf16 = false;
   MRLevel lev[kMaxLev];
   double *x = nullptr, *r = nullptr, *p = nullptr, *q = nullptr, *bt = nullptr;
-  // FP32 V-cycle input r32 and output z32; z32old holds the previous output
-  // (flexible CG), the two swap roles every step
-  float *r32 = nullptr, *z32 = nullptr, *z32old = nullptr;
+  float *r32 = nullptr, *z32 = nullptr;   // FP32 V-cycle input and output
   double* scal = nullptr;      // [R][S_COUNT]
   double* partial = nullptr;   // [2G][R]
   // autotuned block rows (warps) per CTA, right-hand sides per lane and gather ahead (1) or not of
@@ -584,6 +615,13 @@ struct MR {
   int ahead[kMaxLev][4] = {};
   bool tuned = false;
   bool tc = false;             // smoother sweeps on tcgen05 (BF16 blocks)
+  // the CG loop as one graph (a conditional WHILE node around one iteration), with the iteration
+  // counter, the columns' counts and their residual histories [R][maxit + 1] on the device
+  cudaGraphExec_t gsolve = nullptr;
+  long long gsolve_kernels = 0;
+  bool gsolve_failed = false;
+  int *it_dev = nullptr, *iters_dev = nullptr;
+  double* hist_dev = nullptr;
   int* tc_err = nullptr;       // set by a tensor-core kernel whose wait timed out
   // FP64 level-0 apply on tcgen05 by exact splitting: B operand images of the
   // slices of A_0, row exponents, slices of x and column exponents (device_ozaki.cu)
@@ -637,10 +675,18 @@ void upload_conv(void* dst, const std::vector<double>& src, cudaStream_t s) {
 }  // namespace
 
 MR* mr_new() { return new MR(); }
-void mr_delete(MR* m) { delete m; }
+void mr_drop_graph(MR* m) {
+  if (m && m->gsolve) cudaGraphExecDestroy(m->gsolve);
+  if (m) m->gsolve = nullptr;
+}
+void mr_delete(MR* m) {
+  mr_drop_graph(m);
+  delete m;
+}
 
 // Carves the multi-column buffers after `off`; returns the new end offset.
-size_t mr_layout(const cdg::Hierarchy& H, int R, int precision, int tc_fp64, MR* mr, char* base, size_t off) {
+size_t mr_layout(const cdg::Hierarchy& H, int R, int precision, int tc_fp64, int maxit, MR* mr, char* base,
+                 size_t off) {
   MRCarver c{base, off};
   MR tmp;
   MR& M = mr ? *mr : tmp;
@@ -679,10 +725,12 @@ size_t mr_layout(const cdg::Hierarchy& H, int R, int precision, int tc_fp64, MR*
   M.bt = c.take<double>(nv);
   M.r32 = c.take<float>(nv);
   M.z32 = c.take<float>(nv);
-  M.z32old = c.take<float>(nv);
   M.scal = c.take<double>((size_t)R * S_COUNT);
   M.partial = c.take<double>((size_t)2 * M.G * R);
   M.tc_err = c.take<int>(1);
+  M.it_dev = c.take<int>(1);
+  M.iters_dev = c.take<int>(R);
+  M.hist_dev = c.take<double>((size_t)R * (maxit + 1));
   M.oz = tc_fp64 != 0 && oz_feasible(H.A_t[0], np);
   if (M.oz) {
     M.oz_img = c.take<char>(oz_image_bytes(H.A_t[0]));
@@ -938,18 +986,98 @@ bool mr_autotune(DeviceState& D, MR& M, double omega, cudaStream_t s) {
 }
 
 // sums G partials per column (G = M.G unless given) into the CG scalars
-void mr_finalize(MR& M, int which, bool flexible, double tol, cudaStream_t s, int G = 0) {
+void mr_finalize(MR& M, int which, double tol, cudaStream_t s, int G = 0) {
   mr_finalize_kernel<<<(M.R + kFinCols - 1) / kFinCols, kFinThreads, 0, s>>>(M.R, G > 0 ? G : M.G, M.partial, which,
-                                                                           flexible ? 1 : 0, tol, M.scal);
+                                                                           tol, M.scal);
   count_launch();
 }
 
 template <typename TY>
-void mr_dot(DeviceState& D, MR& M, const double* x, const TY* y, const TY* w, int which, double tol, cudaStream_t s) {
+void mr_dot(DeviceState& D, MR& M, const double* x, const TY* y, int which, double tol, cudaStream_t s) {
   const int nrows = (int)(D.ne * D.np);
   const dim3 T(threads_for(M.R), (unsigned)M.rows_per_cta);
-  mr_dot_kernel<TY><<<M.G / M.rows_per_cta, T, 0, s>>>(nrows, M.R, M.G, x, y, w, M.partial);
-  mr_finalize(M, which, w != nullptr, tol, s);
+  mr_dot_kernel<TY><<<M.G / M.rows_per_cta, T, 0, s>>>(nrows, M.R, M.G, x, y, M.partial);
+  count_launch();
+  mr_finalize(M, which, tol, s);
+}
+
+// the V-cycle maps r32 (FP32 copy of r, written by mr_update_kernel after the first step) to z32;
+// z = z32 widened exactly, so the FP64 steps read z32
+bool mr_precond(DeviceState& D, MR& M, const cdg_options& o, cudaStream_t s) {
+  return M.bf16 ? mr_vcycle<__nv_bfloat16>(D, M, o, M.r32, M.z32, s) : mr_vcycle<float>(D, M, o, M.r32, M.z32, s);
+}
+
+void mr_direction(DeviceState& D, MR& M, int first, cudaStream_t s) {
+  if (M.oz) cudaMemsetAsync(M.oz_maxb, 0, sizeof(int) * M.R, s);
+  mr_p_kernel<<<(unsigned)(M.G / M.rows_per_cta), dim3(threads_for(M.R), (unsigned)M.rows_per_cta), 0, s>>>(
+      (int)(D.ne * D.np), M.R, M.G, M.scal, first, M.z32, M.p, M.oz ? M.oz_maxb : nullptr);
+  count_launch();
+}
+
+// q = A p, alpha, x and r updates, r.r
+bool mr_part1(DeviceState& D, MR& M, const cdg_options& o, cudaStream_t s) {
+  bool ok;
+  if (M.oz) {   // p's column exponents come from mr_p_kernel, p . A p from the apply's epilogue
+    int gq = 0;
+    ok = mr_apply64(D, M, M.p, M.q, s, true, &gq);
+    mr_finalize(M, 0, o.tol, s, gq);
+  } else {
+    ok = mr_apply64(D, M, M.p, M.q, s);
+    mr_dot<double>(D, M, M.p, M.q, 0, o.tol, s);
+  }
+  // the update (five reads, three writes) runs two CTAs per SM: 256 columns of 200,000 rows 456 us, with
+  // the four of the dots 496 us (the dots 162 against 202 us, the p update 147 against 198 us)
+  const int Gu = 2 * 152 * M.rows_per_cta;
+  mr_update_kernel<<<2 * 152, dim3(threads_for(M.R), (unsigned)M.rows_per_cta), 0, s>>>(
+      (int)(D.ne * D.np), M.R, Gu, M.scal, M.p, M.q, M.x, M.r, M.r32, M.z32, M.partial);
+  count_launch();
+  mr_finalize(M, 1, o.tol, s, Gu);
+  return ok;
+}
+
+// z = V(r), beta, p
+bool mr_part2(DeviceState& D, MR& M, const cdg_options& o, cudaStream_t s) {
+  const bool ok = mr_precond(D, M, o, s);
+  mr_dot<float>(D, M, M.r, M.z32, 2, o.tol, s);
+  mr_direction(D, M, 0, s);
+  return ok;
+}
+
+// The CG loop as one executable graph, WHILE (cond) { part 1; check; part 2 }, as cdg_solve has it: the
+// condition starts at 1 on every launch, and the check clears it.  false: refused, the host drives the loop.
+bool mr_capture(DeviceState& D, MR& M, const cdg_options& o) {
+  cudaGraph_t g = nullptr;
+  if (cudaGraphCreate(&g, 0) != cudaSuccess) return false;
+  cudaGraphConditionalHandle cond;
+  cudaError_t e = cudaGraphConditionalHandleCreate(&cond, g, 1, cudaGraphCondAssignDefault);
+  cudaGraphNodeParams p = {};
+  p.type = cudaGraphNodeTypeConditional;
+  p.conditional.handle = cond;
+  p.conditional.type = cudaGraphCondTypeWhile;
+  p.conditional.size = 1;
+  cudaGraphNode_t node;
+  if (e == cudaSuccess) e = cudaGraphAddNode(&node, g, nullptr, nullptr, 0, &p);
+  if (e == cudaSuccess)
+    e = cudaStreamBeginCaptureToGraph(D.stream, p.conditional.phGraph_out[0], nullptr, nullptr, 0,
+                                      cudaStreamCaptureModeThreadLocal);
+  if (e != cudaSuccess) {
+    cudaGraphDestroy(g);
+    return false;
+  }
+  const long long before = launch_count();
+  bool ok = mr_part1(D, M, o, D.stream);
+  mr_check_kernel<<<1, 256, 0, D.stream>>>(cond, M.R, o.maxit, M.scal, M.it_dev, M.hist_dev, M.iters_dev, M.tc_err);
+  count_launch();
+  ok = mr_part2(D, M, o, D.stream) && ok;
+  cudaGraph_t captured = nullptr;
+  e = cudaStreamEndCapture(D.stream, &captured);
+  // captured launches run when the graph is launched: counted there, per iteration
+  M.gsolve_kernels = launch_count() - before;
+  count_launch(-M.gsolve_kernels);
+  if (ok && e == cudaSuccess) e = cudaGraphInstantiate(&M.gsolve, g, 0);
+  cudaGraphDestroy(g);
+  if (!ok || e != cudaSuccess) M.gsolve = nullptr;
+  return M.gsolve != nullptr;
 }
 
 }  // namespace
@@ -974,13 +1102,7 @@ int dev_solve_multi(cdg_handle* h, const double* f_q, double* u, double* res_his
   cudaEventRecord(D.ev_in, cs);
   cudaStreamWaitEvent(s, D.ev_in, 0);
   const size_t nv = (size_t)D.ne * D.np * R;
-  const size_t nrows = (size_t)D.ne * D.np;
   const unsigned T = threads_for(R);
-  const dim3 Tv(T, (unsigned)M.rows_per_cta);   // vector kernels
-  const unsigned Gv = (unsigned)(M.G / M.rows_per_cta);
-  // the update (four reads, three writes) runs two CTAs per SM: 256 columns of 200,000 rows 456 us, with
-  // the four of the dots 496 us (the dots 162 against 202 us, the p update 147 against 198 us)
-  const int Gu = 2 * 152 * M.rows_per_cta;
   const unsigned gv = 4 * 152;
   bool ok = true;
   if (o.autotune && !M.tuned) {
@@ -992,18 +1114,13 @@ int dev_solve_multi(cdg_handle* h, const double* f_q, double* u, double* res_his
   }
   cudaMemsetAsync(M.scal, 0, sizeof(double) * (size_t)R * S_COUNT, s);
   M.tc = M.bf16 && o.tensor_cores != 0 && D.np <= 16;
-  if (M.tc || M.oz) cudaMemsetAsync(M.tc_err, 0, sizeof(int), s);
+  cudaMemsetAsync(M.tc_err, 0, sizeof(int), s);
   MR_NP_DISPATCH(D.np, mr_rhs_kernel<NP><<<(unsigned)D.ne, T, 0, s>>>(R, D.nq, (int)D.ne, D.perm0, D.rhs_vol, f_q, M.bt));
   count_launch();
   cudaMemsetAsync(M.x, 0, sizeof(double) * nv, s);
   cudaMemcpyAsync(M.r, M.bt, sizeof(double) * nv, cudaMemcpyDeviceToDevice, s);
-  mr_dot<double>(D, M, M.bt, M.bt, nullptr, 3, o.tol, s);
-  mr_dot<double>(D, M, M.r, M.r, nullptr, 4, o.tol, s);
-  // the V-cycle maps r32 (FP32 copy of r, written by mr_update_kernel after the
-  // first step) to z32; z = z32 widened exactly, so the FP64 steps read z32
-  auto precond = [&]() -> bool {
-    return M.bf16 ? mr_vcycle<__nv_bfloat16>(D, M, o, M.r32, M.z32, s) : mr_vcycle<float>(D, M, o, M.r32, M.z32, s);
-  };
+  mr_dot<double>(D, M, M.bt, M.bt, 3, o.tol, s);
+  mr_dot<double>(D, M, M.r, M.r, 4, o.tol, s);
   std::vector<double> hs((size_t)R * S_COUNT);
   cudaMemcpyAsync(hs.data(), M.scal, sizeof(double) * hs.size(), cudaMemcpyDeviceToHost, s);
   cudaError_t e = cudaStreamSynchronize(s);
@@ -1026,33 +1143,62 @@ int dev_solve_multi(cdg_handle* h, const double* f_q, double* u, double* res_his
       ++ndone;
     }
   }
+  auto close = [&](int r) {   // a column whose scalars say that it is done
+    done[r] = 1;
+    ++ndone;
+    if (hs[(size_t)r * S_COUNT + S_BREAK] != 0.0) {
+      status = CDG_EBREAKDOWN;
+      h->err = "CG breakdown in column " + std::to_string(r);
+    }
+  };
   if (ndone < R) {
     mr_convert_kernel<double, float><<<gv, 256, 0, s>>>(nv, M.r, M.r32);
     count_launch();
-    ok = precond();
-    mr_dot<float>(D, M, M.r, M.z32, nullptr, 2, o.tol, s);
-    if (M.oz) cudaMemsetAsync(M.oz_maxb, 0, sizeof(int) * R, s);
-    mr_p_kernel<<<Gv, Tv, 0, s>>>((int)nrows, R, M.G, M.scal, 1, M.z32, M.p, M.oz ? M.oz_maxb : nullptr);
-    count_launch();
-    while (ok) {
+    ok = mr_precond(D, M, o, s);
+    mr_dot<float>(D, M, M.r, M.z32, 2, o.tol, s);
+    mr_direction(D, M, 1, s);
+    if (ok && o.solve_graph && o.maxit > 0 && !M.gsolve && !M.gsolve_failed && !mr_capture(D, M, o)) {
+      M.gsolve_failed = true;   // refused by this driver: keep the host-driven loop
+      cudaGetLastError();
+    }
+    const bool in_graph = ok && o.solve_graph && o.maxit > 0 && M.gsolve;
+    if (in_graph) {
+      mr_open_kernel<<<1, 256, 0, s>>>(R, M.scal, M.it_dev, M.iters_dev);
+      count_launch();
+      e = cudaGraphLaunch(M.gsolve, s);
+      if (e == cudaSuccess) e = cudaMemcpyAsync(&it, M.it_dev, sizeof(int), cudaMemcpyDeviceToHost, s);
+      if (e == cudaSuccess) e = cudaMemcpyAsync(iters, M.iters_dev, sizeof(int) * R, cudaMemcpyDeviceToHost, s);
+      if (e == cudaSuccess)
+        e = cudaMemcpyAsync(hs.data(), M.scal, sizeof(double) * hs.size(), cudaMemcpyDeviceToHost, s);
+      if (e == cudaSuccess) e = cudaStreamSynchronize(s);
+      std::vector<double> hh;   // the columns' entries 1 .. it
+      if (e == cudaSuccess && res_hist && it > 0) {
+        hh.resize((size_t)R * it);
+        e = cudaMemcpy2DAsync(hh.data(), sizeof(double) * it, M.hist_dev + 1, sizeof(double) * stride,
+                              sizeof(double) * it, R, cudaMemcpyDeviceToHost, s);
+      }
+      if (e == cudaSuccess) e = cudaStreamSynchronize(s);
+      if (e != cudaSuccess) {
+        h->err = std::string("solve_multi: ") + cudaGetErrorString(e);
+        return CDG_ECUDA;
+      }
+      count_launch(M.gsolve_kernels * it);
+      for (int r = 0; r < R; ++r) {
+        if (res_hist)
+          for (int k = 1; k <= iters[r]; ++k) res_hist[(size_t)r * stride + k] = hh[(size_t)r * it + k - 1];
+        if (!done[r] && hs[(size_t)r * S_COUNT + S_DONE] != 0.0) close(r);
+      }
+      if (ndone < R) status = CDG_ENOCONV;
+    }
+    while (ok && !in_graph) {
       if (it >= o.maxit) {
         status = CDG_ENOCONV;
         break;
       }
-      if (M.oz) {   // p's column exponents come from mr_p_kernel, p . A p from the apply's epilogue
-        int gq = 0;
-        ok = mr_apply64(D, M, M.p, M.q, s, true, &gq);
-        mr_finalize(M, 0, false, o.tol, s, gq);
-      } else {
-        ok = mr_apply64(D, M, M.p, M.q, s);
-        mr_dot<double>(D, M, M.p, M.q, nullptr, 0, o.tol, s);
-      }
-      mr_update_kernel<<<2 * 152, Tv, 0, s>>>((int)nrows, R, Gu, M.scal, M.p, M.q, M.x, M.r, M.r32, M.partial);
-      count_launch();
-      mr_finalize(M, 1, false, o.tol, s, Gu);
+      ok = mr_part1(D, M, o, s);
       cudaMemcpyAsync(hs.data(), M.scal, sizeof(double) * hs.size(), cudaMemcpyDeviceToHost, s);
       int tc_err_it = 0;
-      if (M.tc || M.oz) cudaMemcpyAsync(&tc_err_it, M.tc_err, sizeof(int), cudaMemcpyDeviceToHost, s);
+      cudaMemcpyAsync(&tc_err_it, M.tc_err, sizeof(int), cudaMemcpyDeviceToHost, s);
       e = cudaStreamSynchronize(s);
       if (e != cudaSuccess) {
         h->err = std::string("solve_multi: ") + cudaGetErrorString(e);
@@ -1064,23 +1210,10 @@ int dev_solve_multi(cdg_handle* h, const double* f_q, double* u, double* res_his
         if (done[r]) continue;
         iters[r] = it;
         if (res_hist) res_hist[(size_t)r * stride + it] = rel(r);
-        const double* sc = &hs[(size_t)r * S_COUNT];
-        if (sc[S_DONE] != 0.0) {
-          done[r] = 1;
-          ++ndone;
-          if (sc[S_BREAK] != 0.0) {
-            status = CDG_EBREAKDOWN;
-            h->err = "CG breakdown in column " + std::to_string(r);
-          }
-        }
+        if (hs[(size_t)r * S_COUNT + S_DONE] != 0.0) close(r);
       }
       if (ndone == R) break;
-      std::swap(M.z32, M.z32old);
-      ok = precond();
-      mr_dot<float>(D, M, M.r, M.z32, M.z32old, 2, o.tol, s);
-      if (M.oz) cudaMemsetAsync(M.oz_maxb, 0, sizeof(int) * R, s);
-      mr_p_kernel<<<Gv, Tv, 0, s>>>((int)nrows, R, M.G, M.scal, 0, M.z32, M.p, M.oz ? M.oz_maxb : nullptr);
-      count_launch();
+      ok = mr_part2(D, M, o, s);
     }
   }
   if (!ok) {
@@ -1090,7 +1223,7 @@ int dev_solve_multi(cdg_handle* h, const double* f_q, double* u, double* res_his
   mr_out_kernel<<<(unsigned)D.ne, T, 0, s>>>(R, D.np, D.perm0, M.x, (int)D.ne, u);
   count_launch();
   int tc_err = 0;
-  if (M.tc || M.oz) cudaMemcpyAsync(&tc_err, M.tc_err, sizeof(int), cudaMemcpyDeviceToHost, s);
+  cudaMemcpyAsync(&tc_err, M.tc_err, sizeof(int), cudaMemcpyDeviceToHost, s);
   e = cudaStreamSynchronize(s);
   if (e == cudaSuccess) e = cudaGetLastError();
   if (e != cudaSuccess) {

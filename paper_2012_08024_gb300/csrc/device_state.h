@@ -14,8 +14,9 @@ constexpr int kDotBlocks = 8 * 152;   // fixed grid of the vector kernels of bat
 constexpr int kDotBlocks1 = 2 * 152;  // the same for single-mesh handles (their dot partials: 2 CTAs per SM)
 
 // per-segment CG scalars (one row of S_COUNT doubles per mesh of the handle)
-// S_HDONE: the segment's residual history is closed (single-graph solve)
-enum Scal { S_RZ = 0, S_PQ, S_RR, S_BB, S_ALPHA, S_BETA, S_DONE, S_BREAK, S_IT, S_HDONE, S_FLAG = 15, S_COUNT = 16 };
+// S_HDONE: the segment's residual history is closed (single-graph solve); S_RZO: the new r times the
+// previous z (Polak-Ribiere)
+enum Scal { S_RZ = 0, S_PQ, S_RR, S_BB, S_ALPHA, S_BETA, S_DONE, S_BREAK, S_IT, S_HDONE, S_RZO, S_FLAG = 15, S_COUNT = 16 };
 
 struct DevLevel {
   int n = 0;
@@ -193,7 +194,9 @@ namespace cdg { struct Hierarchy; }
 MR* mr_new();
 void mr_delete(MR* m);
 // tc_fp64: the FP64 level-0 apply of the outer CG on tcgen05 by exact splitting (device_ozaki.cu)
-size_t mr_layout(const cdg::Hierarchy& H, int R, int precision, int tc_fp64, MR* mr, char* base, size_t off);
+size_t mr_layout(const cdg::Hierarchy& H, int R, int precision, int tc_fp64, int maxit, MR* mr, char* base,
+                 size_t off);
+void mr_drop_graph(MR* m);   // the captured solve (captured again by the next one)
 void mr_upload(const cdg::Hierarchy& H, MR& M, cudaStream_t s);
 int dev_apply_multi(cdg_handle* h, const double* x, double* y, void* stream);
 

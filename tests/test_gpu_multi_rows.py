@@ -60,3 +60,26 @@ def test_solve_columns(R, nu_pre):
         for r in (0, R // 2, R - 1):
             want = S1.solve(f[r].contiguous())[0]
             assert float((u[r] - want).norm() / want.norm()) <= 1e-9, r
+
+
+@pytest.mark.parametrize("prec,split", [("fp32", False), ("fp32", True), ("bf16", False)])
+@pytest.mark.parametrize("maxit", [500, 3, 0])
+def test_graph_and_host_driven_loops_agree(prec, split, maxit):
+    """The CG loop as one graph launch and as a host-driven loop: the same kernels in the same order."""
+    import torch
+    from paper_2012_08024_gb300 import Solver
+    mesh, R = jittered_square(13), 37
+    out = []
+    for graph in (True, False):
+        S = Solver(mesh, p=3, max_levels=3, precision=prec, nrhs=R, tc_fp64_apply=split, maxit=maxit, autotune=False,
+                   single_graph=graph).bind()
+        f = sine_combination_sources(S.quadrature_points()[0], R, mmax=4)
+        f[5] = 0.0   # a column that is converged before the loop
+        for _ in range(2):   # captured, then replayed
+            out.append(S.solve_multi(torch.tensor(f, device="cuda")))
+    u0, h0, i0, rc0 = out[0]
+    assert i0[5] == 0 and (maxit or not i0.any())
+    for u, h, i, rc in out[1:]:
+        assert rc == rc0 and np.array_equal(i, i0)
+        assert all(np.array_equal(a, b) for a, b in zip(h, h0))
+        assert np.array_equal(u.cpu().numpy(), u0.cpu().numpy())
