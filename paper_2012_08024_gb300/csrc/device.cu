@@ -94,6 +94,13 @@ std::vector<int> padded_columns(const cdg::BSR& A, int width) {
 // kernels that read them as FP64 numbers.
 inline bool digit_form(const cdg_options& o) { return o.fuse_transfers == 0; }
 
+// CTAs per segment of the vector kernels: kDotBlocks1 for one mesh (kDotBlocks over a batch), but no
+// more than leaves a thread four elements (one step of its loop): fewer partials to sum.
+int vector_ctas(int64_t ndofs, int nseg) {
+  const int64_t most = nseg == 1 ? kDotBlocks1 : std::max(1, kDotBlocks / nseg);
+  return (int)std::max<int64_t>(1, std::min(most, (ndofs / nseg + 4 * kThreads - 1) / (4 * kThreads)));
+}
+
 size_t layout(const cdg::Hierarchy& H, int precision, int nrhs, DeviceState* S, char* base, int mr_precision,
               int gmres_m, int maxit, int tc_fp64, bool fixed) {
   Carver c{base};
@@ -187,7 +194,7 @@ size_t layout(const cdg::Hierarchy& H, int precision, int nrhs, DeviceState* S, 
   }
   D.nc = (int)(H.lev.back().n * D.lev[nlev - 1].np);
   D.nseg = (int)H.seg_rows[0].size() - 1;
-  D.bps = D.nseg == 1 ? kDotBlocks1 : std::max(1, kDotBlocks / D.nseg);
+  D.bps = vector_ctas(D.ndofs, D.nseg);
   D.seg_dof = c.take<long long>(D.nseg + 1);
   D.crow_seg = c.take<int>(D.nc);
   D.crow_off = c.take<int>(D.nseg + 1);
@@ -212,7 +219,6 @@ size_t layout(const cdg::Hierarchy& H, int precision, int nrhs, DeviceState* S, 
   D.p = c.take<double>(vecbytes_elems);
   D.q = c.take<double>(vecbytes_elems);
   D.bt = c.take<double>(vecbytes_elems);
-  D.zold = c.take<double>(vecbytes_elems);
   if (precision) {
     D.r32 = c.take<float>(vecbytes_elems);
     D.z32 = c.take<float>(vecbytes_elems);
@@ -229,6 +235,7 @@ size_t layout(const cdg::Hierarchy& H, int precision, int nrhs, DeviceState* S, 
   D.hist_dev = c.take<double>((size_t)D.nseg * (maxit + 1));
   D.npartial = std::max<int>(std::max(kDotBlocks, D.nseg * D.bps), (int)((int64_t)ne * np / 64 + 2));
   D.partial = c.take<double>((size_t)D.npartial * 2);
+  D.partial_pq = c.take<double>(D.npartial);
   if (gmres_m > 0) {
     D.gm_m = gmres_m;
     D.gm_ld = (vecbytes_elems + 31) & ~size_t(31);   // every basis vector starts 256-byte aligned
@@ -561,16 +568,13 @@ __global__ void convert_kernel(size_t n, const TI* __restrict__ a, TO* __restric
     b[i] = cvt<TO>(a[i]);
 }
 
-__device__ __forceinline__ double block_sum(double v) {
-  __shared__ double red[kThreads / 32];
-  for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-  if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = v;
-  __syncthreads();
-  double s = 0.0;
-  if (threadIdx.x == 0)
-    for (int w = 0; w < kThreads / 32; ++w) s += red[w];
-  __syncthreads();
-  return s;
+constexpr int kWarps = kThreads / 32;
+using cdgk::cta_sum;
+using cdgk::lanes_sum;
+using cdgk::summing_warp;
+
+__device__ __forceinline__ bool is_summer() {   // the thread that holds cta_sum and writes it
+  return (int)threadIdx.x == summing_warp<kWarps>() * 32;
 }
 
 // Segmented vector kernels: block seg * bps + c handles chunk c of segment
@@ -584,125 +588,122 @@ __device__ __forceinline__ void seg_range(const long long* __restrict__ seg_dof,
   hi = a + len * (c + 1) / bps;
 }
 
-// partial[blk] = sum x.y over the block's chunk (and partial[npart + blk] = sum x.w)
+// partial[blk] = sum x.y over the block's chunk; Y is FP64, or FP32 (the V-cycle's output, widened exactly)
+template <typename TY>
 __global__ void __launch_bounds__(kThreads) dot_kernel(const long long* __restrict__ seg_dof, int bps,
-                                                       const double* __restrict__ x, const double* __restrict__ y,
-                                                       const double* __restrict__ w, double* __restrict__ partial,
-                                                       int npart) {
+                                                       const double* __restrict__ x, const TY* __restrict__ y,
+                                                       double* __restrict__ partial) {
   int seg;
   size_t lo, hi;
   seg_range(seg_dof, bps, seg, lo, hi);
   // four elements' loads in flight per step; the sums run over the thread's
   // elements in ascending order (the rounding does not depend on the unrolling)
-  double s = 0.0, s2 = 0.0;
+  double s = 0.0;
   const size_t bd = blockDim.x;
   size_t i = lo + threadIdx.x;
   for (; i + 3 * bd < hi; i += 4 * bd) {
-    double xv[4], yv[4], wv[4];
+    double xv[4];
+    TY yv[4];
 #pragma unroll
     for (int u = 0; u < 4; ++u) {
       xv[u] = x[i + u * bd];
       yv[u] = y[i + u * bd];
-      wv[u] = w ? w[i + u * bd] : 0.0;
     }
 #pragma unroll
-    for (int u = 0; u < 4; ++u) {
-      s = fma(xv[u], yv[u], s);
-      if (w) s2 = fma(xv[u], wv[u], s2);
-    }
+    for (int u = 0; u < 4; ++u) s = fma(xv[u], cvt<double>(yv[u]), s);
   }
-  for (; i < hi; i += bd) {
-    s = fma(x[i], y[i], s);
-    if (w) s2 = fma(x[i], w[i], s2);
-  }
-  s = block_sum(s);
-  if (w) s2 = block_sum(s2);
-  if (threadIdx.x == 0) {
-    partial[blockIdx.x] = s;
-    if (w) partial[npart + blockIdx.x] = s2;
-  }
+  for (; i < hi; i += bd) s = fma(x[i], cvt<double>(y[i]), s);
+  __shared__ double red[kThreads];
+  s = cta_sum<kWarps>(s, red);
+  if (is_summer()) partial[blockIdx.x] = s;
 }
 
-// One block per segment: sums its cnt partials in a fixed order and updates the
-// segment's CG scalars.  which: 0 PQ (alpha; breakdown if p.Ap <= 0), 1 RR
-// (iteration count, convergence ||r|| <= tol ||b||), 2 RZ (beta: Fletcher-Reeves,
-// or Polak-Ribiere with the second partial (r_new, z_old) when flexible),
-// 3 BB, 4 initial RR.  A segment marked done gets alpha = beta = 0.
-__global__ void finalize_kernel(const double* __restrict__ partial, int cnt, int npart, int which, int flexible,
-                                double tol, double* __restrict__ scal) {
-  __shared__ double red[kThreads / 32];
-  const int m = blockIdx.x;
-  const double* pm = partial + (size_t)m * cnt;
-  double s = 0.0, s2 = 0.0;
-  for (int i = threadIdx.x; i < cnt; i += blockDim.x) {
-    s += pm[i];
-    if (which == 2 && flexible) s2 += partial[npart + (size_t)m * cnt + i];
+// The sum of the n partials p, in every thread of the CTA and in an order that depends on n only: every
+// CTA that forms it gets the same bits.  Up to four warps add (see cta_sum).
+__device__ __forceinline__ double partials_sum(const double* __restrict__ p, int n) {
+  __shared__ double part[4];
+  const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int used = n > 64 ? 4 : 1;
+  __syncthreads();   // part may still be read from an earlier sum
+  if (w < used) {
+    double s = 0.0;
+    for (int i = threadIdx.x; i < n; i += 32 * used) s += p[i];
+    s = lanes_sum(s);
+    if (lane == 0) part[w] = s;
   }
-  for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
-  if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = s;
   __syncthreads();
-  double tot = 0.0;
-  if (threadIdx.x == 0)
-    for (int w = 0; w < kThreads / 32; ++w) tot += red[w];
-  __syncthreads();
-  for (int o = 16; o > 0; o >>= 1) s2 += __shfl_xor_sync(0xffffffffu, s2, o);
-  if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = s2;
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    double tot2 = 0.0;
-    for (int w = 0; w < kThreads / 32; ++w) tot2 += red[w];
-    double* sc = scal + (size_t)m * S_COUNT;
-    const bool done = sc[S_DONE] != 0.0;
-    if (which == 0) {
-      sc[S_PQ] = tot;
-      if (!done && !(tot > 0.0)) {
-        sc[S_BREAK] = 1.0;
-        sc[S_DONE] = 1.0;
-      }
-      sc[S_ALPHA] = sc[S_DONE] != 0.0 ? 0.0 : sc[S_RZ] / tot;
-    } else if (which == 1 || which == 4) {
-      if (!done) {
-        sc[S_RR] = tot;
-        if (which == 1) sc[S_IT] += 1.0;
-        if (!isfinite(tot)) {
-          sc[S_BREAK] = 1.0;
-          sc[S_DONE] = 1.0;
-        } else if (sqrt(tot) <= tol * sqrt(sc[S_BB])) {
-          sc[S_DONE] = 1.0;
-        }
-      }
-    } else if (which == 2) {
-      const double rz_old = sc[S_RZ];
-      sc[S_BETA] = done ? 0.0 : (flexible ? (tot - tot2) / rz_old : tot / rz_old);
-      sc[S_RZ] = tot;
-    } else {
-      sc[S_BB] = tot;
-      if (!(tot > 0.0)) sc[S_DONE] = 1.0;
+  return used == 1 ? part[0] : (part[0] + part[1]) + (part[2] + part[3]);
+}
+
+// The CG scalars without kernels of their own: a vector kernel that needs alpha or beta sums the
+// partials itself, in every CTA, and its CTA 0 of a segment records the result.  A separate one-CTA
+// kernel cost 4 us three times per iteration (a launch, and some forty dependent FP64 additions of 70
+// clocks each), of 97 us for the 32^2 (p = 2) solve.  What such a kernel writes is never what its other
+// CTAs read: r.z goes to S_RZN and moves on to S_RZ in the next update.
+
+// One CTA per segment: ||b||^2 (which 3) or the first ||r||^2 (4) from its cnt partials.
+__global__ void finalize_kernel(const double* __restrict__ partial, int cnt, int which, double tol,
+                                double* __restrict__ scal) {
+  const double tot = partials_sum(partial + (size_t)blockIdx.x * cnt, cnt);
+  if (threadIdx.x != 0) return;
+  double* sc = scal + (size_t)blockIdx.x * S_COUNT;
+  if (which == 3) {
+    sc[S_BB] = tot;
+    if (!(tot > 0.0)) sc[S_DONE] = 1.0;
+  } else if (sc[S_DONE] == 0.0) {
+    sc[S_RR] = tot;
+    if (!isfinite(tot)) {
+      sc[S_BREAK] = 1.0;
+      sc[S_DONE] = 1.0;
+    } else if (sqrt(tot) <= tol * sqrt(sc[S_BB])) {
+      sc[S_DONE] = 1.0;
     }
   }
 }
 
-// x += alpha p; r -= alpha q; partial of r.r (per segment chunk)
+// alpha = r.z / p.A p from the pq_cnt partials of the segment (0 in a segment that is done or breaks
+// down: p.A p <= 0), x += alpha p, r -= alpha q, and the partial of r.r.  With an FP32 V-cycle (FLEX)
+// also r32, the copy of r it reads, and (npart further) the partial of r times its last output z.
+template <bool FLEX>
 __global__ void __launch_bounds__(kThreads) cg_update_kernel(const long long* __restrict__ seg_dof, int bps,
-                                                             const double* __restrict__ scal,
-                                                             const double* __restrict__ p,
+                                                             const double* __restrict__ pq, int pq_cnt,
+                                                             double* __restrict__ scal, const double* __restrict__ p,
                                                              const double* __restrict__ q, double* __restrict__ x,
-                                                             double* __restrict__ r, double* __restrict__ partial) {
+                                                             double* __restrict__ r, float* __restrict__ r32,
+                                                             const float* __restrict__ z,
+                                                             double* __restrict__ partial, int npart) {
   int seg;
   size_t lo, hi;
   seg_range(seg_dof, bps, seg, lo, hi);
-  const double alpha = scal[(size_t)seg * S_COUNT + S_ALPHA];
-  double s = 0.0;
+  double* sc = scal + (size_t)seg * S_COUNT;
+  __shared__ double alpha_s;
+  const double tot = partials_sum(pq + (size_t)seg * pq_cnt, pq_cnt);
+  if (threadIdx.x == 0) {   // one thread divides: the FP64 pipe serves every warp that does
+    const double rz = sc[S_RZN];
+    const bool done = sc[S_DONE] != 0.0;
+    alpha_s = done || !(tot > 0.0) ? 0.0 : rz / tot;
+    if (blockIdx.x == (unsigned)(seg * bps)) {
+      sc[S_PQ] = tot;
+      sc[S_ALPHA] = alpha_s;
+      sc[S_RZ] = rz;
+      if (!done && !(tot > 0.0)) sc[S_BREAK] = 1.0;   // S_DONE follows in cg_check_kernel: CTAs still read it
+    }
+  }
+  __syncthreads();
+  const double alpha = alpha_s;
+  double s = 0.0, s2 = 0.0;
   const size_t bd = blockDim.x;
   size_t i = lo + threadIdx.x;
   for (; i + 3 * bd < hi; i += 4 * bd) {   // four elements' loads in flight, ascending sum
     double pv[4], qv[4], xv[4], rv[4];
+    float zv[4];
 #pragma unroll
     for (int u = 0; u < 4; ++u) {
       pv[u] = p[i + u * bd];
       qv[u] = q[i + u * bd];
       xv[u] = x[i + u * bd];
       rv[u] = r[i + u * bd];
+      if constexpr (FLEX) zv[u] = z[i + u * bd];
     }
 #pragma unroll
     for (int u = 0; u < 4; ++u) {
@@ -710,6 +711,10 @@ __global__ void __launch_bounds__(kThreads) cg_update_kernel(const long long* __
       const double ri = fma(-alpha, qv[u], rv[u]);
       r[i + u * bd] = ri;
       s = fma(ri, ri, s);
+      if constexpr (FLEX) {
+        r32[i + u * bd] = cvt<float>(ri);
+        s2 = fma(ri, cvt<double>(zv[u]), s2);
+      }
     }
   }
   for (; i < hi; i += bd) {
@@ -717,9 +722,18 @@ __global__ void __launch_bounds__(kThreads) cg_update_kernel(const long long* __
     const double ri = fma(-alpha, q[i], r[i]);
     r[i] = ri;
     s = fma(ri, ri, s);
+    if constexpr (FLEX) {
+      r32[i] = cvt<float>(ri);
+      s2 = fma(ri, cvt<double>(z[i]), s2);
+    }
   }
-  s = block_sum(s);
-  if (threadIdx.x == 0) partial[blockIdx.x] = s;
+  __shared__ double red[kThreads];
+  s = cta_sum<kWarps>(s, red);
+  if constexpr (FLEX) s2 = cta_sum<kWarps>(s2, red);
+  if (is_summer()) {
+    partial[blockIdx.x] = s;
+    if constexpr (FLEX) partial[npart + blockIdx.x] = s2;
+  }
 }
 
 // Single-graph solve: mark the segments converged before the loop as closed
@@ -727,53 +741,118 @@ __global__ void hist_init_kernel(int nseg, double* __restrict__ scal) {
   for (int m = threadIdx.x; m < nseg; m += blockDim.x) scal[(size_t)m * S_COUNT + S_HDONE] = scal[(size_t)m * S_COUNT + S_DONE];
 }
 
-// Single-graph solve, after G1 of iteration it: record ||r||/||b|| and the iteration count of every
-// segment still open (a segment closes in the iteration it converges or breaks down), and keep the
-// loop running while a segment is open and it < maxit.
-__global__ void cg_check_kernel(cudaGraphConditionalHandle cond, int nseg, int maxit, double* __restrict__ scal,
-                                int* __restrict__ it_dev, double* __restrict__ hist, int* __restrict__ iters,
-                                const int* __restrict__ wait_err) {
-  __shared__ int open;
-  if (threadIdx.x == 0) open = 0;
-  __syncthreads();
-  const int it = *it_dev + 1;
-  for (int m = threadIdx.x; m < nseg; m += blockDim.x) {
+// One CTA, after the update of an iteration: ||r||^2 of every segment from its bps partials (and r.z_old,
+// npart further, for the flexible beta), convergence ||r|| <= tol ||b||, breakdown.  In the single-graph
+// solve (in_graph) also ||r||/||b|| and the iteration count of every segment still open (a segment closes
+// in the iteration it converges or breaks down), and whether the loop goes on: a segment is open, there
+// are iterations left, and no device wait has expired (its output would not be a V-cycle).
+constexpr int kCheckThreads = 512;
+
+__global__ void __launch_bounds__(kCheckThreads) cg_check_kernel(cudaGraphConditionalHandle cond, int in_graph,
+                                                                 int nseg, int bps, const double* __restrict__ partial,
+                                                                 int npart, int flexible, double tol, int maxit,
+                                                                 double* __restrict__ scal, int* __restrict__ it_dev,
+                                                                 double* __restrict__ hist, int* __restrict__ iters,
+                                                                 const int* __restrict__ wait_err) {
+  const int it = in_graph ? *it_dev + 1 : 0;
+  int open = 0;
+  auto close = [&](int m, double rr, double rzo) {
     double* sc = scal + (size_t)m * S_COUNT;
-    if (sc[S_HDONE] != 0.0) continue;
+    if (sc[S_BREAK] != 0.0) sc[S_DONE] = 1.0;
+    sc[S_RZO] = rzo;
+    if (sc[S_DONE] == 0.0) {
+      sc[S_RR] = rr;
+      sc[S_IT] += 1.0;
+      if (!isfinite(rr)) {
+        sc[S_BREAK] = 1.0;
+        sc[S_DONE] = 1.0;
+      } else if (sqrt(rr) <= tol * sqrt(sc[S_BB])) {
+        sc[S_DONE] = 1.0;
+      }
+    }
+    if (!in_graph || sc[S_HDONE] != 0.0) return;
     hist[(size_t)m * (maxit + 1) + it] = sc[S_BB] > 0.0 ? sqrt(sc[S_RR] / sc[S_BB]) : 0.0;
     iters[m] = it;
     if (sc[S_DONE] != 0.0) sc[S_HDONE] = 1.0;
-    else atomicOr(&open, 1);
+    else open = 1;
+  };
+  if (nseg == 1) {
+    const double rr = partials_sum(partial, bps);
+    const double rzo = flexible ? partials_sum(partial + npart, bps) : 0.0;
+    if (threadIdx.x == 0) close(0, rr, rzo);
+  } else {
+    __shared__ double rr_s[kCheckThreads], rzo_s[kCheckThreads];
+    for (int m0 = 0; m0 < nseg; m0 += kCheckThreads) {
+      const int cnt = min(kCheckThreads, nseg - m0);
+      for (int m = threadIdx.x >> 5; m < cnt; m += kCheckThreads / 32) {   // a warp sums a segment
+        double rr = 0.0, rzo = 0.0;
+        for (int i = threadIdx.x & 31; i < bps; i += 32) {
+          rr += partial[(size_t)(m0 + m) * bps + i];
+          if (flexible) rzo += partial[npart + (size_t)(m0 + m) * bps + i];
+        }
+        rr = lanes_sum(rr);
+        if (flexible) rzo = lanes_sum(rzo);
+        if ((threadIdx.x & 31) == 0) {
+          rr_s[m] = rr;
+          rzo_s[m] = rzo;
+        }
+      }
+      __syncthreads();
+      if ((int)threadIdx.x < cnt) close(m0 + threadIdx.x, rr_s[threadIdx.x], rzo_s[threadIdx.x]);   // a thread closes it
+      __syncthreads();
+    }
   }
-  __syncthreads();
-  if (threadIdx.x == 0) {
+  open = __syncthreads_or(open);
+  if (in_graph && threadIdx.x == 0) {
     *it_dev = it;
-    // a device wait that expired (persistent V-cycle) ends the loop: its output is not a V-cycle
     cudaGraphSetConditional(cond, (open != 0 && it < maxit && *wait_err == 0) ? 1u : 0u);
   }
 }
 
-// p = z + beta p (first: p = z)
+// beta from the rz_cnt partials of r.z of the segment, p = z + beta p (first: p = z); z FP64, or FP32
+// (then the flexible, Polak-Ribiere beta).  A segment that is done gets beta = 0.
+template <typename TZ>
 __global__ void __launch_bounds__(kThreads) cg_p_kernel(const long long* __restrict__ seg_dof, int bps,
-                                                        const double* __restrict__ scal, int first,
-                                                        const double* __restrict__ z, double* __restrict__ p) {
+                                                        const double* __restrict__ rzp, int rz_cnt,
+                                                        double* __restrict__ scal, int first,
+                                                        const TZ* __restrict__ z, double* __restrict__ p) {
   int seg;
   size_t lo, hi;
   seg_range(seg_dof, bps, seg, lo, hi);
-  const double beta = first ? 0.0 : scal[(size_t)seg * S_COUNT + S_BETA];
+  double* sc = scal + (size_t)seg * S_COUNT;
+  const double tot = partials_sum(rzp + (size_t)seg * rz_cnt, rz_cnt);
+  __shared__ double beta_s;
+  if (threadIdx.x == 0) {
+    beta_s = first || sc[S_DONE] != 0.0 ? 0.0
+             : sizeof(TZ) == 4          ? (tot - sc[S_RZO]) / sc[S_RZ]
+                                        : tot / sc[S_RZ];
+    if (blockIdx.x == (unsigned)(seg * bps)) {
+      sc[S_BETA] = beta_s;
+      sc[S_RZN] = tot;
+    }
+  }
+  __syncthreads();
+  const double beta = beta_s;
   const size_t bd = blockDim.x;
   size_t i = lo + threadIdx.x;
   for (; i + 3 * bd < hi; i += 4 * bd) {
-    double zv[4], pv[4];
+    TZ zv[4];
+    double pv[4];
 #pragma unroll
     for (int u = 0; u < 4; ++u) {
       zv[u] = z[i + u * bd];
       pv[u] = first ? 0.0 : p[i + u * bd];
     }
 #pragma unroll
-    for (int u = 0; u < 4; ++u) p[i + u * bd] = first ? zv[u] : fma(beta, pv[u], zv[u]);
+    for (int u = 0; u < 4; ++u) {
+      const double zd = cvt<double>(zv[u]);
+      p[i + u * bd] = first ? zd : fma(beta, pv[u], zd);
+    }
   }
-  for (; i < hi; i += bd) p[i] = first ? z[i] : fma(beta, p[i], z[i]);
+  for (; i < hi; i += bd) {
+    const double zd = cvt<double>(z[i]);
+    p[i] = first ? zd : fma(beta, p[i], zd);
+  }
 }
 
 // b (tree order, or user order) from f at volume points and g_D / g_N at boundary points
@@ -1303,8 +1382,11 @@ void coarse_solve(DeviceState& D, const T* b, T* x, cudaStream_t s) {
 // the coarse level's last post-smoothing sweep carries the prolongation; the
 // separate kernels remain for degree steps of the p-multigrid front end, for
 // the coarsest level and for V(nu, 0).
+// dot (digit form, one mesh): the last sweep also leaves the per-CTA partials of z0 . b0 there, *dot_cnt
+// of them (0: it could not).
 template <typename T>
-bool vcycle(DeviceState& D, const cdg_options& o, const T* b0, T* z0, cudaStream_t s) {
+bool vcycle(DeviceState& D, const cdg_options& o, const T* b0, T* z0, cudaStream_t s, double* dot = nullptr,
+            int* dot_cnt = nullptr) {
   const int nlev = D.nlev;
   const double w = o.omega;
   double* flag = D.scal + S_FLAG;
@@ -1375,6 +1457,16 @@ bool vcycle(DeviceState& D, const cdg_options& o, const T* b0, T* z0, cudaStream
       if (carry && k + 1 == o.nu_post) {
         if (!launch_smooth_prolong<T>(D, l - 1, x, (const T*)L.bh, out, w, o.nu_pre >= 1, s, flag)) return false;
         prolonged[l - 1] = 1;
+      } else if (out == z0 && dot && D.fixed && sizeof(T) == 8) {
+        FxOp q = operator_op(L, 3);
+        q.x = (const double*)x;
+        q.b = (const double*)L.bh;
+        q.y = (double*)out;
+        q.omega = w;
+        q.dot = dot;
+        q.dotv = (const double*)b0;
+        *dot_cnt = (int)fx_grid(q);
+        if (!fx_run(q, s)) return false;
       } else if (!level_bsr<T>(D, L, 3, x, (const T*)L.bh, out, w, nullptr, s)) {
         return false;
       }
@@ -1394,42 +1486,47 @@ bool vcycle(DeviceState& D, const cdg_options& o, const T* b0, T* z0, cudaStream
   return true;
 }
 
-int precond(cdg_handle* h, const double* r, double* z, cudaStream_t s) {
+int bad_np(cdg_handle* h) {
+  h->err = "unsupported number of basis functions per element";
+  return CDG_EINVAL;
+}
+
+// z = V(r) in the V-cycle precision T, by the persistent kernel where it is asked for and accepted
+template <typename T>
+int cycle(cdg_handle* h, const T* r, T* z, cudaStream_t s, double* dot = nullptr, int* dot_cnt = nullptr) {
   DeviceState& D = *h->dev;
-  const size_t n = (size_t)D.ndofs;
-  bool ok;
   const bool pv = h->opt.persistent_vcycle != 0 && !D.pv_failed;
-  if (D.precision == 0) {
-    ok = pv && vcycle_persistent(D, h->opt, false, r, z, D.pv_count, D.pv_err, s);
-    if (!ok) {
-      if (pv) cudaGetLastError();   // a refused cooperative launch: take the per-phase kernels
-      D.pv_failed = D.pv_failed || pv;
-      ok = vcycle<double>(D, h->opt, r, z, s);
-    }
-  } else {
-    launch(convert_kernel<double, float>, vec_grid(n), kThreads, s, n, r, D.r32);
-    ok = pv && vcycle_persistent(D, h->opt, true, D.r32, D.z32, D.pv_count, D.pv_err, s);
-    if (!ok) {
-      if (pv) cudaGetLastError();
-      D.pv_failed = D.pv_failed || pv;
-      ok = vcycle<float>(D, h->opt, D.r32, D.z32, s);
-    }
-    launch(convert_kernel<float, double>, vec_grid(n), kThreads, s, n, D.z32, z);
-  }
+  bool ok = pv && vcycle_persistent(D, h->opt, sizeof(T) == 4, r, z, D.pv_count, D.pv_err, s);
   if (!ok) {
-    h->err = "unsupported number of basis functions per element";
-    return CDG_EINVAL;
+    if (pv) cudaGetLastError();   // a refused cooperative launch: take the per-phase kernels
+    D.pv_failed = D.pv_failed || pv;
+    ok = vcycle<T>(D, h->opt, r, z, s, dot, dot_cnt);
   }
+  if (!ok) return bad_np(h);
   CDG_CHECK_LAUNCH(h, "vcycle");
   return CDG_OK;
 }
 
-int dot_to(cdg_handle* h, const double* x, const double* y, const double* w, int which, cudaStream_t s) {
+int precond(cdg_handle* h, const double* r, double* z, cudaStream_t s) {
   DeviceState& D = *h->dev;
-  const unsigned g = (unsigned)(D.nseg * D.bps);
-  launch(dot_kernel, g, kThreads, s, (const long long*)D.seg_dof, D.bps, x, y, w, D.partial, D.npartial);
-  launch(finalize_kernel, (unsigned)D.nseg, kThreads, s, (const double*)D.partial, D.bps, D.npartial, which,
-         w != nullptr ? 1 : 0, h->opt.tol, D.scal);
+  const size_t n = (size_t)D.ndofs;
+  if (D.precision == 0) return cycle<double>(h, r, z, s);
+  launch(convert_kernel<double, float>, vec_grid(n), kThreads, s, n, r, D.r32);
+  const int rc = cycle<float>(h, D.r32, D.z32, s);
+  launch(convert_kernel<float, double>, vec_grid(n), kThreads, s, n, D.z32, z);
+  return rc;
+}
+
+template <typename TY>
+void dot(DeviceState& D, const double* x, const TY* y, double* partial, cudaStream_t s) {
+  launch(dot_kernel<TY>, (unsigned)(D.nseg * D.bps), kThreads, s, (const long long*)D.seg_dof, D.bps, x, y, partial);
+}
+
+// which 3: ||x||^2 as S_BB; 4: as the first S_RR
+int dot_to(cdg_handle* h, const double* x, const double* y, int which, cudaStream_t s) {
+  DeviceState& D = *h->dev;
+  dot<double>(D, x, y, D.partial, s);
+  launch(finalize_kernel, (unsigned)D.nseg, kThreads, s, (const double*)D.partial, D.bps, which, h->opt.tol, D.scal);
   CDG_CHECK_LAUNCH(h, "dot");
   return CDG_OK;
 }
@@ -1480,7 +1577,7 @@ int dev_apply0(cdg_handle* h, int mode, const double* x, const double* b, double
 }
 
 int dev_dot(cdg_handle* h, const double* x, const double* y, int which, cudaStream_t s) {
-  return dot_to(h, x, y, nullptr, which, s);
+  return dot_to(h, x, y, which, s);
 }
 
 int dev_cuda_fail(cdg_handle* h, cudaError_t e, const char* where) { return cuda_fail(h, e, where); }
@@ -1942,54 +2039,67 @@ int dev_vcycle(cdg_handle* h, const double* r, double* z, void* stream) {
 }
 
 // One CG iteration is split in two captured graphs: G1 = [q = A p, p.q, x and r
-// updates, r.r] and G2 = [z = V(r), r.z, p = z + beta p].  The host reads the
+// updates, r.r, convergence] and G2 = [z = V(r), r.z, p = z + beta p].  The host reads the
 // per-segment scalars between them (convergence of every mesh is decided on the
-// device; converged meshes get alpha = beta = 0).
-static int cg_part1(cdg_handle* h, cudaStream_t s) {
+// device; converged meshes get alpha = beta = 0).  cond: the conditional handle when the whole loop is
+// one graph.
+static int cg_part1(cdg_handle* h, cudaStream_t s, const cudaGraphConditionalHandle* cond) {
   DeviceState& D = *h->dev;
   const DevLevel& L0 = D.lev[0];
   const unsigned gseg = (unsigned)(D.nseg * D.bps);
+  // p.q: by the apply itself where one mesh makes every CTA's partial the mesh's
+  int cnt = D.bps;
   if (D.nseg == 1) {
-    const unsigned g = D.fixed ? fx_grid(operator_op(L0, 0)) : rows_grid(L0.n, D.np);
-    level_bsr<double>(D, L0, 0, D.p, (const double*)nullptr, D.q, h->opt.omega, D.partial, s);
-    launch(finalize_kernel, 1u, kThreads, s, (const double*)D.partial, (int)g, D.npartial, 0, 0, h->opt.tol,
-           D.scal);
+    cnt = (int)(D.fixed ? fx_grid(operator_op(L0, 0)) : rows_grid(L0.n, D.np));
+    level_bsr<double>(D, L0, 0, D.p, (const double*)nullptr, D.q, h->opt.omega, D.partial_pq, s);
   } else {
     level_bsr<double>(D, L0, 0, D.p, (const double*)nullptr, D.q, h->opt.omega, nullptr, s);
-    int rc = dot_to(h, D.p, D.q, nullptr, 0, s);
-    if (rc != CDG_OK) return rc;
+    dot<double>(D, D.p, D.q, D.partial_pq, s);
   }
-  launch(cg_update_kernel, gseg, kThreads, s, (const long long*)D.seg_dof, D.bps, (const double*)D.scal,
-         (const double*)D.p, (const double*)D.q, D.x, D.r, D.partial);
-  launch(finalize_kernel, (unsigned)D.nseg, kThreads, s, (const double*)D.partial, D.bps, D.npartial, 1, 0,
-         h->opt.tol, D.scal);
+  const bool flexible = D.precision != 0;
+  launch(flexible ? cg_update_kernel<true> : cg_update_kernel<false>, gseg, kThreads, s,
+         (const long long*)D.seg_dof, D.bps, (const double*)D.partial_pq, cnt, D.scal, (const double*)D.p,
+         (const double*)D.q, D.x, D.r, D.r32, (const float*)D.z32, D.partial, D.npartial);
+  launch(cg_check_kernel, 1u, kCheckThreads, s, cond ? *cond : cudaGraphConditionalHandle{}, cond ? 1 : 0, D.nseg, D.bps,
+         (const double*)D.partial, D.npartial, flexible ? 1 : 0, h->opt.tol, h->opt.maxit, D.scal, D.it_dev, D.hist_dev,
+         D.iters_dev, (const int*)D.pv_err);
   CDG_CHECK_LAUNCH(h, "cg");
   return CDG_OK;
 }
 
-static int cg_part2(cdg_handle* h, cudaStream_t s) {
+static int cg_direction(cdg_handle* h, int first, cudaStream_t s) {
   DeviceState& D = *h->dev;
-  const bool flexible = D.precision != 0;
-  const size_t n = (size_t)D.ndofs;
-  if (flexible) cudaMemcpyAsync(D.zold, D.z, sizeof(double) * n, cudaMemcpyDeviceToDevice, s);
-  int rc = precond(h, D.r, D.z, s);
-  if (rc != CDG_OK) return rc;
-  if ((rc = dot_to(h, D.r, D.z, flexible ? D.zold : nullptr, 2, s)) != CDG_OK) return rc;
-  launch(cg_p_kernel, (unsigned)(D.nseg * D.bps), kThreads, s, (const long long*)D.seg_dof, D.bps,
-         (const double*)D.scal, 0, (const double*)D.z, D.p);
+  const unsigned gseg = (unsigned)(D.nseg * D.bps);
+  int rc, cnt = 0;
+  if (D.precision == 0) {
+    if ((rc = cycle<double>(h, D.r, D.z, s, D.nseg == 1 ? D.partial : nullptr, &cnt)) != CDG_OK) return rc;
+    if (cnt == 0) dot<double>(D, D.r, D.z, D.partial, s);
+    launch(cg_p_kernel<double>, gseg, kThreads, s, (const long long*)D.seg_dof, D.bps, (const double*)D.partial,
+           cnt ? cnt : D.bps, D.scal, first, (const double*)D.z, D.p);
+  } else {
+    if ((rc = cycle<float>(h, D.r32, D.z32, s)) != CDG_OK) return rc;
+    dot<float>(D, D.r, D.z32, D.partial, s);
+    launch(cg_p_kernel<float>, gseg, kThreads, s, (const long long*)D.seg_dof, D.bps, (const double*)D.partial, D.bps,
+           D.scal, first, (const float*)D.z32, D.p);
+  }
   CDG_CHECK_LAUNCH(h, "cg");
   return CDG_OK;
+}
+
+static int cg_part2(cdg_handle* h, cudaStream_t s, const cudaGraphConditionalHandle*) {
+  return cg_direction(h, 0, s);
 }
 
 // Captures one part into an executable graph on the private stream.
-static int capture(cdg_handle* h, int (*part)(cdg_handle*, cudaStream_t), cudaGraphExec_t* exec,
+static int capture(cdg_handle* h, int (*part)(cdg_handle*, cudaStream_t, const cudaGraphConditionalHandle*),
+                   cudaGraphExec_t* exec,
                    long long* kernels) {
   DeviceState& D = *h->dev;
   cudaGraph_t g = nullptr;
   const long long before = g_launches.load();
   cudaError_t e = cudaStreamBeginCapture(D.stream, cudaStreamCaptureModeThreadLocal);
   if (e != cudaSuccess) return cuda_fail(h, e, "graph capture");
-  const int rc = part(h, D.stream);
+  const int rc = part(h, D.stream, nullptr);
   e = cudaStreamEndCapture(D.stream, &g);
   // captured launches run when the graph is launched: count them there
   *kernels = g_launches.load() - before;
@@ -2005,7 +2115,7 @@ static int capture(cdg_handle* h, int (*part)(cdg_handle*, cudaStream_t), cudaGr
   return CDG_OK;
 }
 
-// The whole CG loop as one executable graph: WHILE (cond) { G1; check; G2 }.  The condition
+// The whole CG loop as one executable graph: WHILE (cond) { G1; G2 }, G1 ending in the check.  The condition
 // starts at 1 on every launch; the check kernel clears it when every segment has converged or
 // maxit iterations are done, so the loop always ends.  G2 of the last iteration is not needed
 // (it changes z and p only).
@@ -2034,12 +2144,8 @@ static int capture_solve(cdg_handle* h) {
     cudaGraphDestroy(g);
     return cuda_fail(h, e, "solve graph capture");
   }
-  int rc = cg_part1(h, D.stream);
-  if (rc == CDG_OK) {
-    launch(cg_check_kernel, 1u, 64u, D.stream, cond, D.nseg, h->opt.maxit, D.scal, D.it_dev, D.hist_dev,
-           D.iters_dev, (const int*)D.pv_err);
-    rc = cg_part2(h, D.stream);
-  }
+  int rc = cg_part1(h, D.stream, &cond);
+  if (rc == CDG_OK) rc = cg_part2(h, D.stream, nullptr);
   cudaGraph_t captured = nullptr;
   const cudaError_t e2 = cudaStreamEndCapture(D.stream, &captured);
   D.gsolve_kernels = g_launches.load() - before;
@@ -2102,8 +2208,8 @@ int dev_solve(cdg_handle* h, const double* f_q, const double* gD, const double* 
     cudaMemsetAsync(D.x, 0, sizeof(double) * n, s);
     cudaMemcpyAsync(D.r, D.bt, sizeof(double) * n, cudaMemcpyDeviceToDevice, s);
   }
-  if ((rc = dot_to(h, D.bt, D.bt, nullptr, 3, s)) != CDG_OK) return rc;
-  if ((rc = dot_to(h, D.r, D.r, nullptr, 4, s)) != CDG_OK) return rc;
+  if ((rc = dot_to(h, D.bt, D.bt, 3, s)) != CDG_OK) return rc;
+  if ((rc = dot_to(h, D.r, D.r, 4, s)) != CDG_OK) return rc;
   std::vector<double> hs((size_t)S_COUNT * nseg);
   cudaMemcpyAsync(hs.data(), D.scal, sizeof(double) * hs.size(), cudaMemcpyDeviceToHost, s);
   cudaError_t e = cudaStreamSynchronize(s);
@@ -2132,10 +2238,8 @@ int dev_solve(cdg_handle* h, const double* f_q, const double* gD, const double* 
       done[0] = status != CDG_ENOCONV;
     }
   } else if (ndone < nseg) {
-    if ((rc = precond(h, D.r, D.z, s)) != CDG_OK) return rc;
-    if ((rc = dot_to(h, D.r, D.z, nullptr, 2, s)) != CDG_OK) return rc;
-    launch(cg_p_kernel, (unsigned)(nseg * D.bps), kThreads, s, (const long long*)D.seg_dof, D.bps,
-           (const double*)D.scal, 1, (const double*)D.z, D.p);
+    if (D.precision != 0) launch(convert_kernel<double, float>, vec_grid(n), kThreads, s, n, (const double*)D.r, D.r32);
+    if ((rc = cg_direction(h, 1, s)) != CDG_OK) return rc;
     if (o.solve_graph && o.maxit > 0 && !D.gsolve && !D.gsolve_failed && capture_solve(h) != CDG_OK) {
       D.gsolve_failed = true;   // refused by this driver: keep the host-driven loop
       h->err.clear();

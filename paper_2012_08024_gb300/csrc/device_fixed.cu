@@ -43,30 +43,12 @@
 #include <algorithm>
 
 #include "device_fixed.cuh"
+#include "device_kernels.cuh"
 #include "device_state.h"
 
 namespace {
 
 using namespace fx;
-
-__device__ __forceinline__ double warp_sum(double v) {
-  for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-  return v;
-}
-
-// dot[CTA] = the CTA's sum of v
-template <int WARPS>
-__device__ __forceinline__ void block_dot(double v, double* __restrict__ dot) {
-  __shared__ double red[WARPS];
-  v = warp_sum(v);
-  if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = v;
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    double s = 0.0;
-    for (int w = 0; w < WARPS; ++w) s += red[w];
-    dot[blockIdx.x] = s;
-  }
-}
 
 template <int NP, int MODE, bool WPR>
 __global__ void __launch_bounds__(kFxThreads, fx_ctas_per_sm(NP)) fx_kernel(const __grid_constant__ FxOp q) {
@@ -77,8 +59,12 @@ __global__ void __launch_bounds__(kFxThreads, fx_ctas_per_sm(NP)) fx_kernel(cons
   double dsum = 0.0;
   for (int pack = blockIdx.x * kFxWarps + (threadIdx.x >> 5); pack < packs; pack += stride)
     dsum = fx_pack<NP, MODE, WPR, false>(q, pack, digits[threadIdx.x >> 5], dsum);
-  if constexpr (MODE == 0)
-    if (q.dot) block_dot<kFxWarps>(dsum, q.dot);
+  if constexpr (MODE == 0 || MODE == 3)
+    if (q.dot) {
+      __shared__ double red[kFxThreads];
+      dsum = cdgk::cta_sum<kFxWarps>(dsum, red);
+      if ((int)threadIdx.x == cdgk::summing_warp<kFxWarps>() * 32) q.dot[blockIdx.x] = dsum;
+    }
 }
 
 // FP64 blocks to digits, in place: one warp per block row (the row exponents

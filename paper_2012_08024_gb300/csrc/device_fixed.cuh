@@ -133,13 +133,16 @@ __device__ __forceinline__ void fx_mac(const DigitRow<NP>& r, const int2* __rest
   s.carry();
 }
 
-// what becomes of a row's sum (modes below); returns the dot partial of mode 0
+// what becomes of a row's sum (modes below); returns the dot partial of modes 0 and 3
 template <int MODE>
 __device__ __forceinline__ double finish(double acc, size_t o, double xo, double bo, double* y, double* y2,
-                                         double omega, double dsum) {
+                                         double omega, double dsum, const double* dotv) {
   if constexpr (MODE == 1) y[o] = bo - acc;
-  else if constexpr (MODE == 3) y[o] = fma(omega, bo - xo - acc, xo);
-  else if constexpr (MODE == 4) y[o] = xo + acc;
+  else if constexpr (MODE == 3) {
+    const double v = fma(omega, bo - xo - acc, xo);
+    y[o] = v;
+    return dotv ? fma(v, dotv[o], dsum) : dsum;
+  } else if constexpr (MODE == 4) y[o] = xo + acc;
   else y[o] = acc;
   if constexpr (MODE == 6) y2[o] = omega * acc;
   return MODE == 0 ? fma(xo, acc, dsum) : dsum;
@@ -161,7 +164,7 @@ struct Pack {
 
 // One warp on one pack of rows: acc = (A x)_(K, i), then by MODE: 0 y = acc; 1 y = b - acc;
 // 3 y = x + omega (b - x - acc); 8 y = acc, block t meeting element t; with one block per row (no
-// rowptr): 4 y += acc; 6 y = acc, y2 = omega acc; 7 y = acc.  Returns the dot partial of mode 0.
+// rowptr): 4 y += acc; 6 y = acc, y2 = omega acc; 7 y = acc.  Returns the dot partial of modes 0 and 3.
 // q.cols: the rows' columns, q.width of them per row (missing: -1), so that the gathers of x need not
 // wait for the row pointer; one-block modes meet element cols[K] (nullptr: K).
 // COHERENT: vectors are read through L2 only (written earlier in the same kernel).
@@ -297,7 +300,7 @@ __device__ __forceinline__ double fx_pack(const FxOp& q, int pack, int2* __restr
   if (!any_flush) acc = fx_value(hi, lo, ea + ex - 1022);
   if (ea == kNotFinite) acc = nan("");
   if (writes && (MODE == 3 || (MODE == 0 && q.dot))) xo = vload<COHERENT>(q.x + o);
-  return writes ? finish<MODE>(acc, o, xo, bo, q.y, q.y2, q.omega, dsum) : dsum;
+  return writes ? finish<MODE>(acc, o, xo, bo, q.y, q.y2, q.omega, dsum, q.dotv) : dsum;
 }
 
 }  // namespace fx

@@ -7,7 +7,7 @@
 
 // One product with a block-sparse matrix in digit form and what is done with it:
 // mode 0 y = A x (dot: per-CTA partials of x . y, fx_grid of them), 1 y = b - A x,
-// 3 y = x + omega (b - x - A x), 8 y = A x with block t meeting element t; with one block per row
+// 3 y = x + omega (b - x - A x) (dot: partials of y . dotv), 8 y = A x with block t meeting element t; with one block per row
 // (no rowptr): 4 y += A x, 6 y = A x and y2 = omega A x, 7 y = A x.
 // x and y do not overlap.
 struct FxOp {
@@ -24,6 +24,7 @@ struct FxOp {
   double* y2 = nullptr;
   double omega = 0.0;
   double* dot = nullptr;
+  const double* dotv = nullptr;
 };
 
 constexpr int kFxSms = 152;

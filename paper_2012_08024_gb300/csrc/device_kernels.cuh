@@ -142,6 +142,36 @@ __device__ __forceinline__ T row_acc(int K, int i, const int* __restrict__ rowpt
   return acc;
 }
 
+// Sums over a CTA of WARPS warps (threads x), done by one warp: the FP64 pipe of this GPU takes 64 clocks
+// for a warp's addition, so a shuffle reduction in every warp of every CTA costs microseconds (64 warps
+// per SM, five additions each: 2.5 us per sum).  One warp adds the other warps' lanes pairwise and then
+// its own lanes: WARPS + 4 additions per CTA; CTAs on one SM take different warps, and so quadrants.
+template <int WARPS>
+__device__ __forceinline__ int summing_warp() { return (int)(blockIdx.x + blockIdx.x / 152) % WARPS; }
+
+__device__ __forceinline__ double lanes_sum(double v) {
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+  return v;
+}
+
+// the sum of v over the CTA, valid in the summing warp; red: [32 WARPS] in shared memory
+template <int WARPS>
+__device__ __forceinline__ double cta_sum(double v, double* red) {
+  __syncthreads();   // red may still be read
+  red[threadIdx.x] = v;
+  __syncthreads();
+  if ((int)(threadIdx.x >> 5) != summing_warp<WARPS>()) return 0.0;
+  double t[WARPS];
+#pragma unroll
+  for (int w = 0; w < WARPS; ++w) t[w] = red[w * 32 + (threadIdx.x & 31)];
+#pragma unroll
+  for (int h = 1; h < WARPS; h *= 2)
+#pragma unroll
+    for (int w = 0; w + h < WARPS; w += 2 * h) t[w] += t[w + h];
+  return lanes_sum(t[0]);
+}
+
 // The same for a whole warp on one block row: floor(32 / n_p) groups of n_p lanes share its blocks
 // (group g takes blocks g, g + G, ...; two at a time in flight), lane i of a group row i; the sums
 // of the groups are added in a fixed order.  Valid in the lanes of group 0.  x aligned for VecLoad.

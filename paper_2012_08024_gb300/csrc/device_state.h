@@ -15,8 +15,8 @@ constexpr int kDotBlocks1 = 2 * 152;  // the same for single-mesh handles (their
 
 // per-segment CG scalars (one row of S_COUNT doubles per mesh of the handle)
 // S_HDONE: the segment's residual history is closed (single-graph solve); S_RZO: the new r times the
-// previous z (Polak-Ribiere)
-enum Scal { S_RZ = 0, S_PQ, S_RR, S_BB, S_ALPHA, S_BETA, S_DONE, S_BREAK, S_IT, S_HDONE, S_RZO, S_FLAG = 15, S_COUNT = 16 };
+// previous z (Polak-Ribiere); S_RZN: r.z as the direction update leaves it, S_RZ from the next update on
+enum Scal { S_RZ = 0, S_PQ, S_RR, S_BB, S_ALPHA, S_BETA, S_DONE, S_BREAK, S_IT, S_HDONE, S_RZO, S_RZN, S_FLAG = 15, S_COUNT = 16 };
 
 struct DevLevel {
   int n = 0;
@@ -85,13 +85,13 @@ struct DeviceState {
   double* dk_blk = nullptr;
   double* kappa = nullptr;
   // CG vectors (FP64, tree order)
-  double *x = nullptr, *r = nullptr, *z = nullptr, *p = nullptr, *q = nullptr, *bt = nullptr,
-         *zold = nullptr;
+  double *x = nullptr, *r = nullptr, *z = nullptr, *p = nullptr, *q = nullptr, *bt = nullptr;
   float *r32 = nullptr, *z32 = nullptr;
   // staging for host-pointer solves
   double *f_stage = nullptr, *gD_stage = nullptr, *gN_stage = nullptr, *u_stage = nullptr;
   double* scal = nullptr;       // [nseg][S_COUNT]
-  double* partial = nullptr;
+  double* partial = nullptr;    // [2][npartial]: r.r (and r.z_old), then r.z
+  double* partial_pq = nullptr; // [npartial]: p.A p
   int npartial = 0;
   // segments (meshes of a batched handle)
   int nseg = 1, bps = 1;        // blocks per segment of the segmented vector kernels
