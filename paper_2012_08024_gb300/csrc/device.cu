@@ -268,6 +268,7 @@ __global__ void __launch_bounds__(kThreads, 8 / UNR) bsr_kernel(int n, const int
                                                        const T* __restrict__ Dinv, const T* __restrict__ x,
                                                        const T* __restrict__ b, T* __restrict__ y, T omega,
                                                        double* __restrict__ dot) {
+  cdgk::wait_for_inputs();
   constexpr int RPW = 32 / NP;
   const int lane = threadIdx.x & 31;
   const int warp = (int)((blockIdx.x * (size_t)blockDim.x + threadIdx.x) >> 5);
@@ -430,6 +431,8 @@ __global__ void __launch_bounds__(kRowThreads) bsr_row_kernel(int n, const int* 
                                                               const T* __restrict__ x, const T* __restrict__ b,
                                                               T* __restrict__ y, T omega) {
   const int K = blockIdx.x * (kRowThreads / 32) + (threadIdx.x >> 5);
+  if (K < n) cdgk::touch_row<T, NP>(K, rowptr, col, A);
+  cdgk::wait_for_inputs();
   if (K >= n) return;
   const T acc = cdgk::split_row_acc<T, NP>(K, rowptr, col, A, x);
   const int i = threadIdx.x & 31;
@@ -444,6 +447,7 @@ template <typename T, int NP>
 __global__ void __launch_bounds__(kRowThreads) restrict_row_kernel(int nc, const int* __restrict__ childptr,
                                                                    const T* __restrict__ L, const T* __restrict__ r,
                                                                    T* __restrict__ bc) {
+  cdgk::wait_for_inputs();
   const int Ag = blockIdx.x * (kRowThreads / 32) + (threadIdx.x >> 5);
   if (Ag >= nc) return;
   const T acc = cdgk::split_restrict<T, NP>(Ag, childptr, L, r);
@@ -456,6 +460,7 @@ template <typename T, int NP, bool WRITE_X>
 __global__ void __launch_bounds__(kThreads) smooth_first_kernel(int n, const T* __restrict__ Dinv,
                                                                 const T* __restrict__ b, T* __restrict__ bh,
                                                                 T* __restrict__ x, T omega) {
+  cdgk::wait_for_inputs();
   constexpr int RPW = 32 / NP;
   const int lane = threadIdx.x & 31;
   const int warp = (int)((blockIdx.x * (size_t)blockDim.x + threadIdx.x) >> 5);
@@ -467,7 +472,7 @@ __global__ void __launch_bounds__(kThreads) smooth_first_kernel(int n, const T* 
   const T* bk = b + (size_t)K * NP;
   T s = T(0);
 #pragma unroll
-  for (int j = 0; j < NP; ++j) s = fma(ldg(D + j), ldg(bk + j), s);
+  for (int j = 0; j < NP; ++j) s = fma(ldg(D + j), cdgk::ld<cdgk::kPlain>(bk + j), s);
   bh[(size_t)K * NP + i] = s;
   if (WRITE_X) x[(size_t)K * NP + i] = omega * s;
 }
@@ -477,6 +482,7 @@ template <typename T, int NP>
 __global__ void __launch_bounds__(kThreads) restrict_kernel(int nc, const int* __restrict__ childptr,
                                                             const T* __restrict__ L, const T* __restrict__ r,
                                                             T* __restrict__ bc) {
+  cdgk::wait_for_inputs();
   constexpr int RPW = 32 / NP;
   const int lane = threadIdx.x & 31;
   const int warp = (int)((blockIdx.x * (size_t)blockDim.x + threadIdx.x) >> 5);
@@ -489,7 +495,7 @@ __global__ void __launch_bounds__(kThreads) restrict_kernel(int nc, const int* _
     const T* LK = L + (size_t)K * NP * NP + i;
     const T* rk = r + (size_t)K * NP;
 #pragma unroll
-    for (int j = 0; j < NP; ++j) s = fma(ldg(LK + j * NP), ldg(rk + j), s);
+    for (int j = 0; j < NP; ++j) s = fma(ldg(LK + j * NP), cdgk::ld<cdgk::kPlain>(rk + j), s);
   }
   bc[(size_t)Ag * NP + i] = s;
 }
@@ -499,6 +505,7 @@ template <typename T, int NP, bool ADD>
 __global__ void __launch_bounds__(kThreads) prolong_kernel(int n, const int* __restrict__ parent,
                                                            const T* __restrict__ L, const T* __restrict__ xc,
                                                            T* __restrict__ x) {
+  cdgk::wait_for_inputs();
   constexpr int RPW = 32 / NP;
   const int lane = threadIdx.x & 31;
   const int warp = (int)((blockIdx.x * (size_t)blockDim.x + threadIdx.x) >> 5);
@@ -510,7 +517,7 @@ __global__ void __launch_bounds__(kThreads) prolong_kernel(int n, const int* __r
   const T* xa = xc + (size_t)parent[K] * NP;
   T s = T(0);
 #pragma unroll
-  for (int j = 0; j < NP; ++j) s = fma(ldg(LK + j), ldg(xa + j), s);
+  for (int j = 0; j < NP; ++j) s = fma(ldg(LK + j), cdgk::ld<cdgk::kPlain>(xa + j), s);
   const size_t row = (size_t)K * NP + i;
   x[row] = ADD ? x[row] + s : s;
 }
@@ -524,13 +531,25 @@ __global__ void coarse_kernel(int nc, const int* __restrict__ crow_seg, const in
                               const TI* __restrict__ b, TO* __restrict__ x) {
   const int row = (int)((blockIdx.x * (size_t)blockDim.x + threadIdx.x) >> 5);
   const int lane = threadIdx.x & 31;
-  if (row >= nc) return;
+  if (row >= nc) {
+    cdgk::wait_for_inputs();
+    return;
+  }
   const int m = crow_seg[row];
   const int r0 = crow_off[m], nm = crow_off[m + 1] - r0;
   const double* a = Ainv + cinv_off[m] + (size_t)(row - r0) * nm;
   const TI* bm = b + r0;
+  // the row's first values before the right-hand side is there
+  constexpr int kAhead = 8;
+  double av[kAhead];
+#pragma unroll
+  for (int k = 0; k < kAhead; ++k) av[k] = lane + 32 * k < nm ? a[lane + 32 * k] : 0.0;
+  cdgk::wait_for_inputs();
   double s = 0.0;
-  for (int j = lane; j < nm; j += 32) s = fma(a[j], cvt<double>(bm[j]), s);
+#pragma unroll
+  for (int k = 0; k < kAhead; ++k)
+    if (lane + 32 * k < nm) s = fma(av[k], cvt<double>(bm[lane + 32 * k]), s);
+  for (int j = lane + 32 * kAhead; j < nm; j += 32) s = fma(a[j], cvt<double>(bm[j]), s);
   for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
   if (lane == 0) x[row] = ADD ? cvt<TO>(cvt<double>(x[row]) + s) : cvt<TO>(s);
 }
@@ -543,6 +562,7 @@ __global__ void coarse_kernel(int nc, const int* __restrict__ crow_seg, const in
 template <typename T>
 __global__ void __launch_bounds__(kThreads) ptrunc_restrict_kernel(int n, int npf, int npc,
                                                                    const T* __restrict__ r, T* __restrict__ bc) {
+  cdgk::wait_for_inputs();
   const size_t tot = (size_t)n * npc;
   for (size_t t = blockIdx.x * (size_t)blockDim.x + threadIdx.x; t < tot; t += (size_t)gridDim.x * blockDim.x) {
     const size_t K = t / npc;
@@ -553,6 +573,7 @@ __global__ void __launch_bounds__(kThreads) ptrunc_restrict_kernel(int n, int np
 template <typename T, bool ADD>
 __global__ void __launch_bounds__(kThreads) ptrunc_prolong_kernel(int n, int npf, int npc,
                                                                   const T* __restrict__ xc, T* __restrict__ x) {
+  cdgk::wait_for_inputs();
   const size_t tot = (size_t)n * npf;
   for (size_t t = blockIdx.x * (size_t)blockDim.x + threadIdx.x; t < tot; t += (size_t)gridDim.x * blockDim.x) {
     const size_t K = t / npf;
@@ -564,6 +585,7 @@ __global__ void __launch_bounds__(kThreads) ptrunc_prolong_kernel(int n, int npf
 
 template <typename TI, typename TO>
 __global__ void convert_kernel(size_t n, const TI* __restrict__ a, TO* __restrict__ b) {
+  cdgk::wait_for_inputs();
   for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < n; i += (size_t)gridDim.x * blockDim.x)
     b[i] = cvt<TO>(a[i]);
 }
@@ -593,6 +615,7 @@ template <typename TY>
 __global__ void __launch_bounds__(kThreads) dot_kernel(const long long* __restrict__ seg_dof, int bps,
                                                        const double* __restrict__ x, const TY* __restrict__ y,
                                                        double* __restrict__ partial) {
+  cdgk::wait_for_inputs();
   int seg;
   size_t lo, hi;
   seg_range(seg_dof, bps, seg, lo, hi);
@@ -644,6 +667,7 @@ __device__ __forceinline__ double partials_sum(const double* __restrict__ p, int
 // One CTA per segment: ||b||^2 (which 3) or the first ||r||^2 (4) from its cnt partials.
 __global__ void finalize_kernel(const double* __restrict__ partial, int cnt, int which, double tol,
                                 double* __restrict__ scal) {
+  cdgk::wait_for_inputs();
   const double tot = partials_sum(partial + (size_t)blockIdx.x * cnt, cnt);
   if (threadIdx.x != 0) return;
   double* sc = scal + (size_t)blockIdx.x * S_COUNT;
@@ -672,6 +696,7 @@ __global__ void __launch_bounds__(kThreads) cg_update_kernel(const long long* __
                                                              double* __restrict__ r, float* __restrict__ r32,
                                                              const float* __restrict__ z,
                                                              double* __restrict__ partial, int npart) {
+  cdgk::wait_for_inputs();
   int seg;
   size_t lo, hi;
   seg_range(seg_dof, bps, seg, lo, hi);
@@ -754,6 +779,7 @@ __global__ void __launch_bounds__(kCheckThreads) cg_check_kernel(cudaGraphCondit
                                                                  double* __restrict__ scal, int* __restrict__ it_dev,
                                                                  double* __restrict__ hist, int* __restrict__ iters,
                                                                  const int* __restrict__ wait_err) {
+  cdgk::wait_for_inputs();
   const int it = in_graph ? *it_dev + 1 : 0;
   int open = 0;
   auto close = [&](int m, double rr, double rzo) {
@@ -816,6 +842,7 @@ __global__ void __launch_bounds__(kThreads) cg_p_kernel(const long long* __restr
                                                         const double* __restrict__ rzp, int rz_cnt,
                                                         double* __restrict__ scal, int first,
                                                         const TZ* __restrict__ z, double* __restrict__ p) {
+  cdgk::wait_for_inputs();
   int seg;
   size_t lo, hi;
   seg_range(seg_dof, bps, seg, lo, hi);
@@ -887,6 +914,7 @@ __global__ void __launch_bounds__(kThreads) rhs_kernel(int ne, int nq, int nfq, 
 
 __global__ void permute_kernel(int ne, int np, const int* __restrict__ perm0, const double* __restrict__ in,
                                double* __restrict__ out, int to_tree) {
+  cdgk::wait_for_inputs();
   const size_t n = (size_t)ne * np;
   for (size_t t = blockIdx.x * (size_t)blockDim.x + threadIdx.x; t < n; t += (size_t)gridDim.x * blockDim.x) {
     const size_t k = t / np, i = t - k * np;
@@ -1023,7 +1051,7 @@ inline unsigned rows_grid(int64_t nrows, int np) {
 template <typename T, int NP, int MODE, int UNR>
 void launch_vec(unsigned g, cudaStream_t s, int n, const int* rowptr, const int* col, const T* A, const T* x,
                 const T* b, T* y, double omega, double* dot) {
-  launch(bsr_kernel<T, NP, MODE, true, UNR>, g, kThreads, s, n, rowptr, col, A, (const T*)nullptr, x, b, y,
+  launch_dep(bsr_kernel<T, NP, MODE, true, UNR>, g, kThreads, s, n, rowptr, col, A, (const T*)nullptr, x, b, y,
          (T)omega, MODE == 0 ? dot : (double*)nullptr);
 }
 
@@ -1055,13 +1083,13 @@ bool launch_bsr(int mode, int np, int n, const int* rowptr, const int* col, cons
   }
   CDG_NP_DISPATCH(np, {
     if (mode == 0)
-      launch(bsr_kernel<T, NP, 0, false>, g, kThreads, s, n, rowptr, col, A, (const T*)nullptr, x, b, y, (T)omega,
+      launch_dep(bsr_kernel<T, NP, 0, false>, g, kThreads, s, n, rowptr, col, A, (const T*)nullptr, x, b, y, (T)omega,
              dot);
     else if (mode == 1)
-      launch(bsr_kernel<T, NP, 1, false>, g, kThreads, s, n, rowptr, col, A, (const T*)nullptr, x, b, y, (T)omega,
+      launch_dep(bsr_kernel<T, NP, 1, false>, g, kThreads, s, n, rowptr, col, A, (const T*)nullptr, x, b, y, (T)omega,
              (double*)nullptr);
     else
-      launch(bsr_kernel<T, NP, 3, false>, g, kThreads, s, n, rowptr, col, A, (const T*)nullptr, x, b, y, (T)omega,
+      launch_dep(bsr_kernel<T, NP, 3, false>, g, kThreads, s, n, rowptr, col, A, (const T*)nullptr, x, b, y, (T)omega,
              (double*)nullptr);
   });
   return true;
@@ -1070,8 +1098,8 @@ bool launch_bsr(int mode, int np, int n, const int* rowptr, const int* col, cons
 template <typename T>
 bool launch_smooth_first(int np, int n, const T* Dinv, const T* b, T* bh, T* x, double omega, cudaStream_t s) {
   CDG_NP_DISPATCH(np, {
-    if (x) launch(smooth_first_kernel<T, NP, true>, rows_grid(n, np), kThreads, s, n, Dinv, b, bh, x, (T)omega);
-    else launch(smooth_first_kernel<T, NP, false>, rows_grid(n, np), kThreads, s, n, Dinv, b, bh, x, (T)omega);
+    if (x) launch_dep(smooth_first_kernel<T, NP, true>, rows_grid(n, np), kThreads, s, n, Dinv, b, bh, x, (T)omega);
+    else launch_dep(smooth_first_kernel<T, NP, false>, rows_grid(n, np), kThreads, s, n, Dinv, b, bh, x, (T)omega);
   });
   return true;
 }
@@ -1083,15 +1111,15 @@ bool launch_restrict(int np, int nc, const int* cp, const T* L, const T* r, T* b
   constexpr int kRT = 64;
   const int64_t warps = ((int64_t)nc + 32 / np - 1) / (32 / np);
   const unsigned g = (unsigned)std::max<int64_t>(1, (warps * 32 + kRT - 1) / kRT);
-  CDG_NP_DISPATCH(np, launch(restrict_kernel<T, NP>, g, kRT, s, nc, cp, L, r, bc));
+  CDG_NP_DISPATCH(np, launch_dep(restrict_kernel<T, NP>, g, kRT, s, nc, cp, L, r, bc));
   return true;
 }
 
 template <typename T>
 bool launch_prolong(int np, int n, const int* parent, const T* L, const T* xc, T* x, bool add, cudaStream_t s) {
   CDG_NP_DISPATCH(np, {
-    if (add) launch(prolong_kernel<T, NP, true>, rows_grid(n, np), kThreads, s, n, parent, L, xc, x);
-    else launch(prolong_kernel<T, NP, false>, rows_grid(n, np), kThreads, s, n, parent, L, xc, x);
+    if (add) launch_dep(prolong_kernel<T, NP, true>, rows_grid(n, np), kThreads, s, n, parent, L, xc, x);
+    else launch_dep(prolong_kernel<T, NP, false>, rows_grid(n, np), kThreads, s, n, parent, L, xc, x);
   });
   return true;
 }
@@ -1105,7 +1133,7 @@ bool transfer_restrict(const DeviceState& D, int l, const T* Lb, const T* r, T* 
   const DevLevel& F = D.lev[l];
   const DevLevel& C = D.lev[l + 1];
   if (F.ptrans) {
-    launch(ptrunc_restrict_kernel<T>, vec_grid((size_t)C.n * C.np), kThreads, s, C.n, F.np, C.np, r, bc);
+    launch_dep(ptrunc_restrict_kernel<T>, vec_grid((size_t)C.n * C.np), kThreads, s, C.n, F.np, C.np, r, bc);
     return true;
   }
   return launch_restrict<T>(F.np, C.n, C.childptr, Lb, r, bc, s);
@@ -1116,8 +1144,8 @@ bool transfer_prolong(const DeviceState& D, int l, const T* Lb, const T* xc, T* 
   const DevLevel& F = D.lev[l];
   const DevLevel& C = D.lev[l + 1];
   if (F.ptrans) {
-    if (add) launch(ptrunc_prolong_kernel<T, true>, vec_grid((size_t)F.n * F.np), kThreads, s, F.n, F.np, C.np, xc, x);
-    else launch(ptrunc_prolong_kernel<T, false>, vec_grid((size_t)F.n * F.np), kThreads, s, F.n, F.np, C.np, xc, x);
+    if (add) launch_dep(ptrunc_prolong_kernel<T, true>, vec_grid((size_t)F.n * F.np), kThreads, s, F.n, F.np, C.np, xc, x);
+    else launch_dep(ptrunc_prolong_kernel<T, false>, vec_grid((size_t)F.n * F.np), kThreads, s, F.n, F.np, C.np, xc, x);
     return true;
   }
   return launch_prolong<T>(F.np, F.n, F.parent, Lb, xc, x, add, s);
@@ -1190,9 +1218,9 @@ bool level_bsr(const DeviceState& D, const DevLevel& L, int mode, const T* x, co
       switch (L.np) {
 #define CDG_ROW(NPV)                                                                                             \
   case NPV:                                                                                                      \
-    if (mode == 0) launch(bsr_row_kernel<T, NPV, 0>, g, kRowThreads, s, L.n, rp, cl, M, x, b, y, (T)omega);      \
-    else if (mode == 1) launch(bsr_row_kernel<T, NPV, 1>, g, kRowThreads, s, L.n, rp, cl, M, x, b, y, (T)omega); \
-    else launch(bsr_row_kernel<T, NPV, 3>, g, kRowThreads, s, L.n, rp, cl, M, x, b, y, (T)omega);                \
+    if (mode == 0) launch_dep(bsr_row_kernel<T, NPV, 0>, g, kRowThreads, s, L.n, rp, cl, M, x, b, y, (T)omega);      \
+    else if (mode == 1) launch_dep(bsr_row_kernel<T, NPV, 1>, g, kRowThreads, s, L.n, rp, cl, M, x, b, y, (T)omega); \
+    else launch_dep(bsr_row_kernel<T, NPV, 3>, g, kRowThreads, s, L.n, rp, cl, M, x, b, y, (T)omega);                \
     return true;
         CDG_ROW(3) CDG_ROW(4) CDG_ROW(6) CDG_ROW(10) CDG_ROW(15)
 #undef CDG_ROW
@@ -1244,11 +1272,11 @@ bool level_restrict(const DeviceState& D, int l, const T* r, T* bc, cudaStream_t
     const unsigned g = (unsigned)((nc + kRowThreads / 32 - 1) / (kRowThreads / 32));
     const int* cp = D.lev[l + 1].childptr;
     switch (F.np) {
-      case 3: launch(restrict_row_kernel<T, 3>, g, kRowThreads, s, nc, cp, opL<T>(F), r, bc); return true;
-      case 4: launch(restrict_row_kernel<T, 4>, g, kRowThreads, s, nc, cp, opL<T>(F), r, bc); return true;
-      case 6: launch(restrict_row_kernel<T, 6>, g, kRowThreads, s, nc, cp, opL<T>(F), r, bc); return true;
-      case 10: launch(restrict_row_kernel<T, 10>, g, kRowThreads, s, nc, cp, opL<T>(F), r, bc); return true;
-      case 15: launch(restrict_row_kernel<T, 15>, g, kRowThreads, s, nc, cp, opL<T>(F), r, bc); return true;
+      case 3: launch_dep(restrict_row_kernel<T, 3>, g, kRowThreads, s, nc, cp, opL<T>(F), r, bc); return true;
+      case 4: launch_dep(restrict_row_kernel<T, 4>, g, kRowThreads, s, nc, cp, opL<T>(F), r, bc); return true;
+      case 6: launch_dep(restrict_row_kernel<T, 6>, g, kRowThreads, s, nc, cp, opL<T>(F), r, bc); return true;
+      case 10: launch_dep(restrict_row_kernel<T, 10>, g, kRowThreads, s, nc, cp, opL<T>(F), r, bc); return true;
+      case 15: launch_dep(restrict_row_kernel<T, 15>, g, kRowThreads, s, nc, cp, opL<T>(F), r, bc); return true;
       default: break;
     }
   }
@@ -1363,14 +1391,14 @@ bool launch_smooth_prolong(const DeviceState& D, int l, const T* x, const T* bh,
 template <typename T>
 void coarse_solve(DeviceState& D, const T* b, T* x, cudaStream_t s) {
   const unsigned g = (unsigned)((D.nc * 32 + 255) / 256);
-  launch(coarse_kernel<T, T, false>, g, 256, s, D.nc, D.crow_seg, D.crow_off, D.cinv_off, D.coarse_inv, b, x);
+  launch_dep(coarse_kernel<T, T, false>, g, 256, s, D.nc, D.crow_seg, D.crow_off, D.cinv_off, D.coarse_inv, b, x);
   if constexpr (sizeof(T) == sizeof(double)) {
     const DevLevel& C = D.lev[D.nlev - 1];
     if (!C.A || D.precision != 0) return;   // the work vectors of an FP32 V-cycle hold floats
     double* r = (double*)C.r;
     const bool aligned = (((uintptr_t)b | (uintptr_t)x) & 15) == 0;
     level_bsr<double>(D, C, 1, x, b, r, 0.0, nullptr, s, aligned);
-    launch(coarse_kernel<double, double, true>, g, 256, s, D.nc, D.crow_seg, D.crow_off, D.cinv_off, D.coarse_inv,
+    launch_dep(coarse_kernel<double, double, true>, g, 256, s, D.nc, D.crow_seg, D.crow_off, D.cinv_off, D.coarse_inv,
            (const double*)r, x);
   }
 }
@@ -1511,22 +1539,22 @@ int precond(cdg_handle* h, const double* r, double* z, cudaStream_t s) {
   DeviceState& D = *h->dev;
   const size_t n = (size_t)D.ndofs;
   if (D.precision == 0) return cycle<double>(h, r, z, s);
-  launch(convert_kernel<double, float>, vec_grid(n), kThreads, s, n, r, D.r32);
+  launch_dep(convert_kernel<double, float>, vec_grid(n), kThreads, s, n, r, D.r32);
   const int rc = cycle<float>(h, D.r32, D.z32, s);
-  launch(convert_kernel<float, double>, vec_grid(n), kThreads, s, n, D.z32, z);
+  launch_dep(convert_kernel<float, double>, vec_grid(n), kThreads, s, n, D.z32, z);
   return rc;
 }
 
 template <typename TY>
 void dot(DeviceState& D, const double* x, const TY* y, double* partial, cudaStream_t s) {
-  launch(dot_kernel<TY>, (unsigned)(D.nseg * D.bps), kThreads, s, (const long long*)D.seg_dof, D.bps, x, y, partial);
+  launch_dep(dot_kernel<TY>, (unsigned)(D.nseg * D.bps), kThreads, s, (const long long*)D.seg_dof, D.bps, x, y, partial);
 }
 
 // which 3: ||x||^2 as S_BB; 4: as the first S_RR
 int dot_to(cdg_handle* h, const double* x, const double* y, int which, cudaStream_t s) {
   DeviceState& D = *h->dev;
   dot<double>(D, x, y, D.partial, s);
-  launch(finalize_kernel, (unsigned)D.nseg, kThreads, s, (const double*)D.partial, D.bps, which, h->opt.tol, D.scal);
+  launch_dep(finalize_kernel, (unsigned)D.nseg, kThreads, s, (const double*)D.partial, D.bps, which, h->opt.tol, D.scal);
   CDG_CHECK_LAUNCH(h, "dot");
   return CDG_OK;
 }
@@ -1916,7 +1944,7 @@ int dev_permute(cdg_handle* h, const double* in, double* out, bool to_tree, void
   if (!h || !h->dev) return h ? (h->err = "not bound", CDG_ESTATE) : CDG_EINVAL;
   DeviceState& D = *h->dev;
   cudaStream_t s = (cudaStream_t)stream;
-  launch(permute_kernel, vec_grid((size_t)D.ndofs), kThreads, s, (int)D.ne, D.np, D.perm0, in, out, to_tree);
+  launch_dep(permute_kernel, vec_grid((size_t)D.ndofs), kThreads, s, (int)D.ne, D.np, D.perm0, in, out, to_tree);
   CDG_CHECK_LAUNCH(h, "permute");
   return CDG_OK;
 }
@@ -2000,9 +2028,9 @@ int dev_convert(const void* in, void* out, long long n, int to_fp32, void* strea
   if (n == 0) return CDG_OK;
   cudaStream_t s = (cudaStream_t)stream;
   if (to_fp32)
-    launch(convert_kernel<double, float>, vec_grid((size_t)n), kThreads, s, (size_t)n, (const double*)in, (float*)out);
+    launch_dep(convert_kernel<double, float>, vec_grid((size_t)n), kThreads, s, (size_t)n, (const double*)in, (float*)out);
   else
-    launch(convert_kernel<float, double>, vec_grid((size_t)n), kThreads, s, (size_t)n, (const float*)in, (double*)out);
+    launch_dep(convert_kernel<float, double>, vec_grid((size_t)n), kThreads, s, (size_t)n, (const float*)in, (double*)out);
   return cudaGetLastError() == cudaSuccess ? CDG_OK : CDG_ECUDA;
 }
 
@@ -2057,10 +2085,10 @@ static int cg_part1(cdg_handle* h, cudaStream_t s, const cudaGraphConditionalHan
     dot<double>(D, D.p, D.q, D.partial_pq, s);
   }
   const bool flexible = D.precision != 0;
-  launch(flexible ? cg_update_kernel<true> : cg_update_kernel<false>, gseg, kThreads, s,
+  launch_dep(flexible ? cg_update_kernel<true> : cg_update_kernel<false>, gseg, kThreads, s,
          (const long long*)D.seg_dof, D.bps, (const double*)D.partial_pq, cnt, D.scal, (const double*)D.p,
          (const double*)D.q, D.x, D.r, D.r32, (const float*)D.z32, D.partial, D.npartial);
-  launch(cg_check_kernel, 1u, kCheckThreads, s, cond ? *cond : cudaGraphConditionalHandle{}, cond ? 1 : 0, D.nseg, D.bps,
+  launch_dep(cg_check_kernel, 1u, kCheckThreads, s, cond ? *cond : cudaGraphConditionalHandle{}, cond ? 1 : 0, D.nseg, D.bps,
          (const double*)D.partial, D.npartial, flexible ? 1 : 0, h->opt.tol, h->opt.maxit, D.scal, D.it_dev, D.hist_dev,
          D.iters_dev, (const int*)D.pv_err);
   CDG_CHECK_LAUNCH(h, "cg");
@@ -2074,12 +2102,12 @@ static int cg_direction(cdg_handle* h, int first, cudaStream_t s) {
   if (D.precision == 0) {
     if ((rc = cycle<double>(h, D.r, D.z, s, D.nseg == 1 ? D.partial : nullptr, &cnt)) != CDG_OK) return rc;
     if (cnt == 0) dot<double>(D, D.r, D.z, D.partial, s);
-    launch(cg_p_kernel<double>, gseg, kThreads, s, (const long long*)D.seg_dof, D.bps, (const double*)D.partial,
+    launch_dep(cg_p_kernel<double>, gseg, kThreads, s, (const long long*)D.seg_dof, D.bps, (const double*)D.partial,
            cnt ? cnt : D.bps, D.scal, first, (const double*)D.z, D.p);
   } else {
     if ((rc = cycle<float>(h, D.r32, D.z32, s)) != CDG_OK) return rc;
     dot<float>(D, D.r, D.z32, D.partial, s);
-    launch(cg_p_kernel<float>, gseg, kThreads, s, (const long long*)D.seg_dof, D.bps, (const double*)D.partial, D.bps,
+    launch_dep(cg_p_kernel<float>, gseg, kThreads, s, (const long long*)D.seg_dof, D.bps, (const double*)D.partial, D.bps,
            D.scal, first, (const float*)D.z32, D.p);
   }
   CDG_CHECK_LAUNCH(h, "cg");
@@ -2195,14 +2223,14 @@ int dev_solve(cdg_handle* h, const double* f_q, const double* gD, const double* 
   cudaMemsetAsync(D.pv_err, 0, sizeof(int), s);
   // right-hand side in tree order
   if (b_user) {
-    launch(permute_kernel, vec_grid(n), kThreads, s, (int)D.ne, D.np, D.perm0, b_user, D.bt, 1);
+    launch_dep(permute_kernel, vec_grid(n), kThreads, s, (int)D.ne, D.np, D.perm0, b_user, D.bt, 1);
   } else if ((rc = dev_rhs(h, f_q, gD, gN, D.bt, false, s)) != CDG_OK) {
     return rc;
   }
   // initial guess and residual
   const DevLevel& L0 = D.lev[0];
   if (use_u0) {
-    launch(permute_kernel, vec_grid(n), kThreads, s, (int)D.ne, D.np, D.perm0, u_dev, D.x, 1);
+    launch_dep(permute_kernel, vec_grid(n), kThreads, s, (int)D.ne, D.np, D.perm0, u_dev, D.x, 1);
     level_bsr<double>(D, L0, 1, D.x, D.bt, D.r, o.omega, nullptr, s);
   } else {
     cudaMemsetAsync(D.x, 0, sizeof(double) * n, s);
@@ -2238,7 +2266,7 @@ int dev_solve(cdg_handle* h, const double* f_q, const double* gD, const double* 
       done[0] = status != CDG_ENOCONV;
     }
   } else if (ndone < nseg) {
-    if (D.precision != 0) launch(convert_kernel<double, float>, vec_grid(n), kThreads, s, n, (const double*)D.r, D.r32);
+    if (D.precision != 0) launch_dep(convert_kernel<double, float>, vec_grid(n), kThreads, s, n, (const double*)D.r, D.r32);
     if ((rc = cg_direction(h, 1, s)) != CDG_OK) return rc;
     if (o.solve_graph && o.maxit > 0 && !D.gsolve && !D.gsolve_failed && capture_solve(h) != CDG_OK) {
       D.gsolve_failed = true;   // refused by this driver: keep the host-driven loop
@@ -2317,7 +2345,7 @@ int dev_solve(cdg_handle* h, const double* f_q, const double* gD, const double* 
       g_launches.fetch_add(D.g2_kernels, std::memory_order_relaxed);
     }
   }
-  launch(permute_kernel, vec_grid(n), kThreads, s, (int)D.ne, D.np, D.perm0, D.x, u_dev, 0);
+  launch_dep(permute_kernel, vec_grid(n), kThreads, s, (int)D.ne, D.np, D.perm0, D.x, u_dev, 0);
   if (host_ptrs) cudaMemcpyAsync(u, D.u_stage, sizeof(double) * n, cudaMemcpyDeviceToHost, s);
   int pv_err = 0;
   cudaMemcpyAsync(&pv_err, D.pv_err, sizeof(int), cudaMemcpyDeviceToHost, s);
@@ -2347,13 +2375,13 @@ int dev_adjoint(cdg_handle* h, int what, const double* lam_user, const double* u
   cudaStream_t s = (cudaStream_t)stream;
   const size_t n = (size_t)D.ndofs;
   // lambda (and u) to tree order in the CG work vectors (free outside a solve)
-  launch(permute_kernel, vec_grid(n), kThreads, s, (int)D.ne, D.np, D.perm0, lam_user, D.r, 1);
+  launch_dep(permute_kernel, vec_grid(n), kThreads, s, (int)D.ne, D.np, D.perm0, lam_user, D.r, 1);
   if (what == 0) {
     const size_t tot = (size_t)D.ne * D.nq;
     CDG_NP_DISPATCH(D.np, launch(rhs_adjoint_kernel<NP>, (unsigned)((tot + 255) / 256), 256, s, (int)D.ne, D.nq,
                                  D.perm0, D.rhs_vol, D.r, out));
   } else {
-    launch(permute_kernel, vec_grid(n), kThreads, s, (int)D.ne, D.np, D.perm0, u_user, D.z, 1);
+    launch_dep(permute_kernel, vec_grid(n), kThreads, s, (int)D.ne, D.np, D.perm0, u_user, D.z, 1);
     CDG_NP_DISPATCH(D.np, launch(kappa_grad_kernel<NP>, rows_grid(D.ne, D.np), kThreads, s, (int)D.ne, D.nfq,
                                  D.perm0, D.dk_own, D.dk_ptr, D.dk_nbr, D.dk_blk, D.kappa, D.r, D.z, D.rhs_bptr,
                                  D.rhs_bface, D.rhs_bdata, D.btag, gD, out));

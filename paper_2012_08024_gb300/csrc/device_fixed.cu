@@ -57,8 +57,10 @@ __global__ void __launch_bounds__(kFxThreads, fx_ctas_per_sm(NP)) fx_kernel(cons
   const int packs = WPR ? q.n : (q.n + P::RPW - 1) / P::RPW;
   const int stride = gridDim.x * kFxWarps;
   double dsum = 0.0;
+  bool waited = false;
   for (int pack = blockIdx.x * kFxWarps + (threadIdx.x >> 5); pack < packs; pack += stride)
-    dsum = fx_pack<NP, MODE, WPR, false>(q, pack, digits[threadIdx.x >> 5], dsum);
+    dsum = fx_pack<NP, MODE, WPR, false>(q, pack, digits[threadIdx.x >> 5], dsum, waited);
+  if (!waited) cdgk::wait_for_inputs();   // a warp without rows
   if constexpr (MODE == 0 || MODE == 3)
     if (q.dot) {
       __shared__ double red[kFxThreads];
@@ -124,11 +126,10 @@ unsigned go(const FxOp& o, cudaStream_t s, bool launch) {
   if (!launch) return g;
   if (wpr) {
     if constexpr (!fx_one(MODE) && 32 / NP > 1)
-      fx_kernel<NP, MODE, true><<<g, kFxThreads, 0, s>>>(o);
+      launch_dep(fx_kernel<NP, MODE, true>, g, kFxThreads, s, o);
   } else {
-    fx_kernel<NP, MODE, false><<<g, kFxThreads, 0, s>>>(o);
+    launch_dep(fx_kernel<NP, MODE, false>, g, kFxThreads, s, o);
   }
-  count_launch();
   return g;
 }
 

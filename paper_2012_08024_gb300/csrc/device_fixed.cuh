@@ -6,6 +6,7 @@
 #include <cuda_runtime.h>
 
 #include "device_fixed.h"
+#include "device_kernels.cuh"
 
 namespace fx {
 
@@ -149,7 +150,9 @@ __device__ __forceinline__ double finish(double acc, size_t o, double xo, double
 }
 
 template <bool COHERENT>
-__device__ __forceinline__ double vload(const double* p) { return COHERENT ? __ldcg(p) : *p; }
+__device__ __forceinline__ double vload(const double* p) {
+  return cdgk::ld<COHERENT ? cdgk::kCoherent : cdgk::kPlain>(p);
+}
 
 // digits of one warp's gathered values in shared memory
 template <int NP, int MODE, bool WPR>
@@ -167,9 +170,11 @@ struct Pack {
 // rowptr): 4 y += acc; 6 y = acc, y2 = omega acc; 7 y = acc.  Returns the dot partial of modes 0 and 3.
 // q.cols: the rows' columns, q.width of them per row (missing: -1), so that the gathers of x need not
 // wait for the row pointer; one-block modes meet element cols[K] (nullptr: K).
-// COHERENT: vectors are read through L2 only (written earlier in the same kernel).
+// COHERENT: vectors are read through L2 only (written earlier in the same kernel).  waited: whether the
+// kernel has passed wait_for_inputs; the first pack's row pointers, columns and digits are read before.
 template <int NP, int MODE, bool WPR, bool COHERENT>
-__device__ __forceinline__ double fx_pack(const FxOp& q, int pack, int2* __restrict__ digits, double dsum) {
+__device__ __forceinline__ double fx_pack(const FxOp& q, int pack, int2* __restrict__ digits, double dsum,
+                                          bool& waited) {
   using P = Pack<NP, MODE, WPR>;
   constexpr int RPW = P::RPW, CH = P::CH, SPL = P::SPL;
   constexpr bool ONE = P::ONE;
@@ -198,29 +203,37 @@ __device__ __forceinline__ double fx_pack(const FxOp& q, int pack, int2* __restr
   const size_t o = (size_t)K * NP + i;
   const int ea = active ? __ldg(q.EA + o) : 0;
   double xo = 0.0, bo = 0.0;                       // the epilogue's operands, on their way early
-  if (writes) {
-    if constexpr (MODE == 4) xo = vload<COHERENT>(q.y + o);
-    if constexpr (MODE == 1 || MODE == 3) bo = vload<COHERENT>(q.b + o);
-  }
+  auto inputs = [&]() {
+    if (!waited) cdgk::wait_for_inputs();
+    waited = true;
+    if (writes) {
+      if constexpr (MODE == 4) xo = vload<COHERENT>(q.y + o);
+      if constexpr (MODE == 1 || MODE == 3) bo = vload<COHERENT>(q.b + o);
+    }
+  };
+  if (maxc == 0) inputs();
   for (int base = 0; base < maxc; base += CH) {
+    int J[CH];
     double xv[CH];
     int em = 0;
     DigitRow<NP> row;
 #pragma unroll
     for (int c = 0; c < CH; ++c) {
       const int t = base + c;
-      int J = -1;
+      J[c] = -1;
       if constexpr (ONE) {
-        if (active) J = q.cols ? __ldg(q.cols + K) : K;
+        if (active) J[c] = q.cols ? __ldg(q.cols + K) : K;
       } else if (q.cols) {
         const int tt = WPR ? sub + t * SPL : t;
-        if (active && tt < q.width) J = __ldg(q.cols + (size_t)K * q.width + tt);
+        if (active && tt < q.width) J[c] = __ldg(q.cols + (size_t)K * q.width + tt);
       } else if (t < cnt) {
-        J = first + t * SPL;
+        J[c] = first + t * SPL;
       }
-      xv[c] = J >= 0 ? vload<COHERENT>(q.x + (size_t)J * NP + i) : 0.0;
     }
     if (base < cnt) row.load(A + (size_t)(first + base * SPL) * NP * NP, i);
+    if (base == 0) inputs();
+#pragma unroll
+    for (int c = 0; c < CH; ++c) xv[c] = J[c] >= 0 ? vload<COHERENT>(q.x + (size_t)J[c] * NP + i) : 0.0;
 #pragma unroll
     for (int c = 0; c < CH; ++c) em = max(em, biased_exponent(xv[c]));
     em = max(1, __reduce_max_sync(0xffffffffu, em));

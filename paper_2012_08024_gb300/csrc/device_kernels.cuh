@@ -6,6 +6,16 @@
 #include <cuda_runtime.h>
 
 namespace cdgk {
+// Programmatic dependent launch: a kernel launched with launch_dep may start while the kernel before it
+// in the stream still runs.  Before this it may only read what no kernel of a solve writes (row
+// pointers, columns, matrix blocks); every thread passes here before it reads or writes anything else,
+// or returns: the wait ends when all earlier kernels are complete and their writes visible.  Then the
+// next kernel may start in the same way.
+__device__ __forceinline__ void wait_for_inputs() {
+  asm volatile("griddepcontrol.wait;" ::: "memory");
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+}
+
 template <typename T>
 __device__ __forceinline__ T ldg(const T* p) { return __ldg(p); }
 
@@ -59,51 +69,86 @@ __device__ __forceinline__ TO cvt(TI v) {
   else return (TO)v;
 }
 
-// NP consecutive values of x as aligned vector loads; CG: through L2 only
-// (ld.global.cg: coherent within a kernel whose own phases write x), else
-// through the read-only path
-template <typename T, int NP, bool CG = false>
+// How vector values are read: kReadOnly (ld.global.nc) for what nothing writes while the kernel is
+// resident; kPlain for what the kernel before may still be writing when this one starts
+// (wait_for_inputs); kCoherent through L2 only, for what other CTAs of the same kernel write.
+enum Access { kReadOnly, kPlain, kCoherent };
+
+template <Access A>
+__device__ __forceinline__ float ld(const float* p) {
+  if constexpr (A == kReadOnly) return __ldg(p);
+  if constexpr (A == kCoherent) return __ldcg(p);
+  float v;
+  asm volatile("ld.global.f32 %0, [%1];" : "=f"(v) : "l"(p));
+  return v;
+}
+template <Access A>
+__device__ __forceinline__ double ld(const double* p) {
+  if constexpr (A == kReadOnly) return __ldg(p);
+  if constexpr (A == kCoherent) return __ldcg(p);
+  double v;
+  asm volatile("ld.global.f64 %0, [%1];" : "=d"(v) : "l"(p));
+  return v;
+}
+template <Access A>
+__device__ __forceinline__ float2 ld(const float2* p) {
+  if constexpr (A == kReadOnly) return __ldg(p);
+  if constexpr (A == kCoherent) return __ldcg(p);
+  float2 v;
+  asm volatile("ld.global.v2.f32 {%0, %1}, [%2];" : "=f"(v.x), "=f"(v.y) : "l"(p));
+  return v;
+}
+template <Access A>
+__device__ __forceinline__ double2 ld(const double2* p) {
+  if constexpr (A == kReadOnly) return __ldg(p);
+  if constexpr (A == kCoherent) return __ldcg(p);
+  double2 v;
+  asm volatile("ld.global.v2.f64 {%0, %1}, [%2];" : "=d"(v.x), "=d"(v.y) : "l"(p));
+  return v;
+}
+
+// NP consecutive values as aligned vector loads
+template <typename T, int NP, Access A = kReadOnly>
 struct VecLoad;
-template <int NP, bool CG>
-struct VecLoad<float, NP, CG> {
+template <int NP, Access A>
+struct VecLoad<float, NP, A> {
   static __device__ __forceinline__ void load(const float* p, float* v) {
     if constexpr (NP % 2 == 0) {
 #pragma unroll
       for (int j = 0; j < NP; j += 2) {
-        const float2 t = CG ? __ldcg(reinterpret_cast<const float2*>(p + j)) : __ldg(reinterpret_cast<const float2*>(p + j));
+        const float2 t = ld<A>(reinterpret_cast<const float2*>(p + j));
         v[j] = t.x;
         v[j + 1] = t.y;
       }
     } else {
 #pragma unroll
-      for (int j = 0; j < NP; ++j) v[j] = CG ? __ldcg(p + j) : __ldg(p + j);
+      for (int j = 0; j < NP; ++j) v[j] = ld<A>(p + j);
     }
   }
 };
-template <int NP, bool CG>
-struct VecLoad<double, NP, CG> {
+template <int NP, Access A>
+struct VecLoad<double, NP, A> {
   static __device__ __forceinline__ void load(const double* p, double* v) {
     if constexpr (NP % 2 == 0) {
 #pragma unroll
       for (int j = 0; j < NP; j += 2) {
-        const double2 t =
-            CG ? __ldcg(reinterpret_cast<const double2*>(p + j)) : __ldg(reinterpret_cast<const double2*>(p + j));
+        const double2 t = ld<A>(reinterpret_cast<const double2*>(p + j));
         v[j] = t.x;
         v[j + 1] = t.y;
       }
     } else {
 #pragma unroll
-      for (int j = 0; j < NP; ++j) v[j] = CG ? __ldcg(p + j) : __ldg(p + j);
+      for (int j = 0; j < NP; ++j) v[j] = ld<A>(p + j);
     }
   }
 };
 
 // Row i of (A x)_K for block row K: sum over the blocks of the row, block by
 // block and column by column (the same order for every UNR).
-// COHERENT: x is read through L2 only (x may have been written earlier in the same kernel).
 template <typename T, int NP, bool VEC, int UNR, bool COHERENT = false>
 __device__ __forceinline__ T row_acc(int K, int i, const int* __restrict__ rowptr, const int* __restrict__ col,
                                      const T* __restrict__ A, const T* __restrict__ x) {
+  constexpr Access X = COHERENT ? kCoherent : kPlain;
   T acc = T(0);
   const int b0 = rowptr[K], b1 = rowptr[K + 1];
   if constexpr (VEC) {
@@ -117,7 +162,7 @@ __device__ __forceinline__ T row_acc(int K, int i, const int* __restrict__ rowpt
       for (int u = 0; u < UNR; ++u) {
         const int J = ldg(col + bb + u);
         VecLoad<T, NP>::load(A + (size_t)(bb + u) * NP * NP + i * NP, av[u]);
-        VecLoad<T, NP, COHERENT>::load(x + (size_t)J * NP, xv[u]);
+        VecLoad<T, NP, X>::load(x + (size_t)J * NP, xv[u]);
       }
 #pragma unroll
       for (int u = 0; u < UNR; ++u)
@@ -127,7 +172,7 @@ __device__ __forceinline__ T row_acc(int K, int i, const int* __restrict__ rowpt
     for (; bb < b1; ++bb) {
       T av[NP], xv[NP];
       VecLoad<T, NP>::load(A + (size_t)bb * NP * NP + i * NP, av);
-      VecLoad<T, NP, COHERENT>::load(x + (size_t)ldg(col + bb) * NP, xv);
+      VecLoad<T, NP, X>::load(x + (size_t)ldg(col + bb) * NP, xv);
 #pragma unroll
       for (int j = 0; j < NP; ++j) acc = fma(av[j], xv[j], acc);
     }
@@ -136,7 +181,7 @@ __device__ __forceinline__ T row_acc(int K, int i, const int* __restrict__ rowpt
       const T* a = A + (size_t)bb * NP * NP + i * NP;
       const T* xj = x + (size_t)ldg(col + bb) * NP;
 #pragma unroll
-      for (int j = 0; j < NP; ++j) acc = fma(ldg(a + j), COHERENT ? __ldcg(xj + j) : ldg(xj + j), acc);
+      for (int j = 0; j < NP; ++j) acc = fma(ldg(a + j), ld<X>(xj + j), acc);
     }
   }
   return acc;
@@ -179,6 +224,7 @@ template <typename T, int NP, bool COHERENT = false>
 __device__ __forceinline__ T split_row_acc(int K, const int* __restrict__ rowptr, const int* __restrict__ col,
                                            const T* __restrict__ A, const T* __restrict__ x) {
   constexpr int G = 32 / NP;
+  constexpr Access X = COHERENT ? kCoherent : kPlain;
   const int lane = threadIdx.x & 31;
   const int sub = lane / NP, i = lane - sub * NP;
   T acc = T(0);
@@ -190,7 +236,7 @@ __device__ __forceinline__ T split_row_acc(int K, const int* __restrict__ rowptr
 #pragma unroll
       for (int u = 0; u < 2; ++u) {
         VecLoad<T, NP>::load(A + (size_t)(bb + u * G) * NP * NP + i * NP, av[u]);
-        VecLoad<T, NP, COHERENT>::load(x + (size_t)ldg(col + bb + u * G) * NP, xv[u]);
+        VecLoad<T, NP, X>::load(x + (size_t)ldg(col + bb + u * G) * NP, xv[u]);
       }
 #pragma unroll
       for (int u = 0; u < 2; ++u)
@@ -200,7 +246,7 @@ __device__ __forceinline__ T split_row_acc(int K, const int* __restrict__ rowptr
     if (bb < b1) {
       T av[NP], xv[NP];
       VecLoad<T, NP>::load(A + (size_t)bb * NP * NP + i * NP, av);
-      VecLoad<T, NP, COHERENT>::load(x + (size_t)ldg(col + bb) * NP, xv);
+      VecLoad<T, NP, X>::load(x + (size_t)ldg(col + bb) * NP, xv);
 #pragma unroll
       for (int j = 0; j < NP; ++j) acc = fma(av[j], xv[j], acc);
     }
@@ -214,12 +260,26 @@ __device__ __forceinline__ T split_row_acc(int K, const int* __restrict__ rowptr
   return acc;
 }
 
+// Brings the first blocks that the warp will multiply, and their columns, towards it (split_row_acc).
+template <typename T, int NP>
+__device__ __forceinline__ void touch_row(int K, const int* __restrict__ rowptr, const int* __restrict__ col,
+                                          const T* __restrict__ A) {
+  constexpr int G = 32 / NP;
+  const int lane = threadIdx.x & 31;
+  const int bb = ldg(rowptr + K) + lane / NP;
+  if (lane / NP < G && bb < ldg(rowptr + K + 1)) {
+    asm volatile("prefetch.global.L1 [%0];" ::"l"(col + bb));
+    asm volatile("prefetch.global.L1 [%0];" ::"l"(A + (size_t)bb * NP * NP + (lane % NP) * NP));
+  }
+}
+
 // The sum over the children K of agglomerate Ag of (L_K^T r_K)_i, its children shared by the groups
 // of the warp in the same way; valid in the lanes of group 0.
 template <typename T, int NP, bool COHERENT = false>
 __device__ __forceinline__ T split_restrict(int Ag, const int* __restrict__ childptr, const T* __restrict__ L,
                                             const T* __restrict__ r) {
   constexpr int G = 32 / NP;
+  constexpr Access X = COHERENT ? kCoherent : kPlain;
   const int lane = threadIdx.x & 31;
   const int sub = lane / NP, i = lane - sub * NP;
   T acc = T(0);
@@ -229,7 +289,7 @@ __device__ __forceinline__ T split_restrict(int Ag, const int* __restrict__ chil
       const T* LK = L + (size_t)K * NP * NP + i;
       const T* rk = r + (size_t)K * NP;
 #pragma unroll
-      for (int j = 0; j < NP; ++j) acc = fma(ldg(LK + j * NP), COHERENT ? __ldcg(rk + j) : ldg(rk + j), acc);
+      for (int j = 0; j < NP; ++j) acc = fma(ldg(LK + j * NP), ld<X>(rk + j), acc);
     }
   }
 #pragma unroll

@@ -194,11 +194,12 @@ __device__ __forceinline__ void fx_phase(const FxOp* op) {
   extern __shared__ __align__(16) int2 warp_digits[];   // [warps][most_digits]
   int2* digits = warp_digits + (threadIdx.x >> 5) * most_digits<NP>();
   const FxOp q = *op;   // into registers
+  bool waited = true;   // an ordinary launch
   constexpr int RPW = fx::Pack<NP, MODE, WPR>::RPW;
   const int packs = WPR ? q.n : (q.n + RPW - 1) / RPW;
   const int warps = (int)(gridDim.x * (blockDim.x >> 5));
   for (int p = (int)(blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5)); p < packs; p += warps)
-    fx::fx_pack<NP, MODE, WPR, true>(q, p, digits, 0.0);
+    fx::fx_pack<NP, MODE, WPR, true>(q, p, digits, 0.0, waited);
 }
 
 template <int NP, int MODE>

@@ -175,6 +175,23 @@ float time_calls(cudaStream_t s, cudaEvent_t e0, cudaEvent_t e1, int reps, F&& f
 void count_launch(long long n = 1);
 long long launch_count();
 
+// Launches a kernel that calls cdgk::wait_for_inputs (programmatic dependent launch): its start, and what
+// it reads before that call, overlaps the end of the kernel before it.
+template <typename... KArgs, typename... Args>
+inline void launch_dep(void (*k)(KArgs...), dim3 g, dim3 b, cudaStream_t s, Args... args) {
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = g;
+  cfg.blockDim = b;
+  cfg.stream = s;
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[0].val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = 1;
+  cudaLaunchKernelEx(&cfg, k, KArgs(args)...);
+  count_launch();
+}
+
 // device.cu, for the GMRES driver: one V-cycle z = M^{-1} r on level-0 vectors;
 // y = A_0 x (mode 0) or y = b - A_0 x (mode 1) on 256-byte aligned tree-order
 // vectors; a level-0 dot into the CG scalars (dot_to's `which`); CUDA error text
