@@ -265,8 +265,8 @@ size_t layout(const cdg::Hierarchy& H, int precision, int nrhs, DeviceState* S, 
 template <typename T, int NP, int MODE, bool VEC, int UNR = 1>
 __global__ void __launch_bounds__(kThreads, 8 / UNR) bsr_kernel(int n, const int* __restrict__ rowptr,
                                                        const int* __restrict__ col, const T* __restrict__ A,
-                                                       const T* __restrict__ Dinv, const T* __restrict__ x,
-                                                       const T* __restrict__ b, T* __restrict__ y, T omega,
+                                                       const T* __restrict__ Dinv, const T* x,
+                                                       const T* b, T* __restrict__ y, T omega,
                                                        double* __restrict__ dot) {
   cdgk::wait_for_inputs();
   constexpr int RPW = 32 / NP;
@@ -428,7 +428,7 @@ constexpr int kRowThreads = 128;
 template <typename T, int NP, int MODE>
 __global__ void __launch_bounds__(kRowThreads) bsr_row_kernel(int n, const int* __restrict__ rowptr,
                                                               const int* __restrict__ col, const T* __restrict__ A,
-                                                              const T* __restrict__ x, const T* __restrict__ b,
+                                                              const T* x, const T* b,
                                                               T* __restrict__ y, T omega) {
   const int K = blockIdx.x * (kRowThreads / 32) + (threadIdx.x >> 5);
   if (K < n) cdgk::touch_row<T, NP>(K, rowptr, col, A);
@@ -445,7 +445,7 @@ __global__ void __launch_bounds__(kRowThreads) bsr_row_kernel(int n, const int* 
 
 template <typename T, int NP>
 __global__ void __launch_bounds__(kRowThreads) restrict_row_kernel(int nc, const int* __restrict__ childptr,
-                                                                   const T* __restrict__ L, const T* __restrict__ r,
+                                                                   const T* __restrict__ L, const T* r,
                                                                    T* __restrict__ bc) {
   cdgk::wait_for_inputs();
   const int Ag = blockIdx.x * (kRowThreads / 32) + (threadIdx.x >> 5);
@@ -458,7 +458,7 @@ __global__ void __launch_bounds__(kRowThreads) restrict_row_kernel(int nc, const
 // bh = Dinv b; with WRITE_X also x = omega bh (first smoothing step from a zero guess)
 template <typename T, int NP, bool WRITE_X>
 __global__ void __launch_bounds__(kThreads) smooth_first_kernel(int n, const T* __restrict__ Dinv,
-                                                                const T* __restrict__ b, T* __restrict__ bh,
+                                                                const T* b, T* __restrict__ bh,
                                                                 T* __restrict__ x, T omega) {
   cdgk::wait_for_inputs();
   constexpr int RPW = 32 / NP;
@@ -480,7 +480,7 @@ __global__ void __launch_bounds__(kThreads) smooth_first_kernel(int n, const T* 
 // bc[A] = sum over children K of L_K^T r[K]
 template <typename T, int NP>
 __global__ void __launch_bounds__(kThreads) restrict_kernel(int nc, const int* __restrict__ childptr,
-                                                            const T* __restrict__ L, const T* __restrict__ r,
+                                                            const T* __restrict__ L, const T* r,
                                                             T* __restrict__ bc) {
   cdgk::wait_for_inputs();
   constexpr int RPW = 32 / NP;
@@ -503,7 +503,7 @@ __global__ void __launch_bounds__(kThreads) restrict_kernel(int nc, const int* _
 // x[K] (+)= L_K xc[parent K]
 template <typename T, int NP, bool ADD>
 __global__ void __launch_bounds__(kThreads) prolong_kernel(int n, const int* __restrict__ parent,
-                                                           const T* __restrict__ L, const T* __restrict__ xc,
+                                                           const T* __restrict__ L, const T* xc,
                                                            T* __restrict__ x) {
   cdgk::wait_for_inputs();
   constexpr int RPW = 32 / NP;
@@ -528,7 +528,7 @@ __global__ void __launch_bounds__(kThreads) prolong_kernel(int n, const int* __r
 template <typename TI, typename TO, bool ADD = false>
 __global__ void coarse_kernel(int nc, const int* __restrict__ crow_seg, const int* __restrict__ crow_off,
                               const long long* __restrict__ cinv_off, const double* __restrict__ Ainv,
-                              const TI* __restrict__ b, TO* __restrict__ x) {
+                              const TI* b, TO* __restrict__ x) {
   const int row = (int)((blockIdx.x * (size_t)blockDim.x + threadIdx.x) >> 5);
   const int lane = threadIdx.x & 31;
   if (row >= nc) {
@@ -561,7 +561,7 @@ __global__ void coarse_kernel(int nc, const int* __restrict__ crow_seg, const in
 // writes them with zero higher coefficients.
 template <typename T>
 __global__ void __launch_bounds__(kThreads) ptrunc_restrict_kernel(int n, int npf, int npc,
-                                                                   const T* __restrict__ r, T* __restrict__ bc) {
+                                                                   const T* r, T* __restrict__ bc) {
   cdgk::wait_for_inputs();
   const size_t tot = (size_t)n * npc;
   for (size_t t = blockIdx.x * (size_t)blockDim.x + threadIdx.x; t < tot; t += (size_t)gridDim.x * blockDim.x) {
@@ -572,7 +572,7 @@ __global__ void __launch_bounds__(kThreads) ptrunc_restrict_kernel(int n, int np
 
 template <typename T, bool ADD>
 __global__ void __launch_bounds__(kThreads) ptrunc_prolong_kernel(int n, int npf, int npc,
-                                                                  const T* __restrict__ xc, T* __restrict__ x) {
+                                                                  const T* xc, T* __restrict__ x) {
   cdgk::wait_for_inputs();
   const size_t tot = (size_t)n * npf;
   for (size_t t = blockIdx.x * (size_t)blockDim.x + threadIdx.x; t < tot; t += (size_t)gridDim.x * blockDim.x) {
@@ -584,7 +584,7 @@ __global__ void __launch_bounds__(kThreads) ptrunc_prolong_kernel(int n, int npf
 }
 
 template <typename TI, typename TO>
-__global__ void convert_kernel(size_t n, const TI* __restrict__ a, TO* __restrict__ b) {
+__global__ void convert_kernel(size_t n, const TI* a, TO* __restrict__ b) {
   cdgk::wait_for_inputs();
   for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < n; i += (size_t)gridDim.x * blockDim.x)
     b[i] = cvt<TO>(a[i]);
@@ -613,7 +613,7 @@ __device__ __forceinline__ void seg_range(const long long* __restrict__ seg_dof,
 // partial[blk] = sum x.y over the block's chunk; Y is FP64, or FP32 (the V-cycle's output, widened exactly)
 template <typename TY>
 __global__ void __launch_bounds__(kThreads) dot_kernel(const long long* __restrict__ seg_dof, int bps,
-                                                       const double* __restrict__ x, const TY* __restrict__ y,
+                                                       const double* x, const TY* y,
                                                        double* __restrict__ partial) {
   cdgk::wait_for_inputs();
   int seg;
@@ -665,7 +665,7 @@ __device__ __forceinline__ double partials_sum(const double* __restrict__ p, int
 // CTAs read: r.z goes to S_RZN and moves on to S_RZ in the next update.
 
 // One CTA per segment: ||b||^2 (which 3) or the first ||r||^2 (4) from its cnt partials.
-__global__ void finalize_kernel(const double* __restrict__ partial, int cnt, int which, double tol,
+__global__ void finalize_kernel(const double* partial, int cnt, int which, double tol,
                                 double* __restrict__ scal) {
   cdgk::wait_for_inputs();
   const double tot = partials_sum(partial + (size_t)blockIdx.x * cnt, cnt);
@@ -690,11 +690,11 @@ __global__ void finalize_kernel(const double* __restrict__ partial, int cnt, int
 // also r32, the copy of r it reads, and (npart further) the partial of r times its last output z.
 template <bool FLEX>
 __global__ void __launch_bounds__(kThreads) cg_update_kernel(const long long* __restrict__ seg_dof, int bps,
-                                                             const double* __restrict__ pq, int pq_cnt,
-                                                             double* __restrict__ scal, const double* __restrict__ p,
-                                                             const double* __restrict__ q, double* __restrict__ x,
+                                                             const double* pq, int pq_cnt,
+                                                             double* __restrict__ scal, const double* p,
+                                                             const double* q, double* __restrict__ x,
                                                              double* __restrict__ r, float* __restrict__ r32,
-                                                             const float* __restrict__ z,
+                                                             const float* z,
                                                              double* __restrict__ partial, int npart) {
   cdgk::wait_for_inputs();
   int seg;
@@ -774,11 +774,11 @@ __global__ void hist_init_kernel(int nseg, double* __restrict__ scal) {
 constexpr int kCheckThreads = 512;
 
 __global__ void __launch_bounds__(kCheckThreads) cg_check_kernel(cudaGraphConditionalHandle cond, int in_graph,
-                                                                 int nseg, int bps, const double* __restrict__ partial,
+                                                                 int nseg, int bps, const double* partial,
                                                                  int npart, int flexible, double tol, int maxit,
                                                                  double* __restrict__ scal, int* __restrict__ it_dev,
                                                                  double* __restrict__ hist, int* __restrict__ iters,
-                                                                 const int* __restrict__ wait_err) {
+                                                                 const int* wait_err) {
   cdgk::wait_for_inputs();
   const int it = in_graph ? *it_dev + 1 : 0;
   int open = 0;
@@ -839,9 +839,9 @@ __global__ void __launch_bounds__(kCheckThreads) cg_check_kernel(cudaGraphCondit
 // (then the flexible, Polak-Ribiere beta).  A segment that is done gets beta = 0.
 template <typename TZ>
 __global__ void __launch_bounds__(kThreads) cg_p_kernel(const long long* __restrict__ seg_dof, int bps,
-                                                        const double* __restrict__ rzp, int rz_cnt,
+                                                        const double* rzp, int rz_cnt,
                                                         double* __restrict__ scal, int first,
-                                                        const TZ* __restrict__ z, double* __restrict__ p) {
+                                                        const TZ* z, double* __restrict__ p) {
   cdgk::wait_for_inputs();
   int seg;
   size_t lo, hi;
@@ -912,7 +912,7 @@ __global__ void __launch_bounds__(kThreads) rhs_kernel(int ne, int nq, int nfq, 
   b[(size_t)(user_out ? K : k) * NP + i] = s;
 }
 
-__global__ void permute_kernel(int ne, int np, const int* __restrict__ perm0, const double* __restrict__ in,
+__global__ void permute_kernel(int ne, int np, const int* __restrict__ perm0, const double* in,
                                double* __restrict__ out, int to_tree) {
   cdgk::wait_for_inputs();
   const size_t n = (size_t)ne * np;

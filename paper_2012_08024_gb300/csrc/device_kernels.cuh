@@ -10,7 +10,8 @@ namespace cdgk {
 // in the stream still runs.  Before this it may only read what no kernel of a solve writes (row
 // pointers, columns, matrix blocks); every thread passes here before it reads or writes anything else,
 // or returns: the wait ends when all earlier kernels are complete and their writes visible.  Then the
-// next kernel may start in the same way.
+// next kernel may start in the same way.  What an earlier kernel writes is not read-only for the life of
+// this one: its pointers carry no __restrict__, which would let the compiler take the read-only path.
 __device__ __forceinline__ void wait_for_inputs() {
   asm volatile("griddepcontrol.wait;" ::: "memory");
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
