@@ -53,12 +53,12 @@ HBM_FALLBACK_GBS = 6800.0           # profiling-recipe fallback when no measured
 # x 2 flops x 2.07 GHz; the roofline divides by the rate the FMA probe measures in the same run
 FP64_DERIVED_TFLOPS = 152 * 2 * 2 * 2.07e9 / 1e12
 # DRAM bytes (read + write) of one level-0 apply as ncu captured them on the 256 x 256 p = 3
-# square (523,264 blocks): FP64 443,725,568 (profiles/bsr_kernel_tri256_p3_fp64.md), FP32
+# square (523,264 blocks): FP64 not captured since its kernel changed, FP32
 # 223,440,896 (profiles/bsr_kernel_tri256_p3_fp32.md).  Other squares at p = 3 report them scaled by
 # their level-0 block count (the traffic is 1.003-1.005x the algorithmic bytes, which grow with
-# the blocks); other workloads report null.  Set to None whenever bsr_kernel changes, until it is
+# the blocks); other workloads report null.  Set to None whenever the kernel changes, until it is
 # captured again.
-CAPTURED_APPLY = {"blocks": 523_264, "fp64": 443_725_568, "fp32": 223_440_896}
+CAPTURED_APPLY = {"blocks": 523_264, "fp64": None, "fp32": 223_440_896}
 
 
 def apply_traffic(kind, p, nnzb0, dtype):
@@ -615,7 +615,9 @@ def main():
     k_us = e0.elapsed_time(e1) / reps * 1e3
     nnzb0 = S.info["nnzb_l"][0]
     npb = S.np_
-    alg_bytes = nnzb0 * npb * npb * 8 + nnzb0 * 4 + (S.ne + 1) * 4 + 2 * ndof * 8
+    # digits of the blocks, padded columns (dim + 2 per row), row pointers, row exponents, x and y
+    alg_bytes = (nnzb0 * npb * npb * 8 + S.ne * (S.info["dim"] + 2) * 4 + (S.ne + 1) * 4 + S.ne * npb * 4 +
+                 2 * ndof * 8)
     achieved = alg_bytes / (k_us * 1e-6) / 1e9
     peak, peak_src = peaks()
     flops = 2.0 * nnzb0 * npb * npb
@@ -723,15 +725,16 @@ def main():
     if not args.no_cpu_baseline and ws == 1:
         cpu = cpu_baseline(kind, p, nu, coarsen=coarsen, pmg=pmg)
     clocks = cs.summary()
+    # the FP64 apply sums exact integer digit products (no FP64 multiply-adds): bytes bound it
     achieved_tf = flops / (k_us * 1e-6) / 1e12
     fp64_peak = fma_peak if fma_peak else FP64_DERIVED_TFLOPS
-    roofline = {"bound": "alu", "achieved": achieved_tf, "peak": fp64_peak, "unit": "TFLOP/s",
-                "frac": achieved_tf / fp64_peak, "traffic": apply_traffic(kind, p, nnzb0, "fp64"),
-                "peak_source": ("measured in this run: FP64 FMA probe (cdg_fp64_fma_probe)" if fma_peak else
-                                "derived: 152 SMs x 2 FP64 FMA/clk x 2 flops x 2.07 GHz"),
-                "peak_derived_tflops": FP64_DERIVED_TFLOPS, "frac_of_derived": achieved_tf / FP64_DERIVED_TFLOPS,
-                "kernel": "level-0 FP64 block-sparse apply (bsr_kernel<double,%d,0,true>)" % npb,
+    roofline = {"bound": "hbm", "achieved": achieved, "peak": peak, "unit": "GB/s",
+                "frac": achieved / peak, "traffic": apply_traffic(kind, p, nnzb0, "fp64"), "peak_source": peak_src,
+                "kernel": "level-0 FP64 block-sparse apply in integer digits (fx_kernel<%d,0>)" % npb,
                 "alg_bytes_per_launch": alg_bytes, "alg_flops_per_launch": flops, "launch_us": k_us,
+                "fp64_equivalent_tflops": achieved_tf, "fp64_fma_peak_tflops": fp64_peak,
+                "fp64_fma_peak_source": ("measured in this run: FP64 FMA probe (cdg_fp64_fma_probe)" if fma_peak else
+                                         "derived: 152 SMs x 2 FP64 FMA/clk x 2 flops x 2.07 GHz"),
                 "hbm_gbs": achieved, "hbm_peak_gbs": peak, "hbm_peak_source": peak_src,
                 "hbm_frac": achieved / peak}
     if mixed:   # the FP32 V-cycle's block-sparse kernel, HBM-bound

@@ -136,7 +136,8 @@ typedef struct {
                                2012); relative truncation below 2^-56 of the row and column
                                scales.  Used where the FP32 sums provably stay exact (blocks per
                                row x n_p x 8 x 127^2 < 2^23), else the FP64 CUDA-core apply.
-                               0 (default): the FP64 CUDA-core apply. */
+                               0 (default): the FP64 apply on CUDA cores, by integer digit
+                               products. */
   int32_t persistent_vcycle; /* 1: each V-cycle is ONE cooperative persistent kernel whose CTAs
                                walk the cycle's phases with grid barriers (bounded waits; an
                                expired wait ends the solve with CDG_ETIMEOUT); used when every
@@ -276,7 +277,7 @@ int cdg_solve_multi(cdg_handle* h, const double* f_q, double* u, double* res_his
 
 /* y = A_0 x for the R columns of a handle created with nrhs = R (tree order,
  * [n_elements][n_p][R] FP64 device vectors), by the method cdg_solve_multi
- * uses (tc_fp64_apply or the FP64 CUDA-core apply); returns when y is
+ * uses (tc_fp64_apply or the integer digit products); returns when y is
  * written.  Errors: CDG_ESTATE, CDG_ETIMEOUT (a tensor-core wait reached its
  * limit), CDG_ECUDA. */
 int cdg_apply_multi(cdg_handle* h, const double* x, double* y, void* stream);
