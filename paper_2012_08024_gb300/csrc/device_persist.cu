@@ -182,7 +182,7 @@ __device__ void ph_coarse(const PParams& P, const T* b, T* x, bool add) {
 // FP64: a product in digit form, by the same packs as the per-phase kernels.  Three CTAs per SM:
 // V-cycle of the 181^2 (p = 2) mesh 324 -> 278 us against FP64 blocks, 32^2 137 -> 121 us, but the
 // 64-mesh batch 63.5 -> 76.6 ms per solve (its phases wait for memory, and 24 warps per SM hide less
-// than the 40 of the FP64-block kernel); two CTAs 265 us, 102 us, 80.3 ms.
+// than the 40 of the FP64-block kernel; 66.4 ms with the later CG kernels); two CTAs 265 us, 102 us, 80.3 ms.
 template <int NP>
 constexpr int most_digits() {
   constexpr int packed = fx::Pack<NP, 8, false>::DIGITS, shared = fx::Pack<NP, 8, true>::DIGITS;
