@@ -35,8 +35,8 @@
 // its packs; the padded column table lets the gathers of x start with the row
 // pointers.  The kernel waits for memory (issue slots a third used), so resident
 // warps count: 64 registers, 32 warps per SM.  Measured, 131,072 rows of 4
-// blocks at n_p = 10: apply 102.7 -> 76.9 us (5.4 TB/s), level of 1,044 rows 12.6
-// -> 4.7 us; 80 registers 84.7 us; digits streamed through shared memory by
+// blocks at n_p = 10: apply 102.7 -> 76.9 us, level of 1,044 rows 12.6 -> 4.7 us
+// (72.7 us, 6.1 TB/s, and 3.2 us with dependent launches); 80 registers 84.7 us; digits streamed through shared memory by
 // cp.async, one or two packs ahead, 85-104 us (fewer warps fit); 48 registers 90 us.
 #include <cuda_runtime.h>
 

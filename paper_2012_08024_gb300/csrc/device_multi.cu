@@ -89,7 +89,7 @@ struct Cols<4> {
 // blocks at once into shared memory; PF starts the gather of the next block's x before the products of
 // this one.  What bounds the kernel is the latency of the x gathers: the CTA-wide form before it, two
 // barriers per block with the gathers behind them, moved its 638 MB (20,000 rows, n_p = 10, R = 256) in
-// 179 us, 0.52 of the copy rate.  V, PF and the warps per CTA are autotuned; every choice sums a
+// 179 us, 0.52 of the copy rate; this one takes 153 us.  V, PF and the warps per CTA are autotuned; every choice sums a
 // column in the same order.
 constexpr int kMrMaxBR = 4;
 constexpr int kMrStage = 4;
@@ -198,7 +198,7 @@ __global__ void __launch_bounds__(128, mr_min_ctas<V, PF>()) mr_row_kernel(int n
 // neighbours (a first pass, which also brings x into the caches), splits its values and keeps the n_p
 // sums in registers; the digits of a block are read from shared memory, each 16 bytes feeding eight
 // integer multiply-adds.  A_0 has at most dim + 2 blocks per row (compact stencil), so its rows need no
-// flush.  5,000 rows, n_p = 6, 40 columns: 82 us with FP64 multiply-adds (46 us at the FP64 rate).
+// flush.  5,000 rows, n_p = 6, 40 columns: 82 us with FP64 multiply-adds (46 us at the FP64 rate), 50 us here.
 template <int NP>
 __global__ void __launch_bounds__(128, 4) mr_fx_kernel(int n, int R, const int* __restrict__ rowptr,
                                                        const int* __restrict__ col, const int2* __restrict__ A,
