@@ -10,10 +10,16 @@
 // 8 bytes as a double),
 //     a = 2^(EA - 58) (ah 2^30 + al),   |ah| <= 2^28,  |al| <= 2^29,
 // with one exponent EA per scalar row, every entry rounded to 2^-59 of the
-// row's power-of-two bound, and the vector values that a warp gathers are split
-// likewise with one exponent for the warp's values.  Four integer multiply-adds
-// give a product of digits exactly, all sums are exact (whatever their order),
-// and one rounding to FP64 ends the row: 16 clocks in the place of 64.  The
+// row's power-of-two bound, and the n_p values of a neighbour's x_J are split
+// likewise with one exponent of their own.  Four integer multiply-adds give a
+// product of digits exactly, the sum over a block is exact, the blocks' sums are
+// brought to the scale of the largest (nothing above 2^-96 of it is lost), and
+// one rounding to FP64 ends the row: 16 clocks in the place of 64.  A row's
+// result depends on the values that it multiplies and on no others: with one
+// exponent for all that a warp gathers, rows of two meshes of a batch shared one,
+// and a mesh with small data beside one with large data got a wrong solution.
+// (The exponents per block cost 2-4%: apply 72.4 -> 74.3 us, V-cycle of the
+// 128^2 (p = 3) mesh 199 -> 207 us, 64 meshes 52.4 -> 54.5 ms.)  The
 // method is the splitting of Ozaki, Ogita, Oishi and Rump (2012) with integer
 // digits.  58 bits, not fewer, since A x cancels for smooth x, where the small
 // constant-mode entries of A meet the largest values of x: on solutions of the
@@ -23,8 +29,7 @@
 //
 // The sums, over the T <= 28 terms of a block: |sum al xl| <= 2^58 T,
 // |sum (ah xl + al xh)| <= 2^58 T; both are then carried into the next higher
-// one, and |sum ah xh| <= 2^56 T over a row stays within 63 bits for T <= 127 (a
-// flush to FP64 in longer rows).
+// one, and |sum ah xh| <= 2^56 T.
 //
 // Mapping: the n_p lanes of a group own the n_p scalar rows of one block row; a
 // lane loads one value of each x_J, splits it and leaves the digits in shared

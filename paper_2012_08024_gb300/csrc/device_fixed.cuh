@@ -10,19 +10,14 @@
 
 namespace fx {
 
-
 constexpr int kFxThreads = 128;
 constexpr int kFxWarps = kFxThreads / 32;
-constexpr int kMaxTerms = 127;
+constexpr int kMaxTerms = 127;        // of one scale, so that their sums stay within 63 bits
 constexpr int kNotFinite = 1 << 20;   // row exponent of a matrix row that holds an infinity or NaN
+constexpr int kNoScale = -(1 << 24);  // scale of an empty sum, below every other
 
-// blocks of a row per step of a group: the level-0 rows of tetrahedra hold five; where
-// all groups of a warp share a row their terms together stay within kMaxTerms
-constexpr int fx_chunk(int np, bool wpr) {
-  const int c = np == 4 || np == 10 || np == 20 ? 5 : 4;
-  const int most = kMaxTerms / (np * (wpr ? 32 / np : 1));
-  return c < most ? c : most;
-}
+// blocks of a row per step of a group: the level-0 rows of tetrahedra hold five
+constexpr int fx_chunk(int np) { return np == 4 || np == 10 || np == 20 ? 5 : 4; }
 constexpr bool fx_one(int mode) { return mode == 4 || mode == 6 || mode == 7; }   // one block per row
 // resident CTAs of 128 threads per SM that the registers are held to
 constexpr int fx_ctas_per_sm(int np) { return np > 10 ? 4 : 8; }
@@ -61,7 +56,34 @@ __device__ __forceinline__ double scale2(double d, int e) {
   return scalbn(d, e);
 }
 
-// A sum of digit products, hi 2^60 + lo with 0 <= lo < 2^60 after carrying
+// hi 2^60 + lo with 0 <= lo < 2^60, in units that its user keeps
+struct Wide {
+  static constexpr unsigned long long kLow = (1ull << 60) - 1;
+  long long hi = 0;
+  unsigned long long lo = 0;
+  // rounded down to a multiple of 2^d and divided by it, d >= 0
+  __device__ __forceinline__ void down(int d) {
+    if (d < 60) {
+      lo = (((unsigned long long)hi << (60 - d)) & kLow) | (lo >> d);
+      hi >>= d;
+    } else {
+      lo = (unsigned long long)(hi >> min(d - 60, 63)) & kLow;
+      hi >>= 63;
+    }
+  }
+  __device__ __forceinline__ void add(const Wide& o) {
+    lo += o.lo;
+    hi += o.hi + (long long)(lo >> 60);
+    lo &= kLow;
+  }
+};
+
+// Bits between the sum of one block's products (below 2^61 units of hi) and a row's sum: the blocks of a
+// row, each at its own scale, are added in units 2^kHead times those of the block of the largest, so
+// that 2^26 terms fit and nothing above 2^-96 of that block's bound is lost.
+constexpr int kHead = 20;
+
+// A sum of digit products of one scale
 struct Acc {
   long long hh = 0, mm = 0, ll = 0;
   // carries of one block's products into the higher sums
@@ -72,9 +94,15 @@ struct Acc {
     mm &= 0x3FFFFFFF;
   }
   __device__ __forceinline__ unsigned long long low() const { return ((unsigned long long)mm << 30) | ll; }
+  __device__ __forceinline__ Wide wide() const {
+    Wide w;
+    w.hi = hh;
+    w.lo = low();
+    return w;
+  }
 };
 
-// (hi 2^60 + lo) 2^(e - 116), rounded once; e = EA + EX of the digits' scales
+// (hi 2^60 + lo) 2^(e - 116), rounded once; e = EA + EX of the digits' scales (+ kHead after Wide::down by it)
 __device__ __forceinline__ double fx_value(long long hi, unsigned long long lo, int e) {
   const int k = min(60, __clzll(hi ^ (hi >> 63)) - 1);   // low bits that fit beside hi in 63 bits
   const long long v = (long long)((unsigned long long)hi << k) | (long long)(lo >> (60 - k));
@@ -159,11 +187,24 @@ template <int NP, int MODE, bool WPR>
 struct Pack {
   static constexpr int RPW = 32 / NP;
   static constexpr bool ONE = fx_one(MODE);
-  static constexpr int CH = ONE ? 1 : fx_chunk(NP, WPR);
+  static constexpr int CH = ONE ? 1 : fx_chunk(NP);
   static constexpr int SPL = WPR ? RPW : 1;                       // groups that share a block row
   static constexpr int GS = CH * NP + 2 + (CH * NP) % 2;          // digits of one group's chunk (padded against bank conflicts)
   static constexpr int DIGITS = RPW * GS;
 };
+
+// The largest of the v of a group's n_p lanes, in each of them; v holds two 16-bit fields, each taken by itself
+template <int NP>
+__device__ __forceinline__ unsigned group_max(unsigned v, int sub, int i) {
+  if constexpr (32 / NP == 1) {
+    return __reduce_max_sync(0xffffffffu, v & 0xFFFFu) | __reduce_max_sync(0xffffffffu, v >> 16) << 16;
+  } else {
+#pragma unroll
+    for (int o = 1; o < NP; o *= 2)   // the maximum over 2, 4, ... lanes from this one on, around the group
+      v = __vmaxu2(v, __shfl_sync(0xffffffffu, v, sub * NP + (i + o < NP ? i + o : i + o - NP)));
+    return v;
+  }
+}
 
 // One warp on one pack of rows: acc = (A x)_(K, i), then by MODE: 0 y = acc; 1 y = b - acc;
 // 3 y = x + omega (b - x - acc); 8 y = acc, block t meeting element t; with one block per row (no
@@ -195,10 +236,9 @@ __device__ __forceinline__ double fx_pack(const FxOp& q, int pack, int2* __restr
   const int cnt = !active ? 0 : WPR ? (nb - sub + SPL - 1) / SPL : nb;
   const int first = WPR ? b0 + sub : b0;
   const int maxc = __reduce_max_sync(0xffffffffu, cnt);
-  Acc sum;
-  int ex = 0, terms = 0;                           // running exponent field of the x digits, terms summed
-  double flushed = 0.0;
-  bool any_flush = false, special = false;
+  Wide sum;                                        // the row's sum so far, in units of scale E
+  int E = kNoScale;
+  bool special = false;                            // the group met an infinity or NaN
   const bool writes = active && (!WPR || sub == 0);
   const size_t o = (size_t)K * NP + i;
   const int ea = active ? __ldg(q.EA + o) : 0;
@@ -223,7 +263,7 @@ __device__ __forceinline__ double fx_pack(const FxOp& q, int pack, int2* __restr
   for (int base = 0; base < maxc; base += CH) {
     int J[CH];
     double xv[CH];
-    int em = 0;
+    unsigned em[(CH + 1) / 2];   // the blocks' exponent fields, two to a word
     DigitRow<NP> row;
 #pragma unroll
     for (int c = 0; c < CH; ++c) {
@@ -243,42 +283,46 @@ __device__ __forceinline__ double fx_pack(const FxOp& q, int pack, int2* __restr
 #pragma unroll
     for (int c = 0; c < CH; ++c) xv[c] = J[c] >= 0 ? vload<COHERENT>(q.x + (size_t)J[c] * NP + i) : 0.0;
 #pragma unroll
-    for (int c = 0; c < CH; ++c) em = max(em, biased_exponent(xv[c]));
-    em = max(1, __reduce_max_sync(0xffffffffu, em));
-    if (em == 0x7FF) {
-      special = true;
-      break;
+    for (int c = 0; c < CH; c += 2) {
+      unsigned f = biased_exponent(xv[c]);
+      if (c + 1 < CH) f |= (unsigned)biased_exponent(xv[c + 1 < CH ? c + 1 : c]) << 16;
+      em[c / 2] = group_max<NP>(f, sub, i);
     }
-    if (em > ex || terms + CH * NP * SPL > kMaxTerms) {   // the same in every lane
-      if (terms > 0) {
-        flushed += fx_value(sum.hh, sum.low(), ea + ex - 1022);
-        any_flush = true;
-        sum = Acc();
-        terms = 0;
-      }
-      ex = max(em, ex);
+    auto field = [&](int c) { return max(1, (int)(em[c / 2] >> (c & 1) * 16 & 0xFFFF)); };
+    if constexpr (!ONE) {
+      int top = E;
+#pragma unroll
+      for (int c = 0; c < CH; ++c)
+        if (base + c < cnt) top = max(top, ea + field(c) + kHead);
+      sum.down(top - E);
+      E = top;
+    } else {
+      E = ea + field(0);
     }
-    terms += CH * NP * SPL;
     __syncwarp();
 #pragma unroll
     for (int c = 0; c < CH; ++c)
       if (base + c < maxc) {   // the same in every lane
-        const int2 d = split_digits(xv[c], ex);
+        special |= field(c) == 0x7FF;
+        const int2 d = split_digits(xv[c], field(c));
         if (grp) xs[c * NP + i] = d;
       }
     __syncwarp();
 #pragma unroll
     for (int c = 0; c < CH; ++c) {
       if (base + c < cnt) {
-        fx_mac<NP>(row, xs + c * NP, sum);
+        Acc s;
+        fx_mac<NP>(row, xs + c * NP, s);
         if (c + 1 < CH && base + c + 1 < cnt) row.load(A + (size_t)(first + (base + c + 1) * SPL) * NP * NP, i);
+        Wide w = s.wide();
+        if constexpr (!ONE) w.down(E - ea - field(c));
+        sum.add(w);
       }
     }
   }
-  double acc;
+  double acc = 0.0;
   if (special) {
     // an infinity or NaN among the values: FP64 products, so that it spreads as IEEE arithmetic says
-    acc = 0.0;
     for (int t = 0; t < cnt; ++t) {
       const int blk = first + t * SPL;
       const int J = ONE ? (q.cols ? q.cols[K] : K) : q.cols ? q.cols[(size_t)K * q.width + (WPR ? sub + t * SPL : t)] : blk;
@@ -288,15 +332,13 @@ __device__ __forceinline__ double fx_pack(const FxOp& q, int pack, int2* __restr
         acc = fma(scale2(__ll2double_rn(((long long)d.x << 30) + d.y), ea - 58), vload<COHERENT>(xj + j), acc);
       }
     }
-    any_flush = true;
-  } else if (any_flush) {
-    acc = flushed + fx_value(sum.hh, sum.low(), ea + ex - 1022);
   }
-  long long hi = sum.hh;
-  unsigned long long lo = sum.low();
+  bool in_fp64 = special;
   if constexpr (WPR && RPW > 1) {
-    // sum over the groups of the row: the integer sums exactly
-    if (any_flush) {
+    // sum over the groups of the row: the integer sums, brought to one scale, exactly
+    in_fp64 = __any_sync(0xffffffffu, special && grp);
+    if (in_fp64) {
+      if (!special) acc = fx_value(sum.hi, sum.lo, E - 1022);
 #pragma unroll
       for (int m = RPW; m > 1; m = (m + 1) / 2) {
         const int h = (m + 1) / 2;
@@ -304,21 +346,27 @@ __device__ __forceinline__ double fx_pack(const FxOp& q, int pack, int2* __restr
         if (sub + h < m) acc += t;
       }
     } else {
+      int top = E;
 #pragma unroll
       for (int m = RPW; m > 1; m = (m + 1) / 2) {
         const int h = (m + 1) / 2;
-        const long long th = __shfl_down_sync(0xffffffffu, hi, h * NP);
-        const unsigned long long tl = __shfl_down_sync(0xffffffffu, lo, h * NP);
-        if (sub + h < m) {   // at most ten groups: the low parts stay below 2^64
-          hi += th;
-          lo += tl;
-        }
+        const int t = __shfl_down_sync(0xffffffffu, top, h * NP);
+        if (sub + h < m) top = max(top, t);
       }
-      hi += (long long)(lo >> 60);
-      lo &= (1ull << 60) - 1;
+      top = __shfl_sync(0xffffffffu, top, i);
+      sum.down(max(top - E, 0));   // a lane without a group may hold more than group 0
+      E = top;
+#pragma unroll
+      for (int m = RPW; m > 1; m = (m + 1) / 2) {
+        const int h = (m + 1) / 2;
+        Wide t;
+        t.hi = __shfl_down_sync(0xffffffffu, sum.hi, h * NP);
+        t.lo = __shfl_down_sync(0xffffffffu, sum.lo, h * NP);
+        if (sub + h < m) sum.add(t);
+      }
     }
   }
-  if (!any_flush) acc = fx_value(hi, lo, ea + ex - 1022);
+  if (!in_fp64) acc = fx_value(sum.hi, sum.lo, E - 1022);
   if (ea == kNotFinite) acc = nan("");
   if (writes && (MODE == 3 || (MODE == 0 && q.dot))) xo = vload<COHERENT>(q.x + o);
   return writes ? finish<MODE>(acc, o, xo, bo, q.y, q.y2, q.omega, dsum, q.dotv) : dsum;
