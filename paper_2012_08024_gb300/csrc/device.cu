@@ -139,7 +139,7 @@ size_t layout(const cdg::Hierarchy& H, int precision, int nrhs, DeviceState* S, 
       L.A = c.take<double>(A.val.size());
       // digits of A_0 of their own for the many-right-hand-side apply where A itself stays in FP64
       if (!fixed && l == 0 && nrhs > 0) L.Adig = c.take<double>(A.val.size());
-      if (fixed || (l == 0 && nrhs > 0)) L.eA = c.take<int>((size_t)L.n * npl);
+      if (fixed || (l == 0 && nrhs > 0)) L.eA = c.take<unsigned short>((size_t)A.nnzb() * npl);
       if (fixed) {
         L.well = widest_row(A);
         L.ell = c.take<int>((size_t)L.n * L.well + 1);
@@ -157,15 +157,15 @@ size_t layout(const cdg::Hierarchy& H, int precision, int nrhs, DeviceState* S, 
         if (nL) L.L = c.take<double>(nL);
         L.Ahat = c.take<double>(Sh.val.size() + 1);
         if (fixed) {
-          L.eD = c.take<int>((size_t)L.n * npl);
-          L.eH = c.take<int>((size_t)L.n * npl);
+          L.eD = c.take<unsigned short>((size_t)L.n * npl);
+          L.eH = c.take<unsigned short>((size_t)Sh.nnzb() * npl);
           L.whell = widest_row(Sh);
           L.hell = c.take<int>((size_t)L.n * L.whell + 1);
           if (nL) {
             L.Lx = c.take<double>(nL);
-            L.eL = c.take<int>((size_t)L.n * npl);
+            L.eL = c.take<unsigned short>((size_t)L.n * npl);
             L.Rx = c.take<double>(nL);
-            L.eR = c.take<int>((size_t)H.A_t[l + 1].nrows * npl);
+            L.eR = c.take<unsigned short>((size_t)L.n * npl);
           }
         }
       } else {
@@ -1862,17 +1862,17 @@ int dev_bind(cdg_handle* h, void* buf, int64_t bytes, void* stream) {
   }
   if (D.lev[0].Adig) {
     upload(D.lev[0].Adig, H.A_t[0].val, s);
-    fx_encode(D.lev[0].np, D.lev[0].n, D.lev[0].rowptr, D.lev[0].Adig, D.lev[0].eA, s);
+    fx_encode(D.lev[0].np, D.lev[0].nnzb, D.lev[0].Adig, D.lev[0].eA, s);
   }
-  if (D.fixed) {   // FP64 blocks to digits (the restriction reads the next level's children ranges)
+  if (D.fixed) {   // FP64 blocks to digits
     bool ok = true;
     for (int l = 0; l < nlev; ++l) {
       const DevLevel& L = D.lev[l];
-      if (L.A) ok = ok && fx_encode(L.np, L.n, L.rowptr, L.A, L.eA, s);
-      if (L.Ahat) ok = ok && fx_encode(L.np, L.n, L.hrowptr, L.Ahat, L.eH, s);
-      if (L.Dinv) ok = ok && fx_encode(L.np, L.n, nullptr, L.Dinv, L.eD, s);
-      if (L.Lx) ok = ok && fx_encode(L.np, L.n, nullptr, L.Lx, L.eL, s);
-      if (L.Rx) ok = ok && fx_encode(L.np, D.lev[l + 1].n, D.lev[l + 1].childptr, L.Rx, L.eR, s);
+      if (L.A) ok = ok && fx_encode(L.np, L.nnzb, L.A, L.eA, s);
+      if (L.Ahat) ok = ok && fx_encode(L.np, L.hnnzb, L.Ahat, L.eH, s);
+      if (L.Dinv) ok = ok && fx_encode(L.np, L.n, L.Dinv, L.eD, s);
+      if (L.Lx) ok = ok && fx_encode(L.np, L.n, L.Lx, L.eL, s);
+      if (L.Rx) ok = ok && fx_encode(L.np, L.n, L.Rx, L.eR, s);
     }
     if (!ok) {
       h->err = "unsupported number of basis functions per element";

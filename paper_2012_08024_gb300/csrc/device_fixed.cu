@@ -9,23 +9,31 @@
 // clocks.  So an operator entry is kept as two signed integer digits (the same
 // 8 bytes as a double),
 //     a = 2^(EA - 58) (ah 2^30 + al),   |ah| <= 2^28,  |al| <= 2^29,
-// with one exponent EA per scalar row, every entry rounded to 2^-59 of the
-// row's power-of-two bound, and the n_p values of a neighbour's x_J are split
-// likewise with one exponent of their own.  Four integer multiply-adds give a
-// product of digits exactly, the sum over a block is exact, the blocks' sums are
-// brought to the scale of the largest (nothing above 2^-96 of it is lost), and
-// one rounding to FP64 ends the row: 16 clocks in the place of 64.  A row's
-// result depends on the values that it multiplies and on no others: with one
-// exponent for all that a warp gathers, rows of two meshes of a batch shared one,
-// and a mesh with small data beside one with large data got a wrong solution.
-// (The exponents per block cost 2-4%: apply 72.4 -> 74.3 us, V-cycle of the
-// 128^2 (p = 3) mesh 199 -> 207 us, 64 meshes 52.4 -> 54.5 ms.)  The
-// method is the splitting of Ozaki, Ogita, Oishi and Rump (2012) with integer
-// digits.  58 bits, not fewer, since A x cancels for smooth x, where the small
-// constant-mode entries of A meet the largest values of x: on solutions of the
-// 32^2 (p = 1, 2, 3) and 6^3 (p = 1, 2) meshes FP64 sums are 0.5-4.1e-12 off in
-// the 2-norm, 54-bit digits 1.7-44e-12, 58-bit digits 0.07-2.4e-12 (each below
-// FP64's on the same mesh); random vectors 1.0-2.0e-16 against 0.4-0.7e-17.
+// with one exponent EA per scalar row of a block, every entry rounded to 2^-59
+// of the power of two above that row's largest, and the n_p values of a
+// neighbour's x_J are split likewise with one exponent of their own.  Four
+// integer multiply-adds give a product of digits exactly, the sum over a block is
+// exact, the blocks' sums are brought to the scale of the largest (nothing above
+// 2^-96 of it is lost), and one rounding to FP64 ends the row: 16 clocks in the
+// place of 64.  The method is the splitting of Ozaki, Ogita, Oishi and Rump
+// (2012) with integer digits.
+//
+// Why an exponent per block and not a wider one: with one per scalar row of A and
+// one for all the values that a warp gathers, blocks that kappa makes small lost
+// their low digits, a row's result depended on rows that it has no block with,
+// and a mesh of a batch whose data were small beside its neighbour's got a wrong
+// solution.  Now a row is off by no more than 2^-57 n_p sum_J max|a_J| max|x_J|
+// and one rounding.  It costs 0-5% (against the wider exponents: apply of 256^2,
+// p = 3, 72.5 -> 75.0 us; V-cycle of 128^2, p = 3, 199 -> 196 us; 64 meshes at
+// p = 2 52.5 -> 54.3 ms; 101^2 at p = 1 7.0 -> 7.3 ms).
+// Why 58 bits and not fewer: A x cancels for smooth x, where the small
+// constant-mode entries of A meet the largest values of x.  On solutions of the
+// 32^2 (p = 1, 2, 3) and 6^3 (p = 1, 2) meshes FP64 sums are 0.3-3.1e-12 off in
+// the 2-norm, the digits 0.01-0.36e-12, with kappa from 1e-4 to 1e4 at random
+// (24^2, p = 2, 3) 3.3-8.1e-9 against 0.1-0.4e-9, random vectors 0.8-1.9e-16
+// against 0.5e-16; relative to sum |a| |x| of its own row the worst row of these
+// is 7e-16 off with FP64 sums and 4e-15 with digits.  V-cycles (48^2, p = 1, 2,
+// 3, random r): 0.3-1.2e-12 against 0.4-38e-15.
 //
 // The sums, over the T <= 28 terms of a block: |sum al xl| <= 2^58 T,
 // |sum (ah xl + al xh)| <= 2^58 T; both are then carried into the next higher
@@ -41,7 +49,7 @@
 // pointers.  The kernel waits for memory (issue slots a third used), so resident
 // warps count: 64 registers, 32 warps per SM.  Measured, 131,072 rows of 4
 // blocks at n_p = 10: apply 102.7 -> 76.9 us, level of 1,044 rows 12.6 -> 4.7 us
-// (72.7 us, 6.1 TB/s, and 3.2 us with dependent launches); 80 registers 84.7 us; digits streamed through shared memory by
+// (75.0 us, 5.9 TB/s, and 3.2 us with dependent launches); 80 registers 84.7 us; digits streamed through shared memory by
 // cp.async, one or two packs ahead, 85-104 us (fewer warps fit); 48 registers 90 us.
 #include <cuda_runtime.h>
 
@@ -74,38 +82,30 @@ __global__ void __launch_bounds__(kFxThreads, fx_ctas_per_sm(NP)) fx_kernel(cons
     }
 }
 
-// FP64 blocks to digits, in place: one warp per block row (the row exponents
-// first, then block by block through registers)
+// FP64 blocks to digits, in place: one warp per block (its rows' exponents first, then through registers)
 template <int NP>
-__global__ void __launch_bounds__(kFxThreads) fx_encode_kernel(int n, const int* __restrict__ rowptr,
-                                                               double* A, int* __restrict__ EA) {
+__global__ void __launch_bounds__(kFxThreads) fx_encode_kernel(int64_t blocks, double* A, unsigned short* EA) {
   constexpr int PER = (NP * NP + 31) / 32;
   __shared__ int ex[kFxWarps][NP];
   const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-  const int K = blockIdx.x * kFxWarps + w;
-  if (K >= n) return;
-  const int b0 = rowptr ? rowptr[K] : K, b1 = rowptr ? rowptr[K + 1] : K + 1;
+  const int64_t b = (int64_t)blockIdx.x * kFxWarps + w;
+  if (b >= blocks) return;
   for (int i = lane; i < NP; i += 32) ex[w][i] = 1;
   __syncwarp();
-  for (int bb = b0; bb < b1; ++bb)
-    for (int t = lane; t < NP * NP; t += 32) atomicMax(&ex[w][t / NP], biased_exponent(A[(size_t)bb * NP * NP + t]));
+  double v[PER];
+#pragma unroll
+  for (int c = 0; c < PER; ++c) {
+    const int t = c * 32 + lane;
+    v[c] = t < NP * NP ? A[(size_t)b * NP * NP + t] : 0.0;
+    if (t < NP * NP) atomicMax(&ex[w][t / NP], biased_exponent(v[c]));
+  }
   __syncwarp();
-  for (int i = lane; i < NP; i += 32) EA[(size_t)K * NP + i] = ex[w][i] == 0x7FF ? kNotFinite : ex[w][i] - 1022;
-  for (int bb = b0; bb < b1; ++bb) {
-    double v[PER];
+  for (int i = lane; i < NP; i += 32) EA[(size_t)b * NP + i] = (unsigned short)ex[w][i];
+  int2* d = reinterpret_cast<int2*>(A) + (size_t)b * NP * NP;
 #pragma unroll
-    for (int c = 0; c < PER; ++c) {
-      const int t = c * 32 + lane;
-      v[c] = t < NP * NP ? A[(size_t)bb * NP * NP + t] : 0.0;
-    }
-    __syncwarp();
-    int2* d = reinterpret_cast<int2*>(A) + (size_t)bb * NP * NP;
-#pragma unroll
-    for (int c = 0; c < PER; ++c) {
-      const int t = c * 32 + lane;
-      if (t < NP * NP) d[fx_pos(NP, t / NP, t % NP)] = split_digits(v[c], ex[w][t / NP]);
-    }
-    __syncwarp();
+  for (int c = 0; c < PER; ++c) {
+    const int t = c * 32 + lane;
+    if (t < NP * NP) d[fx_pos(NP, t / NP, t % NP)] = split_digits(v[c], ex[w][t / NP]);
   }
 }
 
@@ -175,7 +175,7 @@ FxOp operator_op(const DevLevel& L, int mode) {
 }
 
 // one block per row
-FxOp diagonal_op(const DevLevel& L, int mode, const double* blocks, const int* exps) {
+FxOp diagonal_op(const DevLevel& L, int mode, const double* blocks, const unsigned short* exps) {
   FxOp o;
   o.mode = mode;
   o.np = L.np;
@@ -207,10 +207,10 @@ FxOp restrict_op(const DevLevel& F, const DevLevel& C) {
 unsigned fx_grid(const FxOp& o) { return dispatch(o, nullptr, false); }
 bool fx_run(const FxOp& o, cudaStream_t s) { return dispatch(o, s, true) > 0; }
 
-bool fx_encode(int np, int n, const int* rowptr, double* A, int* EA, cudaStream_t s) {
-  if (n < 1) return true;
-  FX_NP_DISPATCH(np, (fx_encode_kernel<NP><<<(unsigned)((n + kFxWarps - 1) / kFxWarps), kFxThreads, 0, s>>>(n, rowptr,
-                                                                                                          A, EA)));
+bool fx_encode(int np, int64_t blocks, double* A, unsigned short* EA, cudaStream_t s) {
+  if (blocks < 1) return true;
+  FX_NP_DISPATCH(np, (fx_encode_kernel<NP><<<(unsigned)((blocks + kFxWarps - 1) / kFxWarps), kFxThreads, 0, s>>>(
+                         blocks, A, EA)));
   count_launch();
   return true;
 }

@@ -12,12 +12,14 @@ namespace fx {
 
 constexpr int kFxThreads = 128;
 constexpr int kFxWarps = kFxThreads / 32;
-constexpr int kMaxTerms = 127;        // of one scale, so that their sums stay within 63 bits
-constexpr int kNotFinite = 1 << 20;   // row exponent of a matrix row that holds an infinity or NaN
+constexpr int kNotFinite = 0x7FF;     // exponent field of an infinity or NaN
+constexpr int kScale = 2 * 1022;      // a sum's scale is the sum of two exponent fields, E + 1022 each
 constexpr int kNoScale = -(1 << 24);  // scale of an empty sum, below every other
 
-// blocks of a row per step of a group: the level-0 rows of tetrahedra hold five
-constexpr int fx_chunk(int np) { return np == 4 || np == 10 || np == 20 ? 5 : 4; }
+// blocks of a row per step of a group: the level-0 rows of A hold five on tetrahedra (Ahat one less)
+constexpr int fx_chunk(int np, int mode, bool wpr) {
+  return !wpr && mode <= 1 && (np == 4 || np == 10 || np == 20) ? 5 : 4;
+}
 constexpr bool fx_one(int mode) { return mode == 4 || mode == 6 || mode == 7; }   // one block per row
 // resident CTAs of 128 threads per SM that the registers are held to
 constexpr int fx_ctas_per_sm(int np) { return np > 10 ? 4 : 8; }
@@ -187,7 +189,7 @@ template <int NP, int MODE, bool WPR>
 struct Pack {
   static constexpr int RPW = 32 / NP;
   static constexpr bool ONE = fx_one(MODE);
-  static constexpr int CH = ONE ? 1 : fx_chunk(NP);
+  static constexpr int CH = ONE ? 1 : fx_chunk(NP, MODE, WPR);
   static constexpr int SPL = WPR ? RPW : 1;                       // groups that share a block row
   static constexpr int GS = CH * NP + 2 + (CH * NP) % 2;          // digits of one group's chunk (padded against bank conflicts)
   static constexpr int DIGITS = RPW * GS;
@@ -238,10 +240,9 @@ __device__ __forceinline__ double fx_pack(const FxOp& q, int pack, int2* __restr
   const int maxc = __reduce_max_sync(0xffffffffu, cnt);
   Wide sum;                                        // the row's sum so far, in units of scale E
   int E = kNoScale;
-  bool special = false;                            // the group met an infinity or NaN
+  bool special = false, bad_row = false;           // an infinity or NaN among the values, in the matrix row
   const bool writes = active && (!WPR || sub == 0);
   const size_t o = (size_t)K * NP + i;
-  const int ea = active ? __ldg(q.EA + o) : 0;
   double xo = 0.0, bo = 0.0;                       // the epilogue's operands, on their way early
   auto inputs = [&]() {
     if (!waited) cdgk::wait_for_inputs();
@@ -263,7 +264,7 @@ __device__ __forceinline__ double fx_pack(const FxOp& q, int pack, int2* __restr
   for (int base = 0; base < maxc; base += CH) {
     int J[CH];
     double xv[CH];
-    unsigned em[(CH + 1) / 2];   // the blocks' exponent fields, two to a word
+    unsigned ea[(CH + 1) / 2] = {}, em[(CH + 1) / 2];   // exponent fields of blocks and values, two to a word
     DigitRow<NP> row;
 #pragma unroll
     for (int c = 0; c < CH; ++c) {
@@ -278,6 +279,9 @@ __device__ __forceinline__ double fx_pack(const FxOp& q, int pack, int2* __restr
         J[c] = first + t * SPL;
       }
     }
+#pragma unroll
+    for (int c = 0; c < CH; ++c)
+      if (base + c < cnt) ea[c / 2] |= (unsigned)__ldg(q.EA + (size_t)(first + (base + c) * SPL) * NP + i) << (c & 1) * 16;
     if (base < cnt) row.load(A + (size_t)(first + base * SPL) * NP * NP, i);
     if (base == 0) inputs();
 #pragma unroll
@@ -288,23 +292,30 @@ __device__ __forceinline__ double fx_pack(const FxOp& q, int pack, int2* __restr
       if (c + 1 < CH) f |= (unsigned)biased_exponent(xv[c + 1 < CH ? c + 1 : c]) << 16;
       em[c / 2] = group_max<NP>(f, sub, i);
     }
-    auto field = [&](int c) { return max(1, (int)(em[c / 2] >> (c & 1) * 16 & 0xFFFF)); };
-    if constexpr (!ONE) {
-      int top = E;
+    unsigned es[(CH + 1) / 2], ma = ea[0], mx = em[0], ms;   // the blocks' scales; the largest of all three
 #pragma unroll
-      for (int c = 0; c < CH; ++c)
-        if (base + c < cnt) top = max(top, ea + field(c) + kHead);
+    for (int w = 0; w < (CH + 1) / 2; ++w) {
+      em[w] = __vmaxu2(em[w], 0x00010001u);
+      es[w] = ea[w] + em[w];
+      ma = __vmaxu2(ma, ea[w]);
+      mx = __vmaxu2(mx, em[w]);
+      ms = w == 0 ? es[0] : __vmaxu2(ms, es[w]);
+    }
+    auto half = [](unsigned v, int c) { return (int)(v >> (c & 1) * 16 & 0xFFFF); };
+    bad_row |= max(half(ma, 0), half(ma, 1)) == kNotFinite;
+    special |= max(half(mx, 0), half(mx, 1)) == kNotFinite;
+    if constexpr (!ONE) {
+      const int top = max(E, max(half(ms, 0), half(ms, 1)) + kHead);
       sum.down(top - E);
       E = top;
     } else {
-      E = ea + field(0);
+      E = half(ms, 0);
     }
     __syncwarp();
 #pragma unroll
     for (int c = 0; c < CH; ++c)
       if (base + c < maxc) {   // the same in every lane
-        special |= field(c) == 0x7FF;
-        const int2 d = split_digits(xv[c], field(c));
+        const int2 d = split_digits(xv[c], half(em[c / 2], c));
         if (grp) xs[c * NP + i] = d;
       }
     __syncwarp();
@@ -315,7 +326,7 @@ __device__ __forceinline__ double fx_pack(const FxOp& q, int pack, int2* __restr
         fx_mac<NP>(row, xs + c * NP, s);
         if (c + 1 < CH && base + c + 1 < cnt) row.load(A + (size_t)(first + (base + c + 1) * SPL) * NP * NP, i);
         Wide w = s.wide();
-        if constexpr (!ONE) w.down(E - ea - field(c));
+        if constexpr (!ONE) w.down(E - half(es[c / 2], c));
         sum.add(w);
       }
     }
@@ -327,9 +338,10 @@ __device__ __forceinline__ double fx_pack(const FxOp& q, int pack, int2* __restr
       const int blk = first + t * SPL;
       const int J = ONE ? (q.cols ? q.cols[K] : K) : q.cols ? q.cols[(size_t)K * q.width + (WPR ? sub + t * SPL : t)] : blk;
       const double* xj = q.x + (size_t)J * NP;
+      const int e = __ldg(q.EA + (size_t)blk * NP + i) - 1022 - 58;
       for (int j = 0; j < NP; ++j) {
         const int2 d = A[(size_t)blk * NP * NP + fx_pos(NP, i, j)];
-        acc = fma(scale2(__ll2double_rn(((long long)d.x << 30) + d.y), ea - 58), vload<COHERENT>(xj + j), acc);
+        acc = fma(scale2(__ll2double_rn(((long long)d.x << 30) + d.y), e), vload<COHERENT>(xj + j), acc);
       }
     }
   }
@@ -338,7 +350,7 @@ __device__ __forceinline__ double fx_pack(const FxOp& q, int pack, int2* __restr
     // sum over the groups of the row: the integer sums, brought to one scale, exactly
     in_fp64 = __any_sync(0xffffffffu, special && grp);
     if (in_fp64) {
-      if (!special) acc = fx_value(sum.hi, sum.lo, E - 1022);
+      if (!special) acc = fx_value(sum.hi, sum.lo, E - kScale);
 #pragma unroll
       for (int m = RPW; m > 1; m = (m + 1) / 2) {
         const int h = (m + 1) / 2;
@@ -366,8 +378,16 @@ __device__ __forceinline__ double fx_pack(const FxOp& q, int pack, int2* __restr
       }
     }
   }
-  if (!in_fp64) acc = fx_value(sum.hi, sum.lo, E - 1022);
-  if (ea == kNotFinite) acc = nan("");
+  if (!in_fp64) acc = fx_value(sum.hi, sum.lo, E - kScale);
+  if constexpr (WPR && RPW > 1)
+    if (__any_sync(0xffffffffu, bad_row))
+#pragma unroll
+      for (int m = RPW; m > 1; m = (m + 1) / 2) {
+        const int h = (m + 1) / 2;
+        const int t = __shfl_down_sync(0xffffffffu, (int)bad_row, h * NP);
+        bad_row |= sub + h < m && t;
+      }
+  if (bad_row) acc = nan("");
   if (writes && (MODE == 3 || (MODE == 0 && q.dot))) xo = vload<COHERENT>(q.x + o);
   return writes ? finish<MODE>(acc, o, xo, bo, q.y, q.y2, q.omega, dsum, q.dotv) : dsum;
 }

@@ -17,7 +17,7 @@ struct FxOp {
   const int* cols = nullptr;  // [n][width], -1 behind a row's last block; one-block modes: [n] or nullptr (K)
   int width = 0;
   const void* A = nullptr;    // digits
-  const int* EA = nullptr;    // [n][np] row exponents
+  const unsigned short* EA = nullptr;   // [blocks][np] exponents of the digits (fx_encode)
   const double* x = nullptr;
   const double* b = nullptr;
   double* y = nullptr;
@@ -43,11 +43,12 @@ struct DevLevel;
 // products with a level's operators: A (modes 0, 1) or Ahat (3); a diagonal of blocks (6, 7); the
 // prolongation to level F from its parents (4, 7); the restriction from F to the next level C (8)
 FxOp operator_op(const DevLevel& L, int mode);
-FxOp diagonal_op(const DevLevel& L, int mode, const double* blocks, const int* exps);
+FxOp diagonal_op(const DevLevel& L, int mode, const double* blocks, const unsigned short* exps);
 FxOp prolong_op(const DevLevel& F, int mode = 4);
 FxOp restrict_op(const DevLevel& F, const DevLevel& C);
 
 unsigned fx_grid(const FxOp& o);                  // CTAs of fx_run
 bool fx_run(const FxOp& o, cudaStream_t s);       // false: no instance for this np
-// FP64 blocks [blocks][np][np] of n block rows to digits, in place, with the row exponents EA [n][np]
-bool fx_encode(int np, int n, const int* rowptr, double* A, int* EA, cudaStream_t s);
+// FP64 blocks [blocks][np][np] to digits, in place; EA [blocks][np]: the exponent field of the largest entry
+// of each of their scalar rows
+bool fx_encode(int np, int64_t blocks, double* A, unsigned short* EA, cudaStream_t s);

@@ -194,87 +194,97 @@ __global__ void __launch_bounds__(128, mr_min_ctas<V, PF>()) mr_row_kernel(int n
 }
 
 // y = A_0 x in FP64 by integer digits (device_fixed.cu says why and how): a warp owns one block row and
-// 32 right-hand sides, one per lane.  A lane takes the largest exponent of its column over the row's
-// neighbours (a first pass, which also brings x into the caches), splits its values and keeps the n_p
-// sums in registers; the digits of a block are read from shared memory, each 16 bytes feeding eight
-// integer multiply-adds.  A_0 has at most dim + 2 blocks per row (compact stencil), so its rows need no
-// flush.  5,000 rows, n_p = 6, 40 columns: 82 us with FP64 multiply-adds (46 us at the FP64 rate), 50 us here.
+// 32 right-hand sides, one per lane.  A lane splits the n_p values of its column in a block's neighbour
+// (one exponent for them) and keeps the n_p sums, each with its scale, in registers; the digits of a
+// block are read from shared memory, each 16 bytes feeding eight integer multiply-adds.  5,000 rows,
+// n_p = 6, 40 columns: 82 us with FP64 multiply-adds (46 us at the FP64 rate), 50 us here.
 template <int NP>
 __global__ void __launch_bounds__(128, 4) mr_fx_kernel(int n, int R, const int* __restrict__ rowptr,
                                                        const int* __restrict__ col, const int2* __restrict__ A,
-                                                       const int* __restrict__ EA, const double* __restrict__ x,
-                                                       double* __restrict__ y) {
+                                                       const unsigned short* __restrict__ EA,
+                                                       const double* __restrict__ x, double* __restrict__ y) {
   constexpr int NN = NP * NP;
-  constexpr int CARRY = 31 / NP;   // blocks between carries
   __shared__ __align__(16) int2 as_s[kMrMaxBR][(NN + 1) / 2 * 2];
+  __shared__ int ea_s[kMrMaxBR][NP];
   int2* as = as_s[threadIdx.y];
+  int* ea = ea_s[threadIdx.y];
   const int K = blockIdx.x * blockDim.y + threadIdx.y;
   const int lane = threadIdx.x;
   const int r = blockIdx.y * 32 + lane;
   if (K >= n) return;   // a whole warp
   const bool on = r < R;
   const int b0 = rowptr[K], b1 = rowptr[K + 1];
-  int em = 1;
-  if (on)
-    for (int t = b0; t < b1; ++t) {
-      const double* xj = x + (size_t)col[t] * NP * R + r;
+  bool special = false;
+  unsigned bad_rows = 0;
+  fx::Wide acc[NP];
+  int E[NP];
 #pragma unroll
-      for (int j = 0; j < NP; ++j) em = max(em, fx::biased_exponent(xj[(size_t)j * R]));
-    }
-  const bool special = em == 0x7FF;
-  fx::Acc acc[NP];
-  for (int t = b0, since = 0; t < b1; ++t) {
+  for (int i = 0; i < NP; ++i) E[i] = fx::kNoScale;
+  for (int t = b0; t < b1; ++t) {
     __syncwarp();
     for (int u = lane; u < NN; u += 32) as[u] = A[(size_t)t * NN + u];
+    if (lane < NP) ea[lane] = EA[(size_t)t * NP + lane];
     int2 xd[NP];
-    if (on && !special) {
+    int em = 1;
+    if (on) {
       const double* xj = x + (size_t)col[t] * NP * R + r;
+      double xv[NP];
 #pragma unroll
-      for (int j = 0; j < NP; ++j) xd[j] = fx::split_digits(xj[(size_t)j * R], em);
+      for (int j = 0; j < NP; ++j) xv[j] = xj[(size_t)j * R];
+#pragma unroll
+      for (int j = 0; j < NP; ++j) em = max(em, fx::biased_exponent(xv[j]));
+#pragma unroll
+      for (int j = 0; j < NP; ++j) xd[j] = fx::split_digits(xv[j], em);
     }
     __syncwarp();
-    if (on && !special) {
-      if constexpr (NP % 2 == 0) {
-        const int4* a4 = reinterpret_cast<const int4*>(as);
+    if (on) {
+      special |= em == fx::kNotFinite;
 #pragma unroll
-        for (int j = 0; j < NP; j += 2)
+      for (int i = 0; i < NP; ++i) {
+        fx::Acc s;
+        if constexpr (NP % 2 == 0) {
+          const int4* a4 = reinterpret_cast<const int4*>(as) + i;
 #pragma unroll
-          for (int i = 0; i < NP; ++i) {
-            const int4 d = a4[(j >> 1) * NP + i];
-            fx::mac(acc[i], d.x, d.y, xd[j].x, xd[j].y);
-            fx::mac(acc[i], d.z, d.w, xd[j + 1].x, xd[j + 1].y);
+          for (int j = 0; j < NP; j += 2) {
+            const int4 d = a4[(j >> 1) * NP];
+            fx::mac(s, d.x, d.y, xd[j].x, xd[j].y);
+            fx::mac(s, d.z, d.w, xd[j + 1].x, xd[j + 1].y);
           }
-      } else {
+        } else {
 #pragma unroll
-        for (int j = 0; j < NP; ++j)
-#pragma unroll
-          for (int i = 0; i < NP; ++i) {
+          for (int j = 0; j < NP; ++j) {
             const int2 d = as[j * NP + i];
-            fx::mac(acc[i], d.x, d.y, xd[j].x, xd[j].y);
+            fx::mac(s, d.x, d.y, xd[j].x, xd[j].y);
           }
-      }
-      if (++since == CARRY || t + 1 == b1) {
-        since = 0;
-#pragma unroll
-        for (int i = 0; i < NP; ++i) acc[i].carry();
+        }
+        s.carry();
+        if (ea[i] == fx::kNotFinite) bad_rows |= 1u << i;
+        const int e = ea[i] + em + fx::kHead;
+        if (e > E[i]) {
+          acc[i].down(e - E[i]);
+          E[i] = e;
+        }
+        fx::Wide w = s.wide();
+        w.down(E[i] - e + fx::kHead);
+        acc[i].add(w);
       }
     }
   }
   if (!on) return;
 #pragma unroll
   for (int i = 0; i < NP; ++i) {
-    const int ea = EA[(size_t)K * NP + i];
-    double v = fx::fx_value(acc[i].hh, acc[i].low(), ea + em - 1022);
+    double v = fx::fx_value(acc[i].hi, acc[i].lo, E[i] - fx::kScale);
     if (special) {   // an infinity or NaN in the column: FP64 products
       v = 0.0;
-      for (int t = b0; t < b1; ++t)
+      for (int t = b0; t < b1; ++t) {
+        const int e = EA[(size_t)t * NP + i] - 1022 - 58;
         for (int j = 0; j < NP; ++j) {
           const int2 d = A[(size_t)t * NN + fx::fx_pos(NP, i, j)];
-          v = fma(fx::scale2(__ll2double_rn(((long long)d.x << 30) + d.y), ea - 58),
-                  x[((size_t)col[t] * NP + j) * R + r], v);
+          v = fma(fx::scale2(__ll2double_rn(((long long)d.x << 30) + d.y), e), x[((size_t)col[t] * NP + j) * R + r], v);
         }
+      }
     }
-    if (ea == fx::kNotFinite) v = nan("");
+    if (bad_rows >> i & 1) v = nan("");
     y[((size_t)K * NP + i) * R + r] = v;
   }
 }
@@ -923,7 +933,6 @@ bool mr_apply64(DeviceState& D, MR& M, const double* x, double* y, cudaStream_t 
   const int br = rows ? rows : rows_of(M, 0, 0);
   const dim3 grid((unsigned)((L0.n + br - 1) / br), (unsigned)((M.R + 31) / 32)), block(32, (unsigned)br);
   const int2* A = reinterpret_cast<const int2*>(D.fixed ? L0.A : L0.Adig);
-  if (L0.n > 0 && (int64_t)(D.d + 2) * D.np > fx::kMaxTerms) return false;   // the sums of a row (compact stencil)
   MR_NP_DISPATCH(D.np, mr_fx_kernel<NP><<<grid, block, 0, s>>>(L0.n, M.R, L0.rowptr, L0.col, A, L0.eA, x, y));
   count_launch();
   return true;

@@ -185,13 +185,16 @@ __device__ void ph_coarse(const PParams& P, const T* b, T* x, bool add) {
 // than the 40 of the FP64-block kernel; 66.4 ms with the later CG kernels); two CTAs 265 us, 102 us, 80.3 ms.
 template <int NP>
 constexpr int most_digits() {
-  constexpr int packed = fx::Pack<NP, 8, false>::DIGITS, shared = fx::Pack<NP, 8, true>::DIGITS;
-  return packed > shared ? packed : shared;
+  // of the modes that the phases run: 1, 3 and 8 packed or with a row per warp, and one block per row
+  return std::max({fx::Pack<NP, 1, false>::DIGITS, fx::Pack<NP, 1, true>::DIGITS, fx::Pack<NP, 3, false>::DIGITS,
+                   fx::Pack<NP, 3, true>::DIGITS, fx::Pack<NP, 8, false>::DIGITS, fx::Pack<NP, 8, true>::DIGITS,
+                   fx::Pack<NP, 4, false>::DIGITS});
 }
 
 template <int NP, int MODE, bool WPR>
 __device__ __forceinline__ void fx_phase(const FxOp* op) {
   extern __shared__ __align__(16) int2 warp_digits[];   // [warps][most_digits]
+  static_assert(fx::Pack<NP, MODE, WPR>::DIGITS <= most_digits<NP>());
   int2* digits = warp_digits + (threadIdx.x >> 5) * most_digits<NP>();
   const FxOp q = *op;   // into registers
   bool waited = true;   // an ordinary launch
