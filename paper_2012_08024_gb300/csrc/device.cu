@@ -154,7 +154,7 @@ size_t layout(const cdg::Hierarchy& H, int precision, int nrhs, DeviceState* S, 
       const size_t nL = H.L_t[l].size();
       if (precision == 0) {
         L.Dinv = c.take<double>((size_t)L.n * nb2l);
-        if (nL) L.L = c.take<double>(nL);
+        if (nL && !fixed) L.L = c.take<double>(nL);
         L.Ahat = c.take<double>(Sh.val.size() + 1);
         if (fixed) {
           L.eD = c.take<unsigned short>((size_t)L.n * npl);
@@ -1249,20 +1249,13 @@ bool level_smooth_first(const DeviceState& D, const DevLevel& L, const T* b, T* 
   return launch_smooth_first<T>(L.np, L.n, opD<T>(L), b, bh, x, omega, s);
 }
 
-// b_{l+1} = R r_l and x_l (+)= L x_{l+1} inside the V-cycle
+// b_{l+1} = R r_l and x_l (+)= L x_{l+1}
 template <typename T>
 bool level_restrict(const DeviceState& D, int l, const T* r, T* bc, cudaStream_t s) {
   const DevLevel& F = D.lev[l];
   if constexpr (sizeof(T) == 8) {
     if (D.fixed && !F.ptrans) {
-      FxOp o;
-      o.mode = 8;
-      o.np = F.np;
-      o.n = D.lev[l + 1].n;
-      o.blocks = F.n;
-          o.rowptr = D.lev[l + 1].childptr;
-      o.A = F.Rx;
-      o.EA = F.eR;
+      FxOp o = restrict_op(F, D.lev[l + 1]);
       o.x = r;
       o.y = bc;
       return fx_run(o, s);
@@ -1986,8 +1979,8 @@ int dev_level_op(cdg_handle* h, int op, int level, const double* x, const double
     ok = level_smooth_first<double>(D, L, b, (double*)L.bh, (double*)nullptr, h->opt.omega, s) &&
          level_bsr<double>(D, L, 3, x, (const double*)L.bh, y, h->opt.omega, nullptr, s, aligned);
   }
-  else if (op == 3) ok = transfer_restrict<double>(D, level, L.L, x, y, s);
-  else ok = transfer_prolong<double>(D, level, L.L, x, y, true, s);
+  else if (op == 3) ok = level_restrict<double>(D, level, x, y, s);
+  else ok = level_prolong<double>(D, level, x, y, true, s);
   if (!ok) {
     h->err = "unsupported n_p";
     return CDG_EINVAL;

@@ -29,8 +29,8 @@ struct DevLevel {
   double* Dinv = nullptr;
   double* L = nullptr;
   // digit form (DeviceState::fixed): A, Ahat and Dinv then hold digits with the
-  // exponents eA, eH, eD of their blocks' rows; Lx / Rx are L_K and L_K^T in
-  // digits for the V-cycle's prolongation and restriction (L itself stays FP64)
+  // exponents eA, eH, eD of their blocks' rows, and Lx / Rx L_K and L_K^T in
+  // digits for the prolongation and the restriction, in the place of L
   unsigned short *eA = nullptr, *eH = nullptr, *eD = nullptr, *eL = nullptr, *eR = nullptr;
   double *Lx = nullptr, *Rx = nullptr;
   int *ell = nullptr, *hell = nullptr;   // columns of A and Ahat as [n][width], -1 behind a row's last
