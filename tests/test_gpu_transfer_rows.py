@@ -21,7 +21,7 @@ def test_rows_of_the_transfers(k):
     import torch
     from paper_2012_08024_gb300 import Solver
     make, p, kw = CASES[k]
-    S = Solver(make(), p=p, max_levels=3, **kw).bind()
+    S = Solver(make(), p=p, max_levels=6, **kw).bind()
     rng = np.random.default_rng(k)
     npb = S.np_
     for l in range(S.n_levels - 1):
