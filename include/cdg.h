@@ -141,8 +141,10 @@ typedef struct {
   int32_t persistent_vcycle; /* 1: each V-cycle is ONE cooperative persistent kernel whose CTAs
                                walk the cycle's phases with grid barriers (bounded waits; an
                                expired wait ends the solve with CDG_ETIMEOUT); used when every
-                               level has the same n_p (no p-multigrid degree steps), else the
-                               per-phase kernels.  0 (default): one kernel per phase. */
+                               level has the same n_p (no p-multigrid degree steps) and that is
+                               3, 4, 6 or 10, else the per-phase kernels.  Its phases are not
+                               fused: fuse_transfers concerns the per-phase kernels.
+                               0 (default): one kernel per phase. */
 } cdg_options;
 
 #define CDG_MAX_LEVELS 16

@@ -90,9 +90,16 @@ std::vector<int> padded_columns(const cdg::BSR& A, int width) {
   return o;
 }
 
-// The FP64 operators are kept in digit form (device_fixed.cu) unless an option asks for
-// kernels that read them as FP64 numbers.
-inline bool digit_form(const cdg_options& o) { return o.fuse_transfers == 0; }
+// The FP64 operators are kept in digit form (device_fixed.cu) unless an option asks for kernels that
+// read them as FP64 numbers: the fused transfers, where the V-cycle is not the persistent one (which
+// fuses nothing and has its FP64 phases in digits only).
+bool digit_form(const cdg_options& o, const cdg::Hierarchy& H) {
+  if (o.fuse_transfers == 0) return true;
+  if (o.persistent_vcycle == 0 || o.precision != 0 || !persistent_np(H.np)) return false;
+  for (int np : H.np_l)
+    if (np != H.np) return false;
+  return true;
+}
 
 // CTAs per segment of the vector kernels: kDotBlocks1 for one mesh (kDotBlocks over a batch), but no
 // more than leaves a thread four elements (one step of its loop): fewer partials to sum.
@@ -1415,8 +1422,9 @@ bool vcycle(DeviceState& D, const cdg_options& o, const T* b0, T* z0, cudaStream
     coarse_solve<T>(D, b0, z0, s);
     return true;
   }
-  const bool fuse = (o.fuse_transfers & 1) != 0;        // residual + restriction + first coarse step
-  const bool fuse_up = (o.fuse_transfers & 2) != 0;     // prolongation in the coarse level's last sweep
+  // the fused kernels have no digit form (persistent_vcycle whose launch was refused)
+  const bool fuse = !D.fixed && (o.fuse_transfers & 1) != 0;       // residual + restriction + first coarse step
+  const bool fuse_up = !D.fixed && (o.fuse_transfers & 2) != 0;    // prolongation in the coarse level's last sweep
   std::vector<const T*> bl(nlev);
   bl[0] = b0;
   for (int l = 1; l < nlev; ++l) bl[l] = (const T*)D.lev[l].b;
@@ -1689,7 +1697,7 @@ static int gmres_len(const cdg_options& o) { return o.krylov == 1 ? o.restart : 
 
 int dev_bytes(const cdg_handle* h, int64_t* bytes) {
   *bytes = (int64_t)layout(h->H, h->opt.precision == 2 ? 1 : h->opt.precision, h->opt.nrhs, nullptr, nullptr,
-                          h->opt.precision, gmres_len(h->opt), h->opt.maxit, h->opt.tc_fp64_apply, digit_form(h->opt));
+                          h->opt.precision, gmres_len(h->opt), h->opt.maxit, h->opt.tc_fp64_apply, digit_form(h->opt, h->H));
   return CDG_OK;
 }
 
@@ -1801,7 +1809,7 @@ int dev_bind(cdg_handle* h, void* buf, int64_t bytes, void* stream) {
   const int prec = h->opt.precision == 2 ? 1 : h->opt.precision;
   const int64_t need =
       (int64_t)layout(H, prec, h->opt.nrhs, nullptr, nullptr, h->opt.precision, gmres_len(h->opt), h->opt.maxit,
-                      h->opt.tc_fp64_apply, digit_form(h->opt));
+                      h->opt.tc_fp64_apply, digit_form(h->opt, h->H));
   if (bytes < need) {
     h->err = "device buffer too small: need " + std::to_string(need) + " bytes";
     return CDG_ENOMEM;
@@ -1816,7 +1824,7 @@ int dev_bind(cdg_handle* h, void* buf, int64_t bytes, void* stream) {
   D.base = (char*)buf;
   D.bytes = bytes;
   layout(H, prec, h->opt.nrhs, &D, (char*)buf, h->opt.precision, gmres_len(h->opt), h->opt.maxit,
-         h->opt.tc_fp64_apply, digit_form(h->opt));
+         h->opt.tc_fp64_apply, digit_form(h->opt, h->H));
   D.precision = h->opt.precision == 2 ? 1 : h->opt.precision;
   cudaStream_t s = (cudaStream_t)stream;
   const int nlev = D.nlev;

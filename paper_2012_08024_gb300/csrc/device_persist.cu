@@ -401,7 +401,7 @@ int launch_one(const PParams& P, cudaStream_t s, int* grid_out) {
 // count: two device words, cleared here; err: the device error flag.
 bool vcycle_persistent(DeviceState& D, const cdg_options& o, bool fp32, const void* b0, void* z0, unsigned* count,
                        int* err, cudaStream_t s) {
-  if (!fp32 && !D.fixed) return false;
+  if (!fp32 && !D.fixed) return false;   // FP64 phases in digits; digit_form keeps them where this cycle runs
   PParams P = {};
   P.nlev = D.nlev;
   P.nu_pre = o.nu_pre;

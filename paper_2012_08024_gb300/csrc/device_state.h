@@ -218,7 +218,8 @@ void mr_upload(const cdg::Hierarchy& H, MR& M, cudaStream_t s);
 int dev_apply_multi(cdg_handle* h, const double* x, double* y, void* stream);
 
 // device_persist.cu: one V-cycle as one cooperative persistent launch (false: not applicable
-// to this hierarchy, or the launch was refused)
+// to this hierarchy, or the launch was refused), built for these n_p
+inline bool persistent_np(int np) { return np == 3 || np == 4 || np == 6 || np == 10; }
 bool vcycle_persistent(DeviceState& D, const cdg_options& o, bool fp32, const void* b0, void* z0, unsigned* count,
                        int* err, cudaStream_t s);
 
