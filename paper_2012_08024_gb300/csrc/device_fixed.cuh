@@ -107,7 +107,8 @@ struct Acc {
 // (hi 2^60 + lo) 2^(e - 116), rounded once; e = EA + EX of the digits' scales (+ kHead after Wide::down by it)
 __device__ __forceinline__ double fx_value(long long hi, unsigned long long lo, int e) {
   const int k = min(60, __clzll(hi ^ (hi >> 63)) - 1);   // low bits that fit beside hi in 63 bits
-  const long long v = (long long)((unsigned long long)hi << k) | (long long)(lo >> (60 - k));
+  long long v = (long long)((unsigned long long)hi << k) | (long long)(lo >> (60 - k));
+  if (k < 60 && (lo << (4 + k)) != 0) v |= 1;   // the bits that did not fit, so that no tie is seen where there is none
   return scale2(__ll2double_rn(v), e - 56 - k);
 }
 
