@@ -91,14 +91,12 @@ std::vector<int> padded_columns(const cdg::BSR& A, int width) {
 }
 
 // The FP64 operators are kept in digit form (device_fixed.cu) unless an option asks for kernels that
-// read them as FP64 numbers: the fused transfers, where the V-cycle is not the persistent one (which
-// fuses nothing and has its FP64 phases in digits only).
+// read them as FP64 numbers: the fused transfers, or the persistent V-cycle (which fuses nothing) on a
+// large fine level.
 bool digit_form(const cdg_options& o, const cdg::Hierarchy& H) {
-  if (o.fuse_transfers == 0) return true;
-  if (o.persistent_vcycle == 0 || o.precision != 0 || !persistent_np(H.np)) return false;
-  for (int np : H.np_l)
-    if (np != H.np) return false;
-  return true;
+  bool persistent = o.persistent_vcycle != 0 && o.precision == 0 && persistent_np(H.np);
+  for (int np : H.np_l) persistent = persistent && np == H.np;
+  return persistent ? persistent_digits(H.np, H.A_t[0].nrows) : o.fuse_transfers == 0;
 }
 
 // CTAs per segment of the vector kernels: kDotBlocks1 for one mesh (kDotBlocks over a batch), but no

@@ -18,6 +18,7 @@
 
 #include <algorithm>
 #include <cstdint>
+#include <type_traits>
 
 #include "device_fixed.cuh"
 #include "device_kernels.cuh"
@@ -179,10 +180,9 @@ __device__ void ph_coarse(const PParams& P, const T* b, T* x, bool add) {
   }
 }
 
-// FP64: a product in digit form, by the same packs as the per-phase kernels.  Three CTAs per SM:
-// V-cycle of the 181^2 (p = 2) mesh 324 -> 278 us against FP64 blocks, 32^2 137 -> 121 us, but the
-// 64-mesh batch 63.5 -> 76.6 ms per solve (its phases wait for memory, and 24 warps per SM hide less
-// than the 40 of the FP64-block kernel; 66.4 ms with the later CG kernels); two CTAs 265 us, 102 us, 80.3 ms.
+// FP64: a product in digit form, by the same packs as the per-phase kernels.  Two CTAs per SM (128
+// registers) at n_p = 10, where three spill: solves of 256^2 (p = 3) 60.7 against 78.2 ms; three below
+// (72.0 against 72.6 ms for 64 meshes at p = 2, four 83.6).
 template <int NP>
 constexpr int most_digits() {
   // of the modes that the phases run: 1, 3 and 8 packed or with a row per warp, and one block per row
@@ -227,7 +227,7 @@ __device__ __forceinline__ void for_rows(int n, F&& f) {
   for (int K = (int)(blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5)); K < n; K += warps) f(K);
 }
 
-// the phases in the precision of the cycle
+// the phases on FP32 or FP64 blocks
 template <typename T, int NP>
 struct Phase {
   static constexpr bool VEC = NP % 2 == 0;
@@ -272,8 +272,9 @@ struct Phase {
   }
 };
 
+// the FP64 phases in digit form
 template <int NP>
-struct Phase<double, NP> {
+struct FxPhase {
   static __device__ void first(const PLevel& L, const double* b, double* bh, double* x, double w, bool write_x) {
     if (write_x) fx_product<NP, 6>(L.oD, false, b, nullptr, bh, x, w);
     else fx_product<NP, 7>(L.oD, false, b, nullptr, bh, nullptr, w);
@@ -293,9 +294,14 @@ struct Phase<double, NP> {
   }
 };
 
-template <typename T, int NP>
-__global__ void __launch_bounds__(kPThreads, 3) vcycle_persistent_kernel(const __grid_constant__ PParams P) {
-  using Ph = Phase<T, NP>;
+// CTAs per SM that the registers are held to
+template <typename T, int NP, bool FX>
+constexpr int persistent_ctas() { return FX ? (NP >= 10 ? 2 : 3) : sizeof(T) == 8 ? 5 : 3; }
+
+template <typename T, int NP, bool FX>
+__global__ void __launch_bounds__(kPThreads, persistent_ctas<T, NP, FX>())
+    vcycle_persistent_kernel(const __grid_constant__ PParams P) {
+  using Ph = std::conditional_t<FX, FxPhase<NP>, Phase<T, NP>>;
   const T w = (T)P.omega;
   const int nlev = P.nlev;
   // where each level's iterate is at the end of its downward (x_down) and upward (x_fin) visit
@@ -368,11 +374,11 @@ __global__ void __launch_bounds__(kPThreads, 3) vcycle_persistent_kernel(const _
 #undef CDG_SYNC
 }
 
-template <typename T, int NP>
+template <typename T, int NP, bool FX>
 int launch_one(const PParams& P, cudaStream_t s, int* grid_out) {
-  auto kern = vcycle_persistent_kernel<T, NP>;
+  auto kern = vcycle_persistent_kernel<T, NP, FX>;
   int per_sm = 0;
-  const size_t smem = sizeof(T) == 8 ? (kPThreads / 32) * most_digits<NP>() * sizeof(int2) : 0;
+  const size_t smem = FX ? (kPThreads / 32) * most_digits<NP>() * sizeof(int2) : 0;
   if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, kPThreads, smem) != cudaSuccess || per_sm < 1)
     return -1;
   int dev = 0, sms = 0;
@@ -401,7 +407,7 @@ int launch_one(const PParams& P, cudaStream_t s, int* grid_out) {
 // count: two device words, cleared here; err: the device error flag.
 bool vcycle_persistent(DeviceState& D, const cdg_options& o, bool fp32, const void* b0, void* z0, unsigned* count,
                        int* err, cudaStream_t s) {
-  if (!fp32 && !D.fixed) return false;   // FP64 phases in digits; digit_form keeps them where this cycle runs
+  const bool fx = !fp32 && D.fixed;
   PParams P = {};
   P.nlev = D.nlev;
   P.nu_pre = o.nu_pre;
@@ -432,7 +438,7 @@ bool vcycle_persistent(DeviceState& D, const cdg_options& o, bool fp32, const vo
     Q.wprA = warp_per_row(L.np, L.n, L.nnzb);
     Q.wprH = warp_per_row(L.np, L.n, L.hnnzb);
     Q.wprR = l + 1 < D.nlev && warp_per_row(L.np, D.lev[l + 1].n, L.n);
-    if (!fp32) {
+    if (fx) {
       const bool last = l + 1 == D.nlev;
       Q.oA = operator_op(L, 1);
       if (!last) {
@@ -455,11 +461,16 @@ bool vcycle_persistent(DeviceState& D, const cdg_options& o, bool fp32, const vo
   P.wait_limit = D.wait_limit < 0 ? kBarrierLimit : std::min(D.wait_limit, kBarrierLimit);
   cudaMemsetAsync(count, 0, 2 * sizeof(unsigned), s);
   int grid = 0, rc = -1;
+  auto run = [&](auto np) {
+    constexpr int NP = decltype(np)::value;
+    if (fp32) return launch_one<float, NP, false>(P, s, &grid);
+    return fx ? launch_one<double, NP, true>(P, s, &grid) : launch_one<double, NP, false>(P, s, &grid);
+  };
   switch (D.np) {
-    case 3: rc = fp32 ? launch_one<float, 3>(P, s, &grid) : launch_one<double, 3>(P, s, &grid); break;
-    case 4: rc = fp32 ? launch_one<float, 4>(P, s, &grid) : launch_one<double, 4>(P, s, &grid); break;
-    case 6: rc = fp32 ? launch_one<float, 6>(P, s, &grid) : launch_one<double, 6>(P, s, &grid); break;
-    case 10: rc = fp32 ? launch_one<float, 10>(P, s, &grid) : launch_one<double, 10>(P, s, &grid); break;
+    case 3: rc = run(std::integral_constant<int, 3>()); break;
+    case 4: rc = run(std::integral_constant<int, 4>()); break;
+    case 6: rc = run(std::integral_constant<int, 6>()); break;
+    case 10: rc = run(std::integral_constant<int, 10>()); break;
     default: return false;
   }
   if (rc != 0) return false;

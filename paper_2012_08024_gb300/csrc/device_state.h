@@ -220,6 +220,12 @@ int dev_apply_multi(cdg_handle* h, const double* x, double* y, void* stream);
 // device_persist.cu: one V-cycle as one cooperative persistent launch (false: not applicable
 // to this hierarchy, or the launch was refused), built for these n_p
 inline bool persistent_np(int np) { return np == 3 || np == 4 || np == 6 || np == 10; }
+// Whether its FP64 phases run in digits (n elements on level 0) or on FP64 blocks.  A phase of many rows waits
+// for memory, and the digit phases, at two or three CTAs per SM, hide less than the five of the FP64-block
+// kernel: solves at n_p = 6, 131,072 rows 35.6 ms in digits, 33.7 on FP64 blocks; 64 meshes of 356,730 rows
+// 71.0 and 61.1; n_p = 3, 524,288 rows 48.6 and 41.8; but n_p = 6, 8,192 rows 11.1 and 12.8, and n_p = 10,
+// 24,576 rows of tetrahedra 22.7 and 28.5, 131,072 of triangles 60.5 and 63.6.
+inline bool persistent_digits(int np, int64_t n) { return np >= 10 || n <= 20000; }
 bool vcycle_persistent(DeviceState& D, const cdg_options& o, bool fp32, const void* b0, void* z0, unsigned* count,
                        int* err, cudaStream_t s);
 

@@ -77,3 +77,22 @@ def test_solves_of_meshes_of_different_scale(kw):
         S.to_tree(um.reshape(-1), x)
         b, x = b.cpu().numpy(), x.cpu().numpy()
         assert np.linalg.norm(b - A @ x) <= 2e-10 * np.linalg.norm(b), m
+
+
+@pytest.mark.parametrize("p", [1, 2])
+@pytest.mark.parametrize("scale", [2.0 ** 100, 2.0 ** -100, 0.0])
+def test_persistent_cycle_on_fp64_blocks(p, scale):
+    """More than 20,000 elements: the persistent kernel on FP64 blocks."""
+    import torch
+    B = _batch(p, (105, 106), persistent_vcycle=True)
+    cut, n = int(B.elem_offsets[1]) * B.np_, B.info["n_dofs"]
+    r = np.random.default_rng(p).standard_normal(n)
+    z = []
+    for s in (1.0, scale):
+        rs = r.copy()
+        rs[:cut] *= s
+        out = torch.empty(n, dtype=torch.float64, device="cuda")
+        B.vcycle(torch.tensor(rs, device="cuda"), out)
+        z.append(out.cpu().numpy())
+    assert np.array_equal(z[1][cut:], z[0][cut:])
+    assert np.array_equal(z[1][:cut], scale * z[0][:cut])
