@@ -648,7 +648,7 @@ __global__ void __launch_bounds__(kThreads) dot_kernel(const long long* __restri
 
 // The sum of the n partials p, in every thread of the CTA and in an order that depends on n only: every
 // CTA that forms it gets the same bits.  Up to four warps add (see cta_sum).
-__device__ __forceinline__ double partials_sum(const double* __restrict__ p, int n) {
+__device__ __forceinline__ double partials_sum(const double* p, int n) {
   __shared__ double part[4];
   const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int used = n > 64 ? 4 : 1;

@@ -148,7 +148,7 @@ struct VecLoad<double, NP, A> {
 // block and column by column (the same order for every UNR).
 template <typename T, int NP, bool VEC, int UNR, bool COHERENT = false>
 __device__ __forceinline__ T row_acc(int K, int i, const int* __restrict__ rowptr, const int* __restrict__ col,
-                                     const T* __restrict__ A, const T* __restrict__ x) {
+                                     const T* __restrict__ A, const T* x) {
   constexpr Access X = COHERENT ? kCoherent : kPlain;
   T acc = T(0);
   const int b0 = rowptr[K], b1 = rowptr[K + 1];
@@ -223,7 +223,7 @@ __device__ __forceinline__ double cta_sum(double v, double* red) {
 // of the groups are added in a fixed order.  Valid in the lanes of group 0.  x aligned for VecLoad.
 template <typename T, int NP, bool COHERENT = false>
 __device__ __forceinline__ T split_row_acc(int K, const int* __restrict__ rowptr, const int* __restrict__ col,
-                                           const T* __restrict__ A, const T* __restrict__ x) {
+                                           const T* __restrict__ A, const T* x) {
   constexpr int G = 32 / NP;
   constexpr Access X = COHERENT ? kCoherent : kPlain;
   const int lane = threadIdx.x & 31;
@@ -278,7 +278,7 @@ __device__ __forceinline__ void touch_row(int K, const int* __restrict__ rowptr,
 // of the warp in the same way; valid in the lanes of group 0.
 template <typename T, int NP, bool COHERENT = false>
 __device__ __forceinline__ T split_restrict(int Ag, const int* __restrict__ childptr, const T* __restrict__ L,
-                                            const T* __restrict__ r) {
+                                            const T* r) {
   constexpr int G = 32 / NP;
   constexpr Access X = COHERENT ? kCoherent : kPlain;
   const int lane = threadIdx.x & 31;
