@@ -1859,13 +1859,13 @@ int dev_bind(cdg_handle* h, void* buf, int64_t bytes, void* stream) {
     // every synchronous upload above finishes before the host vectors die
     cudaStreamSynchronize(s);
   }
-  if (D.lev[0].Adig) {
-    upload(D.lev[0].Adig, H.A_t[0].val, s);
-    fx_encode(D.lev[0].np, D.lev[0].nnzb, D.lev[0].Adig, D.lev[0].eA, s);
-  }
-  if (D.fixed) {   // FP64 blocks to digits
+  {   // FP64 blocks to digits
     bool ok = true;
-    for (int l = 0; l < nlev; ++l) {
+    if (D.lev[0].Adig) {
+      upload(D.lev[0].Adig, H.A_t[0].val, s);
+      ok = fx_encode(D.lev[0].np, D.lev[0].nnzb, D.lev[0].Adig, D.lev[0].eA, s);
+    }
+    for (int l = 0; D.fixed && l < nlev; ++l) {
       const DevLevel& L = D.lev[l];
       if (L.A) ok = ok && fx_encode(L.np, L.nnzb, L.A, L.eA, s);
       if (L.Ahat) ok = ok && fx_encode(L.np, L.hnnzb, L.Ahat, L.eH, s);
