@@ -714,7 +714,6 @@ __global__ void __launch_bounds__(kThreads) cg_update_kernel(const long long* __
     alpha_s = done || !(tot > 0.0) ? 0.0 : rz / tot;
     if (blockIdx.x == (unsigned)(seg * bps)) {
       sc[S_PQ] = tot;
-      sc[S_ALPHA] = alpha_s;
       sc[S_RZ] = rz;
       if (!done && !(tot > 0.0)) sc[S_BREAK] = 1.0;   // S_DONE follows in cg_check_kernel: CTAs still read it
     }
@@ -858,10 +857,7 @@ __global__ void __launch_bounds__(kThreads) cg_p_kernel(const long long* __restr
     beta_s = first || sc[S_DONE] != 0.0 ? 0.0
              : sizeof(TZ) == 4          ? (tot - sc[S_RZO]) / sc[S_RZ]
                                         : tot / sc[S_RZ];
-    if (blockIdx.x == (unsigned)(seg * bps)) {
-      sc[S_BETA] = beta_s;
-      sc[S_RZN] = tot;
-    }
+    if (blockIdx.x == (unsigned)(seg * bps)) sc[S_RZN] = tot;
   }
   __syncthreads();
   const double beta = beta_s;

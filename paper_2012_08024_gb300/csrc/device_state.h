@@ -14,7 +14,8 @@ constexpr int kDotBlocks = 8 * 152;   // fixed grid of the vector kernels of bat
 constexpr int kDotBlocks1 = 2 * 152;  // the same for single-mesh handles (their dot partials: 2 CTAs per SM)
 
 // per-segment CG scalars (one row of S_COUNT doubles per mesh of the handle)
-// S_HDONE: the segment's residual history is closed (single-graph solve); S_RZO: the new r times the
+// S_ALPHA, S_BETA: many-column solves (others keep theirs in the kernels); S_HDONE: the segment's residual
+// history is closed (single-graph solve); S_RZO: the new r times the
 // previous z (Polak-Ribiere); S_RZN: r.z as the direction update leaves it, S_RZ from the next update on
 enum Scal { S_RZ = 0, S_PQ, S_RR, S_BB, S_ALPHA, S_BETA, S_DONE, S_BREAK, S_IT, S_HDONE, S_RZO, S_RZN, S_FLAG = 15, S_COUNT = 16 };
 
