@@ -253,14 +253,6 @@ __device__ __forceinline__ double fx_pack(const FxOp& q, int pack, int2* __restr
       if constexpr (MODE == 1 || MODE == 3) bo = vload<COHERENT>(q.b + o);
     }
   };
-  if constexpr (!WPR && !ONE && NP <= 6) {
-    // the pack's digits, all of them, towards L1 (32 warps' packs fit there up to n_p = 6): a lane only
-    // holds one block's row at a time.  64 meshes at p = 2: 50.8 -> 49.9 ms; n_p = 10: no gain
-    const int last = __reduce_max_sync(0xffffffffu, b0 + nb), begin = __shfl_sync(0xffffffffu, b0, 0);
-    const char* a1 = reinterpret_cast<const char*>(A + (size_t)last * NP * NP);
-    for (const char* a = reinterpret_cast<const char*>(A + (size_t)begin * NP * NP) + lane * 128; a < a1; a += 4096)
-      asm volatile("prefetch.global.L1 [%0];" ::"l"(a));
-  }
   if (maxc == 0) inputs();
   for (int base = 0; base < maxc; base += CH) {
     int J[CH];
