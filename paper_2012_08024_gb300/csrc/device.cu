@@ -90,13 +90,25 @@ std::vector<int> padded_columns(const cdg::BSR& A, int width) {
   return o;
 }
 
-// The FP64 operators are kept in digit form (device_fixed.cu) unless an option asks for kernels that
-// read them as FP64 numbers: the fused transfers, or the persistent V-cycle (which fuses nothing) on a
-// large fine level.
-bool digit_form(const cdg_options& o, const cdg::Hierarchy& H) {
+// Which levels keep their FP64 operators in digit form (device_fixed.cu): none where an option asks for
+// kernels that read them as FP64 numbers (the fused transfers, or the persistent V-cycle, which fuses
+// nothing, on a large fine level); all of them for the persistent V-cycle in digits; else by level.
+enum Form { kBlocks, kByLevel, kDigits };
+
+Form digit_form(const cdg_options& o, const cdg::Hierarchy& H) {
   bool persistent = o.persistent_vcycle != 0 && o.precision == 0 && persistent_np(H.np);
   for (int np : H.np_l) persistent = persistent && np == H.np;
-  return persistent ? persistent_digits(H.np, H.A_t[0].nrows) : o.fuse_transfers == 0;
+  if (persistent) return persistent_digits(H.np, H.A_t[0].nrows) ? kDigits : kBlocks;
+  return o.fuse_transfers == 0 ? kByLevel : kBlocks;
+}
+
+// By level: digits from n_p = 6 on, where the FP64 pipe is what bounds products of FP64 blocks, and where
+// rows take a warp each; not on levels of many rows at n_p = 3 and 4, whose few products per value that
+// is gathered do not pay for its digits.  Products with A, FP64 blocks against digits: n_p = 3, 720,000
+// rows 55 and 87 us, 10,001 rows 5.3 and 5.4, 2,527 rows 5.3 and 3.3; n_p = 4, 384,000 rows 56 and 71, 2,837
+// rows 7.2 and 4.1; n_p = 6, 405,000 rows 111 and 100; n_p = 10, 131,072 rows 100 and 75.
+bool level_digits(Form form, int np, const cdg::BSR& A) {
+  return form == kDigits || (form == kByLevel && (np >= 6 || warp_per_row(np, (int)A.nrows, A.nnzb())));
 }
 
 // CTAs per segment of the vector kernels: kDotBlocks1 for one mesh (kDotBlocks over a batch), but no
@@ -107,7 +119,7 @@ int vector_ctas(int64_t ndofs, int nseg) {
 }
 
 size_t layout(const cdg::Hierarchy& H, int precision, int nrhs, DeviceState* S, char* base, int mr_precision,
-              int gmres_m, int maxit, int tc_fp64, bool fixed) {
+              int gmres_m, int maxit, int tc_fp64, Form form) {
   Carver c{base};
   const int np = H.np;
   const int nlev = (int)H.lev.size();
@@ -124,7 +136,7 @@ size_t layout(const cdg::Hierarchy& H, int precision, int nrhs, DeviceState* S, 
   D.ndofs = ne * np;
   D.nbf = (int64_t)H.mesh.bf_K.size();
   D.precision = precision;
-  D.fixed = fixed;
+  D.fixed = form != kBlocks;
   const size_t vsz = precision ? sizeof(float) : sizeof(double);
   D.nrhs = nrhs;
   for (int l = 0; l < nlev; ++l) {
@@ -136,6 +148,8 @@ size_t layout(const cdg::Hierarchy& H, int precision, int nrhs, DeviceState* S, 
     L.np = npl;
     L.ptrans = l + 1 < nlev && H.L_t[l].empty();
     L.nnzb = A.nnzb();
+    // the many-column apply reads A_0 in digits whatever its n_p
+    const bool fixed = L.fixed = level_digits(form, npl, A) || (form != kBlocks && l == 0 && nrhs > 0);
     L.rowptr = c.take<int>(A.nrows + 1);
     L.col = c.take<int>(A.nnzb());
     const bool last = l + 1 == nlev;
@@ -1202,7 +1216,7 @@ bool level_bsr(const DeviceState& D, const DevLevel& L, int mode, const T* x, co
   const int* cl = hat ? L.hcol : L.col;
   if (unr == 0) unr = unr_of<T>(L, mode);
   if constexpr (sizeof(T) == 8) {
-    if (D.fixed) {
+    if (L.fixed) {
       FxOp o = operator_op(L, mode);
       o.x = x;
       o.b = b;
@@ -1238,7 +1252,7 @@ template <typename T>
 bool level_smooth_first(const DeviceState& D, const DevLevel& L, const T* b, T* bh, T* x, double omega,
                         cudaStream_t s) {
   if constexpr (sizeof(T) == 8) {
-    if (D.fixed) {
+    if (L.fixed) {
       FxOp o = diagonal_op(L, x ? 6 : 7, L.Dinv, L.eD);
       o.x = b;
       o.y = bh;
@@ -1255,13 +1269,14 @@ template <typename T>
 bool level_restrict(const DeviceState& D, int l, const T* r, T* bc, cudaStream_t s) {
   const DevLevel& F = D.lev[l];
   if constexpr (sizeof(T) == 8) {
-    if (D.fixed && !F.ptrans) {
+    if (F.fixed && !F.ptrans) {
       FxOp o = restrict_op(F, D.lev[l + 1]);
       o.x = r;
       o.y = bc;
       return fx_run(o, s);
     }
-  } else if (!F.ptrans && F.np <= 15 && warp_per_row(F.np, D.lev[l + 1].n, F.n)) {
+  }
+  if (!F.ptrans && F.np <= 15 && warp_per_row(F.np, D.lev[l + 1].n, F.n)) {
     const int nc = D.lev[l + 1].n;
     const unsigned g = (unsigned)((nc + kRowThreads / 32 - 1) / (kRowThreads / 32));
     const int* cp = D.lev[l + 1].childptr;
@@ -1281,7 +1296,7 @@ template <typename T>
 bool level_prolong(const DeviceState& D, int l, const T* xc, T* x, bool add, cudaStream_t s) {
   const DevLevel& F = D.lev[l];
   if constexpr (sizeof(T) == 8) {
-    if (D.fixed && !F.ptrans) {
+    if (F.fixed && !F.ptrans) {
       FxOp o = prolong_op(F, add ? 4 : 7);
       o.x = xc;
       o.y = x;
@@ -1480,7 +1495,7 @@ bool vcycle(DeviceState& D, const cdg_options& o, const T* b0, T* z0, cudaStream
       if (carry && k + 1 == o.nu_post) {
         if (!launch_smooth_prolong<T>(D, l - 1, x, (const T*)L.bh, out, w, o.nu_pre >= 1, s, flag)) return false;
         prolonged[l - 1] = 1;
-      } else if (out == z0 && dot && D.fixed && sizeof(T) == 8) {
+      } else if (out == z0 && dot && L.fixed && sizeof(T) == 8) {
         FxOp q = operator_op(L, 3);
         q.x = (const double*)x;
         q.b = (const double*)L.bh;
@@ -1739,7 +1754,7 @@ static int autotune_bsr(cdg_handle* h, cudaStream_t s) {
   };
   // odd n_p and operators in digit form: those kernels have no variants (levels keep the default)
   // level 0, FP64: the outer apply and residual
-  if (D.lev[0].np % 2 == 0 && !D.fixed) {
+  if (D.lev[0].np % 2 == 0 && !D.lev[0].fixed) {
     DevLevel& L = D.lev[0];
     const size_t nb = sizeof(double) * (size_t)D.ndofs;
     cudaMemsetAsync(D.p, 0, nb, s);
@@ -1754,7 +1769,7 @@ static int autotune_bsr(cdg_handle* h, cudaStream_t s) {
   auto tune_level = [&](auto zero, DevLevel& L, int l) {
     using T = decltype(zero);
     const int np = L.np;
-    if (np % 2 != 0 || (sizeof(T) == 8 && D.fixed)) return;
+    if (np % 2 != 0 || (sizeof(T) == 8 && L.fixed)) return;
     const int ti = sizeof(T) == 8 ? 0 : 1;
     const size_t nb = sizeof(T) * (size_t)L.n * np;
     T *x = (T*)L.x, *b = (T*)L.b, *bh = (T*)L.bh, *y = (T*)L.t;
@@ -1861,8 +1876,9 @@ int dev_bind(cdg_handle* h, void* buf, int64_t bytes, void* stream) {
       upload(D.lev[0].Adig, H.A_t[0].val, s);
       ok = fx_encode(D.lev[0].np, D.lev[0].nnzb, D.lev[0].Adig, D.lev[0].eA, s);
     }
-    for (int l = 0; D.fixed && l < nlev; ++l) {
+    for (int l = 0; l < nlev; ++l) {
       const DevLevel& L = D.lev[l];
+      if (!L.fixed) continue;
       if (L.A) ok = ok && fx_encode(L.np, L.nnzb, L.A, L.eA, s);
       if (L.Ahat) ok = ok && fx_encode(L.np, L.hnnzb, L.Ahat, L.eH, s);
       if (L.Dinv) ok = ok && fx_encode(L.np, L.n, L.Dinv, L.eD, s);
@@ -2073,7 +2089,7 @@ static int cg_part1(cdg_handle* h, cudaStream_t s, const cudaGraphConditionalHan
   // p.q: by the apply itself where one mesh makes every CTA's partial the mesh's
   int cnt = D.bps;
   if (D.nseg == 1) {
-    cnt = (int)(D.fixed ? fx_grid(operator_op(L0, 0)) : rows_grid(L0.n, D.np));
+    cnt = (int)(L0.fixed ? fx_grid(operator_op(L0, 0)) : rows_grid(L0.n, D.np));
     level_bsr<double>(D, L0, 0, D.p, (const double*)nullptr, D.q, h->opt.omega, D.partial_pq, s);
   } else {
     level_bsr<double>(D, L0, 0, D.p, (const double*)nullptr, D.q, h->opt.omega, nullptr, s);

@@ -932,7 +932,7 @@ bool mr_apply64(DeviceState& D, MR& M, const double* x, double* y, cudaStream_t 
                     pq_groups ? M.partial : nullptr, pq_groups, M.tc_err, D.wait_limit, s);
   const int br = rows ? rows : rows_of(M, 0, 0);
   const dim3 grid((unsigned)((L0.n + br - 1) / br), (unsigned)((M.R + 31) / 32)), block(32, (unsigned)br);
-  const int2* A = reinterpret_cast<const int2*>(D.fixed ? L0.A : L0.Adig);
+  const int2* A = reinterpret_cast<const int2*>(L0.fixed ? L0.A : L0.Adig);
   MR_NP_DISPATCH(D.np, mr_fx_kernel<NP><<<grid, block, 0, s>>>(L0.n, M.R, L0.rowptr, L0.col, A, L0.eA, x, y));
   count_launch();
   return true;

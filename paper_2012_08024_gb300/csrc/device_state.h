@@ -29,9 +29,10 @@ struct DevLevel {
   double* A = nullptr;
   double* Dinv = nullptr;
   double* L = nullptr;
-  // digit form (DeviceState::fixed): A, Ahat and Dinv then hold digits with the
+  // digit form (fixed): A, Ahat and Dinv then hold digits with the
   // exponents eA, eH, eD of their blocks' rows, and Lx / Rx L_K and L_K^T in
   // digits for the prolongation and the restriction, in the place of L
+  bool fixed = false;
   unsigned short *eA = nullptr, *eH = nullptr, *eD = nullptr, *eL = nullptr, *eR = nullptr;
   double *Lx = nullptr, *Rx = nullptr;
   int *ell = nullptr, *hell = nullptr;   // columns of A and Ahat as [n][width], -1 behind a row's last
@@ -66,7 +67,7 @@ struct DeviceState {
   int64_t bytes = 0;
   int nlev = 0, np = 0, d = 0, nq = 0, nfq = 0, precision = 0;
   int64_t ne = 0, ndofs = 0, nbf = 0;
-  bool fixed = false;   // FP64 operators in digit form (device_fixed.cu)
+  bool fixed = false;   // FP64 operators of some levels or all in digit form (device_fixed.cu)
   DevLevel lev[kMaxLev];
   double* coarse_inv = nullptr;
   int nc = 0;

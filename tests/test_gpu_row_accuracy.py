@@ -5,7 +5,8 @@ Bound of a scalar row (NumPy's long double is the exact reference: 64 bits and m
 entry a of A is off by at most 2^-58 M, M the largest |a| of its scalar row in the block (2^-59 of the power
 of two above it), and a value of x by at most 2^-58 X, X the largest |x| of the neighbour; so the n_p products of
 the block by 2^-57 n_p M X; what the blocks' sums lose when they are added is below 2^-90 of that, and the
-result is rounded once."""
+result is rounded once.  Levels of many rows at n_p = 3 and 4 hold FP64 blocks: T fused multiply-adds in a row
+are off by at most T 2^-53 sum |a| |x| to first order."""
 import numpy as np
 import pytest
 
@@ -58,6 +59,8 @@ def test_rows_of_the_operators(k, kappa):
             S.apply(level, torch.tensor(x.reshape(-1), device="cuda"), y)
             want, bound, size = exact_rows(e, x)
             off = np.abs(y.cpu().numpy().reshape(n, npb) - want).astype(float)
+            if npb < 6 and n > 4864:
+                bound = (npb * np.diff(e["rowptr"])[:, None] + 1) * 2.0 ** -53 * size
             assert np.all(off <= bound), (level, v, (off / bound).max())
 
 
