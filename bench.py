@@ -53,12 +53,12 @@ HBM_FALLBACK_GBS = 6800.0           # profiling-recipe fallback when no measured
 # x 2 flops x 2.07 GHz; the roofline divides by the rate the FMA probe measures in the same run
 FP64_DERIVED_TFLOPS = 152 * 2 * 2 * 2.07e9 / 1e12
 # DRAM bytes (read + write) of one level-0 apply as ncu captured them on the 256 x 256 p = 3
-# square (523,264 blocks): FP64 not captured since its kernel changed, FP32
+# square (523,264 blocks): FP64 453,168,640 (profiles/fx_kernel_sweep_tri256_p3.md), FP32
 # 223,440,896 (profiles/bsr_kernel_tri256_p3_fp32.md).  Other squares at p = 3 report them scaled by
 # their level-0 block count (the traffic is 1.003-1.005x the algorithmic bytes, which grow with
 # the blocks); other workloads report null.  Set to None whenever the kernel changes, until it is
 # captured again.
-CAPTURED_APPLY = {"blocks": 523_264, "fp64": None, "fp32": 223_440_896}
+CAPTURED_APPLY = {"blocks": 523_264, "fp64": 453_168_640, "fp32": 223_440_896}
 
 
 def apply_traffic(kind, p, nnzb0, dtype):
@@ -615,8 +615,8 @@ def main():
     k_us = e0.elapsed_time(e1) / reps * 1e3
     nnzb0 = S.info["nnzb_l"][0]
     npb = S.np_
-    # digits of the blocks, padded columns (dim + 2 per row), row pointers, row exponents, x and y
-    alg_bytes = (nnzb0 * npb * npb * 8 + S.ne * (S.info["dim"] + 2) * 4 + (S.ne + 1) * 4 + S.ne * npb * 4 +
+    # digits of the blocks and the exponents of their rows, padded columns (dim + 2 per row), row pointers, x and y
+    alg_bytes = (nnzb0 * npb * npb * 8 + S.ne * (S.info["dim"] + 2) * 4 + (S.ne + 1) * 4 + nnzb0 * npb * 2 +
                  2 * ndof * 8)
     achieved = alg_bytes / (k_us * 1e-6) / 1e9
     peak, peak_src = peaks()

@@ -24,16 +24,16 @@
 // and a mesh of a batch whose data were small beside its neighbour's got a wrong
 // solution.  Now a row is off by no more than 2^-57 n_p sum_J max|a_J| max|x_J|
 // and one rounding.  It costs 0-5% (against the wider exponents: apply of 256^2,
-// p = 3, 72.5 -> 75.0 us; V-cycle of 128^2, p = 3, 199 -> 196 us; 64 meshes at
-// p = 2 52.5 -> 54.3 ms; 101^2 at p = 1 7.0 -> 7.3 ms).
+// p = 3, 72.6 -> 75.4 us; V-cycle of 128^2, p = 3, 198 -> 196 us; 64 meshes at
+// p = 2 52.2 -> 53.3 ms; 32^2 at p = 2 4.24 -> 4.36 ms).
 // Why 58 bits and not fewer: A x cancels for smooth x, where the small
 // constant-mode entries of A meet the largest values of x.  On solutions of the
 // 32^2 (p = 1, 2, 3) and 6^3 (p = 1, 2) meshes FP64 sums are 0.3-3.1e-12 off in
 // the 2-norm, the digits 0.01-0.36e-12, with kappa from 1e-4 to 1e4 at random
 // (24^2, p = 2, 3) 3.3-8.1e-9 against 0.1-0.4e-9, random vectors 0.8-1.9e-16
 // against 0.5e-16; relative to sum |a| |x| of its own row the worst row of these
-// is 7e-16 off with FP64 sums and 4e-15 with digits.  V-cycles (48^2, p = 1, 2,
-// 3, random r): 0.3-1.2e-12 against 0.4-38e-15.
+// is 7e-16 off with FP64 sums and 4e-15 with digits.  V-cycles of random r against
+// the exact cycle: 128^2, p = 3, 0.9-1.2e-12 and 0.9-1.4e-13, 64^2, p = 2, 2.3-5.5e-13 and 1.9-3.1e-14.
 //
 // The sums, over the T <= 28 terms of a block: |sum al xl| <= 2^58 T,
 // |sum (ah xl + al xh)| <= 2^58 T; both are then carried into the next higher
@@ -49,8 +49,8 @@
 // pointers.  The kernel waits for memory (issue slots a third used), so resident
 // warps count: 64 registers, 32 warps per SM.  Measured, 131,072 rows of 4
 // blocks at n_p = 10: apply 102.7 -> 76.9 us, level of 1,044 rows 12.6 -> 4.7 us
-// (75.0 us, 5.9 TB/s, and 3.2 us with dependent launches); 80 registers 84.7 us; digits streamed through shared memory by
-// cp.async, one or two packs ahead, 85-104 us (fewer warps fit); 48 registers 90 us.
+// (75.2 us, 6.0 TB/s, and 3.3 us with dependent launches); with 80 registers 79.0 us, with 48 137 us; digits
+// streamed through shared memory by cp.async, one or two packs ahead, 85-104 us (fewer warps fit).
 #include <cuda_runtime.h>
 
 #include <algorithm>

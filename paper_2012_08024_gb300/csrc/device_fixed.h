@@ -32,8 +32,8 @@ constexpr int kFxSms = 152;
 // Whether a level's block rows take a warp each: while they then fit on the GPU at once (32 warps per
 // SM; 16 above n_p = 10), or, up to four times as many, are long (three and more blocks per group of
 // n_p lanes): a row's blocks, not the number of rows, are what there is to spread.  FP64, 256^2, p = 3:
-// 4,135 rows of 7 blocks 8.2 -> 6.9 us; 24^3 tetrahedra, p = 2: 4,875 rows of 10 blocks 12.8 -> 9.4 us;
-// but 8,102 rows of 7 blocks at p = 2 (five groups share a row) 6.3 -> 8.5 us.
+// 4,135 rows of 7 blocks 7.4 -> 6.4 us; 24^3 tetrahedra, p = 2: 4,875 rows of 10 blocks 12.2 -> 8.8 us;
+// but 8,102 rows of 7 blocks at p = 2 (five groups share a row) 6.7 -> 8.9 us.
 inline bool warp_per_row(int np, int n, int64_t blocks) {
   const int groups = 32 / np, resident = kFxSms * (np > 10 ? 16 : 32);
   return groups > 1 && (n <= resident || (blocks >= (int64_t)n * 3 * groups && n <= 4 * resident));

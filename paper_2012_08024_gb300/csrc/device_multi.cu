@@ -197,7 +197,7 @@ __global__ void __launch_bounds__(128, mr_min_ctas<V, PF>()) mr_row_kernel(int n
 // 32 right-hand sides, one per lane.  A lane splits the n_p values of its column in a block's neighbour
 // (one exponent for them) and keeps the n_p sums, each with its scale, in registers; the digits of a
 // block are read from shared memory, each 16 bytes feeding eight integer multiply-adds.  5,000 rows,
-// n_p = 6, 40 columns: 82 us with FP64 multiply-adds (46 us at the FP64 rate), 50 us here.
+// n_p = 6, 40 columns: 82 us with FP64 multiply-adds (46 us at the FP64 rate), 61 us here.
 template <int NP>
 __global__ void __launch_bounds__(128, 4) mr_fx_kernel(int n, int R, const int* __restrict__ rowptr,
                                                        const int* __restrict__ col, const int2* __restrict__ A,
